@@ -89,6 +89,7 @@ struct GraphEntry {
     const void *cells = nullptr;
     unsigned gen_diffuse = 0, gen_small = 0;
     bool profiled = false;
+    bool predicted = false;         // first rounds from the shared expansion
     cudaGraphExec_t exec = nullptr;
     const void *result = nullptr;   // workspace buffer holding the final iterate
     long long kernels = 0;
@@ -101,6 +102,19 @@ struct RoundsEntry {
     int nf, precision, scheme, nsteps;
     double T, tol;
     int rounds;
+};
+
+// The increments of a run of implicit steps as Chebyshev expansions of the run's first
+// field (see pred_plan in stencil.cu): step i of group q adds sum_k coef[q][k * len[q] + i]
+// T_k u, k = 0 .. K[q].  Depends on the arguments below only.
+struct PredPlan {
+    int scheme = 0, nsteps = 0, m_it = 0;
+    double c = 0, lmax = 0;
+    bool use = false;
+    int maxK = 0, maxlen = 0, maxm = 0;
+    std::vector<int> start, len, K;
+    std::vector<int> m;   // iterations of the inner solve that follows, per step
+    std::vector<std::vector<float>> coef;
 };
 
 // ----------------------------------------------------------------------------- meshes
@@ -164,6 +178,7 @@ struct cg_mesh {
     std::vector<std::pair<std::vector<double>, int>> brounds;  // batched rounds per call signature
     std::vector<cgk::GraphEntry> graphs;      // captured diffusions
     std::vector<cgk::RoundsEntry> rounds;     // learned refinement schedules
+    std::vector<cgk::PredPlan> preds;         // shared expansions per (scheme, steps, c)
     std::vector<std::pair<double, double>> spectrum;   // unstructured: lower end of the
                                                        // Chebyshev interval per dte
     cudaStream_t capture_stream = nullptr;    // private stream used only for capture

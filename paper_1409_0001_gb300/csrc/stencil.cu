@@ -1639,7 +1639,10 @@ __global__ void k_from_df_pairs(size_t npairs, const float4 *__restrict__ x, dou
 // with x = u^{n+1} it has A x at hand, so the next step's first residual is
 // c L x = (x - A x) / theta (theta = 1 implicit Euler, 1/2 Crank-Nicolson), written to
 // r and y1 (and the next Crank-Nicolson right-hand side x + c/2 L x to bout).  Its
-// ||b||^2 goes to sc_next, the finished step's ||r||^2 to sc.
+// ||b||^2 goes to sc_next, the finished step's ||r||^2 to sc.  4: a refinement pass that
+// also reduces ||b||^2 (the first pass of a step whose correction comes from the shared
+// expansion); 5: a step's last refinement pass when nothing follows from its r (no r and
+// y1 written).
 template <class TS, int kMode>
 __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc, CoefDF cf,
                                                         int scheme, const DF *__restrict__ xin_all,
@@ -1687,10 +1690,14 @@ __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc
                 const DF lx = df_lap(s, v, (float)nn);
                 float rf = df_f(df_res(bk, v, cf.ce, lx));
                 rr = fmaf(rf, rf, rr);
-                if (kMode == 1) {
+                if (kMode == 1 || kMode == 4) {
                     st(r, k, rf);
                     st(y1, k, gamma * rf);
-                } else {
+                    if (kMode == 4) {
+                        const float bf = df_f(bk);
+                        bb = fmaf(bf, bf, bb);
+                    }
+                } else if (kMode == 2) {
                     DF cl = df_mul(cf.ce, lx);        // = theta c L v
                     DF bn = v;
                     if (scheme == 1) {
@@ -1706,14 +1713,15 @@ __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc
                 }
             });
     }
-    double vals[2] = {block_sum_f(rr), kMode != 1 ? block_sum_f(bb) : 0.0};
+    constexpr bool kBB = kMode == 0 || kMode == 2 || kMode == 4;   // also reduces ||b||^2
+    double vals[2] = {block_sum_f(rr), kBB ? block_sum_f(bb) : 0.0};
     double *partials = partials_all + (size_t)bp.f * 2 * bp.nb;
-    if (arrive(partials, kMode != 1 ? 2 : 1, vals, bp.bid, bp.nb, &sc[bp.f].ticket)) {
+    if (arrive(partials, kBB ? 2 : 1, vals, bp.bid, bp.nb, &sc[bp.f].ticket)) {
         double RR = finish_sum(partials, 0, bp.nb);
-        double BB = kMode != 1 ? finish_sum(partials, 1, bp.nb) : 0.0;
+        double BB = kBB ? finish_sum(partials, 1, bp.nb) : 0.0;
         if (is_thread0()) {
             sc[bp.f].rr = RR;
-            if (kMode == 0) sc[bp.f].bb = BB;
+            if (kMode == 0 || kMode == 4) sc[bp.f].bb = BB;
             if (kMode == 2) sc_next[bp.f].bb = BB;
             sc[bp.f].ticket = 0;
         }
@@ -1725,7 +1733,7 @@ __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc
 // the pair's arithmetic is the packed DF2 form (one f32x2 instruction for both cells,
 // bit-identical to the scalar form); a warp row covers 64 cells; x neighbours by shuffle
 // (and the neighbouring pairs at the tile edges), y neighbours from a shared plane,
-// z neighbours from a register queue.  Modes 0-2 as in k_refine_df; mode 3 is one
+// z neighbours from a register queue.  Modes 0-2, 4 and 5 as in k_refine_df; mode 3 is one
 // explicit Euler step in double-float arithmetic, xout = xin + c L xin
 // (cf.c = dtau / dx^2), with no reduction.  The double-float vectors it reads and writes
 // (x, b) are in the pair layout (k_to_df_pairs / k_from_df_pairs).
@@ -1945,11 +1953,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
                 XO[kz >> 1] = vc;
                 const float2 rf = df2_f(df2_res(df2_of(bc), V, ce2, L));
                 rr = fmaf(rf.x, rf.x, fmaf(rf.y, rf.y, rr));
-                if (kMode == 1) {
+                if (kMode == 1 || kMode == 4) {
                     PR::store(r, kz, rf.x, rf.y);
                     const float2 g1 = mul2(make_float2(gamma, gamma), rf);
                     PR::store(y1, kz, g1.x, g1.y);
-                } else {
+                    if (kMode == 4) {
+                        const float2 fb = df2_f(df2_of(bc));
+                        bb = fmaf(fb.x, fb.x, fmaf(fb.y, fb.y, bb));
+                    }
+                } else if (kMode == 2) {
                     DF2 C = df2_mul(ce2, L);   // theta c L v
                     DF2 Bn = V;
                     if (scheme == 1) {
@@ -2010,14 +2022,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     }
     cp_async_wait<0>();   // no copy outlives the block
     if (kMode == 3) return;   // the explicit step reduces nothing
-    double vals[2] = {block_sum_f(rr), kMode != 1 ? block_sum_f(bb) : 0.0};
+    constexpr bool kBB = kMode == 0 || kMode == 2 || kMode == 4;   // also reduces ||b||^2
+    double vals[2] = {block_sum_f(rr), kBB ? block_sum_f(bb) : 0.0};
     double *partials = partials_all + (size_t)f * 2 * nb;
-    if (arrive(partials, kMode != 1 ? 2 : 1, vals, bid, nb, &sc[f].ticket)) {
+    if (arrive(partials, kBB ? 2 : 1, vals, bid, nb, &sc[f].ticket)) {
         double RR = finish_sum(partials, 0, nb);
-        double BB = kMode != 1 ? finish_sum(partials, 1, nb) : 0.0;
+        double BB = kBB ? finish_sum(partials, 1, nb) : 0.0;
         if (is_thread0()) {
             sc[f].rr = RR;
-            if (kMode == 0) sc[f].bb = BB;
+            if (kMode == 0 || kMode == 4) sc[f].bb = BB;
             if (kMode == 2) sc_next[f].bb = BB;
             sc[f].ticket = 0;
         }
@@ -2213,7 +2226,7 @@ template <> struct Vec4cg<__nv_bfloat16> {
 // unrolled (the register queue rotates without copies).  PER: periodic axes (g.per):
 // halo rows, columns and planes wrap, every cell has both neighbours on a periodic
 // axis, and the tile's rows beyond ny hold the wrapped rows (y mod ny) as neighbours.
-template <class TS, template <class> class L, int ZFIX = 0, bool PER = false>
+template <class TS, template <class> class L, int ZFIX = 0, bool PER = false, bool PRED = false>
 __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z0, int z1,
                                              const Coef32 &cf, const float *sdg, float gamma,
                                              float omega, const TS *yv, const TS *ypv,
@@ -2259,7 +2272,7 @@ __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z
         }
         if (own) {
             if (ypv) ypc = LD::load(ypv, k0);
-            rc = LD::load(rv, k0);
+            if constexpr (!PRED) rc = LD::load(rv, k0);
         }
         if (rowlo) hlo = LD::load(yv, (size_t)((long long)k0 + dlo));
         if (rowhi) hhi = LD::load(yv, (size_t)((long long)k0 + dhi));
@@ -2279,7 +2292,7 @@ __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z
             if (hold && (z + 2 < g.nz || pz)) nup = LD::load(yv, PER ? (size_t)kxy + zp(z + 2) : kn + g.nxy);
             if (own) {
                 if (ypv) nyp = LD::load(ypv, kn);
-                nr = LD::load(rv, kn);
+                if constexpr (!PRED) nr = LD::load(rv, kn);
             }
             if (rowlo) nlo = LD::load(yv, (size_t)((long long)kn + dlo));
             if (rowhi) nhi = LD::load(yv, (size_t)((long long)kn + dhi));
@@ -2295,7 +2308,35 @@ __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z
         if (tx == 0) left = hl;
         if (x == xlast) right = hr;
         __syncthreads();
-        if (own) {
+        if constexpr (PRED) {   // omega the factor of the neighbour differences
+            if (own) {
+                // a wall's neighbour is the cell itself: its difference is zero
+                float4 up = pl[ty][tx], dn = pl[ty + 2][tx], zd = vdn, zu = vup;
+                if (!py && y == 0) up = vc;
+                if (!py && y + 1 == g.ny) dn = vc;
+                if (!pz && z == 0) zd = vc;
+                if (!pz && z + 1 == g.nz) zu = vc;
+                if (!px && x == 0) left = vc.x;
+                if (!px && x + 4 == g.nx) right = vc.w;
+                float4 d, o;
+                d.x = ((left - vc.x) + (vc.y - vc.x)) + ((up.x - vc.x) + (dn.x - vc.x)) + ((zd.x - vc.x) + (zu.x - vc.x));
+                d.y = ((vc.x - vc.y) + (vc.z - vc.y)) + ((up.y - vc.y) + (dn.y - vc.y)) + ((zd.y - vc.y) + (zu.y - vc.y));
+                d.z = ((vc.y - vc.z) + (vc.w - vc.z)) + ((up.z - vc.z) + (dn.z - vc.z)) + ((zd.z - vc.z) + (zu.z - vc.z));
+                d.w = ((vc.z - vc.w) + (right - vc.w)) + ((up.w - vc.w) + (dn.w - vc.w)) + ((zd.w - vc.w) + (zu.w - vc.w));
+                if (ypv) {
+                    o.x = fmaf(omega, d.x, (vc.x - ypc.x) + vc.x);
+                    o.y = fmaf(omega, d.y, (vc.y - ypc.y) + vc.y);
+                    o.z = fmaf(omega, d.z, (vc.z - ypc.z) + vc.z);
+                    o.w = fmaf(omega, d.w, (vc.w - ypc.w) + vc.w);
+                } else {
+                    o.x = fmaf(omega, d.x, vc.x);
+                    o.y = fmaf(omega, d.y, vc.y);
+                    o.z = fmaf(omega, d.z, vc.z);
+                    o.w = fmaf(omega, d.w, vc.w);
+                }
+                V::store(ynv, kz, o);
+            }
+        } else if (own) {
             const float4 up = pl[ty][tx], dn = pl[ty + 2][tx];
             float d0 = d0i, d12 = d12i, d3 = d3i;
             if (!pz && (z == 0 || z + 1 == g.nz)) {   // a z wall: fewer neighbours
@@ -2346,6 +2387,123 @@ __global__ void __launch_bounds__(kThreads, 4) k_cheb_v4(Geo g, int zlen, int nz
     __syncthreads();
     cheb_v4_tile<TS, Vec4, ZFIX, PER>(g, blockIdx.x, blockIdx.y, z0, z1, cf, sdg, gamma, omega, y_all + off,
                            yprev_all ? yprev_all + off : nullptr, r_all + off, ynext_all + off);
+}
+
+// ---------------------------------------------------------------- shared expansion
+// The first refinement round of every implicit step of a run of steps, from ONE Chebyshev
+// recurrence.  With A = I - ce L and u_i the steps' exact solutions, the increment of step
+// i is u_{i+1} - u_i = h_i(L) u_0 for the rational h_i of the scheme (pred_plan), so all
+// increments are combinations of the same vectors T_k(L) u_0, T_k the Chebyshev
+// polynomials on the spectrum of L.  The recurrence runs in FP32 sweeps (k_cheb* without
+// r: T_{k+1} = 2 (T_k - A' T_k) - T_{k-1}, A' = -2 L / mu_max), and k_pred_combine forms
+// every step's increment.  Its FP32 rounding leaves a residual of 1e-9 to 1e-6 of ||b||
+// (it scales with sum_k |coef|, at most 1.6 and mostly below 0.2), which is what an own
+// inner solve per step leaves after its first round; the step's refinement goes on from
+// there as before and its residual is checked as before.  The run's K sweeps take the place
+// of one inner solve per step: at 128^3, 10 steps, b = 8 dx 52 sweeps for 350, b = 2 dx 17
+// for 90.
+constexpr int kPredMaxK = 160;     // highest T_k
+constexpr int kPredMaxSteps = 20;  // steps per run (accumulators of k_pred_combine)
+
+// One step of the recurrence in difference form, T_{k+1} = (T_k - T_{k-1}) + T_k + w D T_k
+// with D the sum of the differences to the neighbours (T_1 = T_0 + w D T_0: tprev ==
+// nullptr).  At the lower end of the spectrum the recurrence amplifies a rounding error
+// by the number of steps left; in this form a constant field stays exactly constant and a
+// smooth one nearly so, while a neighbour sum less nn times the value rounds in proportion
+// to the value: the error of the final field (40 steps, b = 4 dx) is 4e-15 with the
+// differences and 1e-13 without.  Vectorised (nx % 4 == 0): k_cheb_v4's tile.
+template <int ZFIX, bool PER>
+__global__ void __launch_bounds__(kThreads, 4) k_pred_v4(Geo g, int zlen, int nzc, float w,
+                                                      const float *__restrict__ t_all,
+                                                      const float *__restrict__ tprev_all,
+                                                      float *__restrict__ tnext_all) {
+    chain_wait();
+    chain_release();
+    const int f = nzc == (int)gridDim.z ? 0 : (int)blockIdx.z / nzc;
+    const int z0 = ((int)blockIdx.z - f * nzc) * zlen;
+    const int z1 = min(g.nz, z0 + zlen);
+    const size_t off = (size_t)f * g.n;
+    const float dg[8] = {};   // unused by the difference form
+    cheb_v4_tile<float, Vec4, ZFIX, PER, true>(g, blockIdx.x, blockIdx.y, z0, z1, Coef32{}, dg, 0.f, w, t_all + off,
+                                               tprev_all ? tprev_all + off : nullptr, nullptr, tnext_all + off);
+}
+
+// The same step on any mesh: the neighbour sum is carried as an FP32 pair (a TwoSum
+// cascade), so that less nn times the value it is the sum of the differences to FP32
+// accuracy.  Four planes per block (walls) or the z march (a periodic axis).
+template <bool PER>
+__global__ void __launch_bounds__(kThreads) k_pred_any(Geo g, int zlen, int nzc, float w,
+                                                       const float *__restrict__ t_all,
+                                                       const float *__restrict__ tprev_all,
+                                                       float *__restrict__ tnext_all) {
+    chain_wait();
+    chain_release();
+    const int f = blockIdx.z / nzc;
+    const int z0 = (blockIdx.z - f * nzc) * zlen;
+    const size_t off = (size_t)f * g.n;
+    const float *t = t_all + off, *tp = tprev_all ? tprev_all + off : nullptr;
+    float *tn = tnext_all + off;
+    auto load = [&](int k) { return DF{t[k], 0.f}; };
+    auto prev = [&](int k) { return tp ? tp[k] : 0.f; };
+    auto use = [&](int k, DF v, DF s, int nn, float p) {
+        const float d = df_f(df_lap(s, v, (float)nn));
+        tn[k] = fmaf(w, d, tp ? (v.hi - p) + v.hi : v.hi);
+    };
+    if constexpr (PER) sweep25p<DF>(g, z0, min(g.nz, z0 + zlen), load, prev, use);
+    else sweepzb<4, DF>(g, blockIdx.x, blockIdx.y, z0, load, prev, use);
+}
+
+// T_0: the hi parts of a double-float field (pair layout or one pair per cell).
+__global__ void __launch_bounds__(kThreads) k_pred_start(size_t n, bool pairs, const DF *__restrict__ u,
+                                                         float *__restrict__ t0) {
+    chain_wait();
+    chain_release();
+    const size_t step = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (pairs) {
+        for (size_t i = i0; i < n / 2; i += step) {
+            const float4 v = reinterpret_cast<const float4 *>(u)[i];
+            reinterpret_cast<float2 *>(t0)[i] = make_float2(v.x, v.y);
+        }
+    } else {
+        for (size_t i = i0; i < n; i += step) t0[i] = u[i].hi;
+    }
+}
+
+template <int NS> struct PredCoef {
+    float a[(kPredMaxK + 1) * NS];
+};
+
+// d_i = sum_k a[k][i] T_k for NS steps: each T_k is read once for all of them.  Bound by
+// HBM (K + 1 vectors read, NS written) and, for many steps, by the multiply-adds; four
+// cells per thread, two cells to an instruction, four vectors' loads in flight.  The
+// vectors are `stride` floats apart and padded to whole float4s.
+template <int NS>
+__global__ void __launch_bounds__(kThreads) k_pred_combine(size_t n4, size_t stride, int K,
+                                                           const __grid_constant__ PredCoef<NS> cf,
+                                                           const float *__restrict__ t,
+                                                           float *__restrict__ d) {
+    chain_wait();
+    chain_release();
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n4; i += (size_t)gridDim.x * kThreads) {
+        float2 lo[NS], hi[NS];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) lo[q] = hi[q] = make_float2(0.f, 0.f);
+        const float *tp = t + 4 * i;
+#pragma unroll 4
+        for (int k = 0; k <= K; ++k, tp += stride) {
+            const float4 v = *reinterpret_cast<const float4 *>(tp);
+            const float2 a = make_float2(v.x, v.y), b = make_float2(v.z, v.w);
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                const float w = cf.a[k * NS + q];
+                lo[q] = fma2(a, make_float2(w, w), lo[q]);
+                hi[q] = fma2(b, make_float2(w, w), hi[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NS; ++q)
+            *reinterpret_cast<float4 *>(d + q * stride + 4 * i) = make_float4(lo[q].x, lo[q].y, hi[q].x, hi[q].y);
+    }
 }
 
 // ---------------------------------------------------------------- two iterations per sweep
@@ -4772,6 +4930,216 @@ static cg_status diffuse_explicit(cg_mesh *m, int nf, double *cells, const cg_pa
     return CG_OK;
 }
 
+// The expansions of a call's increments.  Step i of a run (i = 0, 1, ..) starting at u_0:
+// implicit Euler u_i = (1 + c mu)^-i u_0, so h_i = -c mu (1 + c mu)^-(i+1); Crank-Nicolson
+// u_i = g^i u_0 with g = (1 - c mu / 2) / (1 + c mu / 2), so h_i = (g - 1) g^i; mu >= 0 the
+// eigenvalues of -L, up to mu_max.  Coefficients by Gauss-Chebyshev quadrature on enough
+// nodes that they have decayed; K where the rest adds at most a third of the FP32 rounding
+// of the sum to the residual: lmax tail_i <= 0.3 * 9e-8 S_i A_rms with S_i = sum |a|,
+// A_rms = 1 + 6.5 ce (the diagonal dominates on rounding noise).
+//
+// Whether it pays: in units of one sweep (16 B per cell) a call's own inner solves take
+// 2 (m - 1) per step and the predicted ones about half of that plus, per run, K recurrence
+// sweeps of 12 B and the combination (K + 1 vectors read, `len` written).  Measured at
+// 128^3, b = 2 dx: see launch site.
+static void pred_build(PredPlan &pl) {
+    const double ce = pl.scheme == CG_SCHEME_CRANK_NICOLSON ? 0.5 * pl.c : pl.c;
+    const double mu_max = (pl.lmax - 1.0) / ce;
+    pl.use = false;
+    if (!(mu_max > 0.0) || pl.nsteps < 2) return;
+    const int groups = (pl.nsteps + kPredMaxSteps - 1) / kPredMaxSteps;
+    const double arms = 1.0 + 6.5 * ce;
+    double cost = 0.0;
+    std::vector<std::vector<double>> sums;   // S_i per run
+    for (int q = 0, s0 = 0; q < groups; ++q) {
+        const int len = (pl.nsteps - s0 + groups - q - 1) / (groups - q);
+        if (q > 0 && len == pl.len[q - 1]) {   // runs of one length share their coefficients
+            pl.coef.push_back(pl.coef[q - 1]);
+            pl.K.push_back(pl.K[q - 1]);
+        } else {
+            std::vector<double> a;   // [k][i]
+            int K = -1, N = 32;
+            for (; N <= 4 * kPredMaxK && K < 0; N *= 2) {
+                const int kc = std::min(N / 2, kPredMaxK + 40);
+                std::vector<double> cs(4 * N);
+                for (int j = 0; j < 4 * N; ++j) cs[j] = std::cos(M_PI * j / (2.0 * N));
+                a.assign((size_t)(kc + 1) * len, 0.0);
+                std::vector<double> h(len);
+                for (int j = 0; j < N; ++j) {   // x_j = cos(pi (j + 1/2) / N), mu = mu_max (1 - x) / 2
+                    const double cm = pl.c * 0.5 * mu_max * (1.0 - cs[2 * j + 1]);
+                    double g, w;
+                    if (pl.scheme == CG_SCHEME_CRANK_NICOLSON) {
+                        g = (1.0 - 0.5 * cm) / (1.0 + 0.5 * cm);
+                        w = -cm / (1.0 + 0.5 * cm);   // g - 1
+                    } else {
+                        g = 1.0 / (1.0 + cm);
+                        w = -cm * g;
+                    }
+                    for (int i = 0; i < len; ++i, w *= g) h[i] = w * 2.0 / N;
+                    for (int k = 0; k <= kc; ++k) {
+                        const double f = (k ? 1.0 : 0.5) * cs[(int)((long long)(2 * j + 1) * k % (4 * N))];
+                        for (int i = 0; i < len; ++i) a[(size_t)k * len + i] += f * h[i];
+                    }
+                }
+                std::vector<double> S(len, 0.0), tail(len, 0.0);
+                for (int k = 0; k <= kc; ++k)
+                    for (int i = 0; i < len; ++i) S[i] += std::fabs(a[(size_t)k * len + i]);
+                int k = kc;
+                for (; k > 0; --k) {   // drop T_k while every step's rest stays below its bound
+                    bool drop = true;
+                    for (int i = 0; i < len; ++i)
+                        drop = drop && pl.lmax * (tail[i] + std::fabs(a[(size_t)k * len + i])) <= 2.7e-8 * S[i] * arms;
+                    if (!drop) break;
+                    for (int i = 0; i < len; ++i) tail[i] += std::fabs(a[(size_t)k * len + i]);
+                }
+                if (k <= kc - 4 && k <= kPredMaxK) K = std::max(k, 1);
+            }
+            if (K < 0) return;
+            std::vector<float> f((size_t)(K + 1) * len);
+            for (size_t j = 0; j < f.size(); ++j) f[j] = (float)a[j];
+            for (int i = 0; i < len; ++i) {   // h_i(0) = 0 also for the rounded coefficients
+                double sum = 0.0;
+                for (int k = 1; k <= K; ++k) sum += f[(size_t)k * len + i];
+                f[i] = (float)-sum;
+            }
+            pl.coef.push_back(f);
+            pl.K.push_back(K);
+            std::vector<double> S(len, 0.0);
+            for (int k = 0; k <= K; ++k)
+                for (int i = 0; i < len; ++i) S[i] += std::fabs(a[(size_t)k * len + i]);
+            sums.push_back(S);
+        }
+        if (sums.size() < pl.coef.size()) sums.push_back(sums.back());
+        pl.start.push_back(s0);
+        pl.len.push_back(len);
+        pl.maxK = std::max(pl.maxK, pl.K.back());
+        pl.maxlen = std::max(pl.maxlen, len);
+        cost += 0.75 * pl.K.back() + 0.25 * (pl.K.back() + 1 + len);
+        s0 += len;
+    }
+    // The iterations of the round that follows: from the residual that rounding leaves in
+    // step i, 9e-8 S_i A_rms ||u_0||, to half of what a double-float residual resolves,
+    // with ||u_i|| / ||u_0|| of a field of white noise (a deposited field of few particles;
+    // smoother fields decay less).  A mode's decay per step depends on mu alone: sampled at
+    // the midpoints of 8^3 frequencies.
+    double mus[120], wts[120];
+    int ns = 0;
+    for (int a = 0; a < 8; ++a)
+        for (int b = a; b < 8; ++b)
+            for (int d = b; d < 8; ++d) {
+                auto l = [](int q) { const double v = std::sin(M_PI * (q + 0.5) / 16.0); return 4.0 * v * v; };
+                mus[ns] = std::min(l(a) + l(b) + l(d), mu_max);
+                wts[ns++] = a == d ? 1.0 : (a == b || b == d) ? 3.0 : 6.0;
+            }
+    std::vector<double> amp(ns, 1.0), norm(pl.nsteps);
+    for (int s = 0; s < pl.nsteps; ++s) {
+        double e = 0.0;
+        for (int q = 0; q < ns; ++q) {
+            e += wts[q] * amp[q] * amp[q];
+            const double cm = pl.c * mus[q];
+            amp[q] *= pl.scheme == CG_SCHEME_CRANK_NICOLSON ? (1.0 - 0.5 * cm) / (1.0 + 0.5 * cm) : 1.0 / (1.0 + cm);
+        }
+        norm[s] = std::sqrt(e / 512.0);
+    }
+    const double sg = (std::sqrt(pl.lmax) - 1.0) / (std::sqrt(pl.lmax) + 1.0);
+    double own = 0.0;
+    for (size_t q = 0; q < pl.start.size(); ++q)
+        for (int i = 0; i < pl.len[q]; ++i) {
+            const int s = pl.start[q] + i;
+            const double est = 9e-8 * sums[q][i] * arms * norm[pl.start[q]] / norm[s];
+            const double target = 1.8e-15 * arms;
+            int mi = (int)std::ceil(std::log(2.0 * std::max(est / target, 1.0)) / -std::log(sg));
+            mi = std::max(2, std::min(mi, 400));
+            pl.m.push_back(mi);
+            pl.maxm = std::max(pl.maxm, mi);
+            cost += mi - 1;
+            own += 2.0 * (pl.m_it - 1);
+        }
+    pl.use = cost <= 0.9 * own;
+}
+
+static const PredPlan &pred_plan(cg_mesh *m, int scheme, int nsteps, int m_it, double c, double lmax) {
+    for (const PredPlan &q : m->preds)
+        if (q.scheme == scheme && q.nsteps == nsteps && q.m_it == m_it && q.c == c && q.lmax == lmax) return q;
+    if (m->preds.size() >= 16) m->preds.erase(m->preds.begin());
+    PredPlan pl;
+    pl.scheme = scheme;
+    pl.nsteps = nsteps;
+    pl.m_it = m_it;
+    pl.c = c;
+    pl.lmax = lmax;
+    pred_build(pl);
+    m->preds.push_back(std::move(pl));
+    return m->preds.back();
+}
+
+template <int NS>
+static void launch_pred_combine(size_t n, size_t stride, const PredPlan &pl, int q, const float *t, float *d,
+                                cudaStream_t st) {
+    PredCoef<NS> cf;
+    const int K = pl.K[q], len = pl.len[q];
+    for (int k = 0; k <= K; ++k)
+        for (int i = 0; i < NS; ++i) cf.a[k * NS + i] = i < len ? pl.coef[q][(size_t)k * len + i] : 0.f;
+    const size_t n4 = (n + 3) / 4;
+    const unsigned grid = (unsigned)std::min<size_t>((n4 + kThreads - 1) / kThreads, 1u << 30);
+    launch_chain(k_pred_combine<NS>, dim3(grid), dim3(kThreads), st, n4, stride, K, cf, t, d);
+}
+
+// Planes per block of the vectorised sweep, unrolled (the register queue rotates by
+// renaming): 128^3 with 1 / 2 / 3 / 4 / 8 planes 6.0 / 5.1 / 6.4 / 6.7 / 6.9 us, 512 x 256 x 256
+// 96.9 / 73.4 / 79.9 / 78.5 / 76.5 us (4.1 -> 5.5 TB/s), with only 1 and 2 unrolled.
+constexpr int kPredPlanes = 2;
+static void launch_pred_sweep(const Geo &g, int nf, float w, const float *t, const float *tp, float *tn,
+                              cudaStream_t st) {
+    const dim3 blk(TX, TY);
+    const int gy = (g.ny + TY - 1) / TY;
+    if (g.nx % 4 == 0) {
+        const int nzc = (g.nz + kPredPlanes - 1) / kPredPlanes;
+        const dim3 grid((g.nx + 4 * TX - 1) / (4 * TX), gy, nzc * nf);
+        if (g.per) launch_chain(k_pred_v4<kPredPlanes, true>, grid, blk, st, g, kPredPlanes, nzc, w, t, tp, tn);
+        else launch_chain(k_pred_v4<kPredPlanes, false>, grid, blk, st, g, kPredPlanes, nzc, w, t, tp, tn);
+    } else {
+        const int zl = g.per ? make_sweep(g, nf).zlen : 4, nzc = (g.nz + zl - 1) / zl;
+        const dim3 grid((g.nx + TX - 1) / TX, gy, nzc * nf);
+        if (g.per) launch_chain(k_pred_any<true>, grid, blk, st, g, zl, nzc, w, t, tp, tn);
+        else launch_chain(k_pred_any<false>, grid, blk, st, g, zl, nzc, w, t, tp, tn);
+    }
+}
+
+// The increments of run q of the plan, from u (double-float): K sweeps, then the
+// combination.  T: (K + 1) vectors of `stride` floats, D: len vectors.
+static void launch_pred(const PredPlan &pl, int q, const Geo &g, int nf, const DF *u, float *T, float *D,
+                        size_t stride, cudaStream_t st) {
+    const size_t n = (size_t)g.n * nf;
+    const double ce = pl.scheme == CG_SCHEME_CRANK_NICOLSON ? 0.5 * pl.c : pl.c;
+    const float e = (float)(2.0 * ce / (pl.lmax - 1.0));   // T_1 = (1 + 2 L / mu_max) T_0
+    CGK_LAUNCH("pred_start", (double)n * 12, st,
+               launch_chain(k_pred_start, dim3(stencil_grid((int)std::min<size_t>(n, 1u << 30))), dim3(kThreads), st, n,
+                            df_pairs(g), u, T));
+    {
+        CGK_TIMED(loop_, "pred_sweep", (double)n * (8.0 + 12.0 * (pl.K[q] - 1)), st, pl.K[q]);
+        for (int k = 0; k < pl.K[q]; ++k)
+            CGK_LAUNCH_UNTIMED(st, launch_pred_sweep(g, nf, k ? 2.0f * e : e, T + k * stride,
+                                                     k ? T + (k - 1) * stride : nullptr, T + (k + 1) * stride, st));
+    }
+    const int len = pl.len[q];
+    CGK_LAUNCH("pred_combine", (double)n * 4 * (pl.K[q] + 1 + len), st, {
+        if (len <= 2) launch_pred_combine<2>(n, stride, pl, q, T, D, st);
+        else if (len <= 5) launch_pred_combine<5>(n, stride, pl, q, T, D, st);
+        else if (len <= 8) launch_pred_combine<8>(n, stride, pl, q, T, D, st);
+        else if (len <= 10) launch_pred_combine<10>(n, stride, pl, q, T, D, st);
+        else if (len <= 13) launch_pred_combine<13>(n, stride, pl, q, T, D, st);
+        else if (len <= 16) launch_pred_combine<16>(n, stride, pl, q, T, D, st);
+        else launch_pred_combine<kPredMaxSteps>(n, stride, pl, q, T, D, st);
+    });
+}
+// (vectors of D a combination of NS >= len steps writes)
+static int pred_vectors(int len) {
+    for (int ns : {2, 5, 8, 10, 13, 16})
+        if (len <= ns) return ns;
+    return kPredMaxSteps;
+}
+
 // Mixed-precision implicit steps: TS is the storage type of the inner solve (float or
 // bf16), XT the type of the iterate and of the refinement residual (IEEE double, or
 // the double-float pair DF).
@@ -4821,9 +5189,20 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     // the resident inner solve (whole mesh in shared memory) where it fits; its flags and
     // faces follow the vectors
     const ResidentPlan rp = (persistent || m->per) ? ResidentPlan{} : plan_resident<TS>(g, nf, m_it);
-    CGK_TRY(m->ws_diffuse.ensure(4 * v64 + 5 * vts + (rp.ok ? rp.ws_bytes : 0)));
+    // the shared expansion of the steps' first rounds (its vectors follow the resident
+    // solve's), where it pays, nothing caps the iterations, and its vectors may be held
+    const PredPlan *pred = nullptr;
+    const size_t base_b = 4 * v64 + 5 * vts + align_up(rp.ok ? rp.ws_bytes : 0);
+    if (kDF && sizeof(TS) == 4 && !persistent) {
+        const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, m_it, c, lmax);
+        if (q.use && p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
+            m->ws_diffuse.ensure(base_b + (size_t)(q.maxK + 1 + pred_vectors(q.maxlen)) * vts) == CG_OK)
+            pred = &q;
+    }
+    if (!pred) CGK_TRY(m->ws_diffuse.ensure(base_b));
     char *wb = m->ws_diffuse.as<char>();
     char *rws = wb + 4 * v64 + 5 * vts;
+    float *PT = (float *)(wb + base_b), *PD = pred ? PT + (size_t)(pred->maxK + 1) * (vts / 4) : nullptr;
     XT *X1 = (XT *)wb, *X2 = (XT *)(wb + v64), *B = (XT *)(wb + 2 * v64), *X0 = (XT *)(wb + 3 * v64);
     TS *R = (TS *)(wb + 4 * v64), *Ya = (TS *)(wb + 4 * v64 + vts), *Yb = (TS *)(wb + 4 * v64 + 2 * vts);
     // two more iterate buffers for two-iterations-per-launch sweeps
@@ -4927,6 +5306,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 if (it->nf == nf && it->precision == p->precision && it->scheme == p->scheme &&
                     it->nsteps == p->nsteps && it->rounds == R && it->T == T && it->tol == p->tol &&
                     it->cells == cells && it->profiled == prof && it->code == shape_used &&
+                    it->predicted == (pred != nullptr) &&
                     it->wait_budget == rbudget)
                     ge = &*it;
                 ++it;
@@ -4948,6 +5328,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 e.gen_diffuse = m->ws_diffuse.gen;
                 e.gen_small = m->ws_small.gen;
                 e.profiled = prof;
+                e.predicted = pred != nullptr;
                 e.code = shape_used;
                 e.wait_budget = rbudget;
                 prof_capture_begin(&e.records, &e.kernels);
@@ -4960,13 +5341,14 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                launch_to_df(g, (size_t)n * nf, cells, (DF *)X0, cs));
                     XT *u = X0, *f1 = X1, *f2 = X2;
                     TS *y1_start = Ya;
+                    int run = -1;   // the current run of the shared expansion
                     for (int s2 = 0; s2 < p->nsteps; ++s2) {
                         RefScal *slot = hist + (size_t)s2 * nf;
                         const XT *bp_ = cn ? B : u;
                         TS *y1 = y1_start;
                         // the first step starts with its own pass; later steps were started
                         // by the previous step's last pass
-                        if (s2 == 0)
+                        if (s2 == 0 && (!pred || cn))
                             CGK_LAUNCH("refine_df_first", (double)n * nf * (8 + (cn ? 8 : 0) + 2 * sizeof(TS)), cs,
                                        launch_refine_df<TS, 0>(g, sw, nf, cfdf, p->scheme,
                                                                (const DF *)u, (const TS *)nullptr,
@@ -4974,22 +5356,40 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                                (DF *)B, R_, y1, (float)gamma,
                                                                partials, slot, slot, cs));
                         XT *xc = u;
-                        for (int r = 0; r < R; ++r) {
+                        if constexpr (sizeof(TS) == 4)
+                            if (pred) {   // the step's first round
+                                if (run + 1 < (int)pred->start.size() && pred->start[run + 1] == s2)
+                                    launch_pred(*pred, ++run, g, nf, (const DF *)u, PT, PD, vts / 4, cs);
+                                const float *d0 = PD + (size_t)(s2 - pred->start[run]) * (vts / 4);
+                                if (cn)
+                                    CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
+                                               launch_refine_df<TS, 1>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
+                                                                       (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
+                                                                       (float)gamma, partials, slot, slot, cs));
+                                else
+                                    CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
+                                               launch_refine_df<TS, 4>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
+                                                                       (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
+                                                                       (float)gamma, partials, slot, slot, cs));
+                                xc = f1;
+                            }
+                        const int mi = pred ? pred->m[s2] : m_it;   // inner iterations of a round
+                        for (int r = pred ? 1 : 0; r < R; ++r) {
                             TS *yc = y1, *yp = nullptr, *yo = (y1 == Ya) ? Yb : Ya;
                             double om = 1.0;
-                            if (m_it > 1 && resident) {
-                                TS *yf = cheb_final_buffer(yc, yo, m_it);
+                            if (mi > 1 && resident) {
+                                TS *yf = cheb_final_buffer(yc, yo, mi);
                                 CGK_LAUNCH(sizeof(TS) == 2 ? "cheb_resident_bf16" : "cheb_resident_fp32",
-                                           (double)n * nf * sizeof(TS) * (3.0 + 4.0 * (m_it - 2)), cs,
+                                           (double)n * nf * sizeof(TS) * (3.0 + 4.0 * (mi - 2)), cs,
                                            {
                                                cudaError_t le = launch_resident<TS>(
-                                                   g, rp, cf32, (float)gamma, sigma_d, m_it, yc, R_,
+                                                   g, rp, cf32, (float)gamma, sigma_d, mi, yc, R_,
                                                    yf, rws, rbudget, cs);
                                                if (cap_err == cudaSuccess) cap_err = le;
                                            });
                                 yc = yf;
-                            } else if (m_it > 1 && cheb_code >= kPairCode && cheb_code < kResidentCode) {
-                                const int np = (m_it - 1) / 2, ns = (m_it - 1) % 2;
+                            } else if (mi > 1 && cheb_code >= kPairCode && cheb_code < kResidentCode) {
+                                const int np = (mi - 1) / 2, ns = (mi - 1) % 2;
                                 CGK_TIMED(loop_, sizeof(TS) == 2 ? "cheb2_bf16" : "cheb2_fp32",
                                           (double)n * nf * sizeof(TS) *
                                               (np > 0 ? 4.0 + 5.0 * (np - 1) : 0.0) +
@@ -4997,12 +5397,12 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                           cs, np + ns);
                                 TS *const pool[4] = {yc, yo, Yc, Yd};   // y1 is Ya or Yb
                                 yc = cheb_pairs<TS>(cheb_code - kPairCode, g, nf, cf32, (float)gamma,
-                                                    sigma_d, m_it, pool, R_, cs);
-                            } else if (m_it > 1) {
+                                                    sigma_d, mi, pool, R_, cs);
+                            } else if (mi > 1) {
                                 CGK_TIMED(loop_, sizeof(TS) == 2 ? "cheb_bf16" : "cheb_fp32",
-                                          (double)n * nf * sizeof(TS) * (3.0 + 4.0 * (m_it - 2)),
-                                          cs, m_it - 1);
-                                for (int k = 1; k < m_it; ++k) {
+                                          (double)n * nf * sizeof(TS) * (3.0 + 4.0 * (mi - 2)),
+                                          cs, mi - 1);
+                                for (int k = 1; k < mi; ++k) {
                                     if (sigma_d > 0.0)
                                         om = (k == 1) ? 1.0 / (1.0 - 1.0 / (2.0 * sigma_d * sigma_d))
                                                       : 1.0 / (1.0 - om / (4.0 * sigma_d * sigma_d));
@@ -5017,10 +5417,19 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                             XT *xn = (xc == f1) ? f2 : f1;
                             // the next step's first Chebyshev iterate goes to Ya: it must not
                             // be the buffer holding this round's correction
-                            const bool emit = (r == R - 1) && (s2 + 1 < p->nsteps);
+                            const bool last = r == R - 1;
+                            const bool emit = last && (s2 + 1 < p->nsteps) && (!pred || cn);
                             y1 = (yc == Ya) ? Yb : Ya;
                             if (emit) y1_start = y1;    // where the next step's y1 is
-                            if (emit)
+                            if (last && !emit)   // nothing follows from this pass's r
+                                CGK_LAUNCH("refine_df_end", (double)n * nf * (24 + sizeof(TS)), cs,
+                                           launch_refine_df<TS, 5>(g, sw, nf, cfdf, p->scheme,
+                                                                   (const DF *)xc, (const TS *)yc,
+                                                                   (const DF *)bp_, (DF *)xn,
+                                                                   (DF *)nullptr, R_, y1,
+                                                                   (float)gamma, partials, slot,
+                                                                   slot, cs));
+                            else if (emit)
                                 CGK_LAUNCH("refine_df_last", (double)n * nf * (24 + 3 * sizeof(TS) + (cn ? 8 : 0)), cs,
                                            launch_refine_df<TS, 2>(g, sw, nf, cfdf, p->scheme,
                                                                    (const DF *)xc, (const TS *)yc,
@@ -5087,11 +5496,16 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 CGK_CUDA(cudaStreamSynchronize(st));
                 if (rep) {
                     long long apps = 1 + (long long)p->nsteps * R * m_it;
+                    if (pred) {   // expansions, then per step one pass and R - 1 rounds
+                        apps = (cn ? 1 : 0) + p->nsteps;
+                        for (int K : pred->K) apps += K;
+                        for (int mi : pred->m) apps += (long long)(R - 1) * mi;
+                    }
                     rep->iters = apps * nf;
                     rep->refine_rounds = (long long)p->nsteps * R;
                     rep->cell_updates = apps * nf * (long long)n;
                     rep->final_rel_residual = worst_g;
-                    rep->inner_iters_per_round = m_it;
+                    rep->inner_iters_per_round = pred ? pred->maxm : m_it;
                     rep->sweep_shape_used = shape_used;
                 }
                 return CG_OK;
