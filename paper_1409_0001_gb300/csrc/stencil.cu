@@ -1739,7 +1739,7 @@ __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc
 // (x, b) are in the pair layout (k_to_df_pairs / k_from_df_pairs).
 template <class TS> struct Pair;
 template <> struct Pair<float> {
-    static __device__ __forceinline__ float2 load(const float *p, size_t i) {
+    static __device__ __forceinline__ float2 load(const float *p, int i) {
         return *reinterpret_cast<const float2 *>(p + i);
     }
     static __device__ __forceinline__ void store(float *p, size_t i, float a, float b) {
@@ -1747,7 +1747,7 @@ template <> struct Pair<float> {
     }
 };
 template <> struct Pair<__nv_bfloat16> {
-    static __device__ __forceinline__ float2 load(const __nv_bfloat16 *p, size_t i) {
+    static __device__ __forceinline__ float2 load(const __nv_bfloat16 *p, int i) {
         return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p + i));
     }
     static __device__ __forceinline__ void store(__nv_bfloat16 *p, size_t i, float a, float b) {
@@ -2174,7 +2174,7 @@ __global__ void __launch_bounds__(kThreads) k_cheb_zb(Geo g, int nzb, Coef32 cf,
 // and is not counted (zero flux).
 template <class TS> struct Vec4;
 template <> struct Vec4<float> {
-    static __device__ __forceinline__ float4 load(const float *p, size_t i) {
+    static __device__ __forceinline__ float4 load(const float *p, int i) {
         return *reinterpret_cast<const float4 *>(p + i);
     }
     static __device__ __forceinline__ void store(float *p, size_t i, float4 v) {
@@ -2182,7 +2182,7 @@ template <> struct Vec4<float> {
     }
 };
 template <> struct Vec4<__nv_bfloat16> {
-    static __device__ __forceinline__ float4 load(const __nv_bfloat16 *p, size_t i) {
+    static __device__ __forceinline__ float4 load(const __nv_bfloat16 *p, int i) {
         uint2 u = *reinterpret_cast<const uint2 *>(p + i);
         __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162 *>(&u.x);
         __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162 *>(&u.y);
@@ -2205,12 +2205,12 @@ __device__ __forceinline__ float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0
 // same (persistent) launch.
 template <class TS> struct Vec4cg;
 template <> struct Vec4cg<float> {
-    static __device__ __forceinline__ float4 load(const float *p, size_t i) {
+    static __device__ __forceinline__ float4 load(const float *p, int i) {
         return __ldcg(reinterpret_cast<const float4 *>(p + i));
     }
 };
 template <> struct Vec4cg<__nv_bfloat16> {
-    static __device__ __forceinline__ float4 load(const __nv_bfloat16 *p, size_t i) {
+    static __device__ __forceinline__ float4 load(const __nv_bfloat16 *p, int i) {
         uint2 u = __ldcg(reinterpret_cast<const uint2 *>(p + i));
         __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162 *>(&u.x);
         __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162 *>(&u.y);
@@ -2221,7 +2221,7 @@ template <> struct Vec4cg<__nv_bfloat16> {
 
 // One tile (128 x-cells x TY rows x planes [z0, z1)) of the vectorised Chebyshev
 // iteration; L is the load policy (Vec4 or Vec4cg), sdg the diagonal table in shared
-// memory.  Every thread of the block must call it (barriers and shuffles inside).
+// memory.  Offsets within a field are 32-bit (a field has fewer than 2^31 cells).  Every thread of the block must call it (barriers and shuffles inside).
 // ZFIX > 0: the caller guarantees at most ZFIX planes per block, so the march is
 // unrolled (the register queue rotates without copies).  PER: periodic axes (g.per):
 // halo rows, columns and planes wrap, every cell has both neighbours on a periodic
@@ -2259,45 +2259,45 @@ __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z
     const int dxl = (PER && x == 0) ? g.nx - 1 : -1;
     const int dxr = (PER && x + 4 >= g.nx) ? 4 - g.nx : 4;
     // plane index of plane q of the z march (wrapped on a periodic z axis)
-    auto zp = [&](int q) -> size_t { return (size_t)(pz ? (q + g.nz) % g.nz : q) * g.nxy; };
+    auto zp = [&](int q) -> int { return (pz ? (q + g.nz) % g.nz : q) * g.nxy; };
     float4 vdn = f4zero(), vc = f4zero(), vup = f4zero(), ypc = f4zero(), rc = f4zero();
     float4 hlo = f4zero(), hhi = f4zero();
     float hl = 0.f, hr = 0.f;
     if (z0 < z1) {
-        const size_t k0 = (size_t)kxy + zp(z0);
+        const int k0 = kxy + zp(z0);
         if (hold) {
-            if (z0 > 0 || pz) vdn = LD::load(yv, (size_t)kxy + zp(z0 - 1));
+            if (z0 > 0 || pz) vdn = LD::load(yv, kxy + zp(z0 - 1));
             vc = LD::load(yv, k0);
-            if (z0 + 1 < g.nz || pz) vup = LD::load(yv, (size_t)kxy + zp(z0 + 1));
+            if (z0 + 1 < g.nz || pz) vup = LD::load(yv, kxy + zp(z0 + 1));
         }
         if (own) {
             if (ypv) ypc = LD::load(ypv, k0);
             if constexpr (!PRED) rc = LD::load(rv, k0);
         }
-        if (rowlo) hlo = LD::load(yv, (size_t)((long long)k0 + dlo));
-        if (rowhi) hhi = LD::load(yv, (size_t)((long long)k0 + dhi));
-        if (xl) hl = ldcg(yv, (int)((long long)k0 + dxl));
-        if (xr) hr = ldcg(yv, (int)((long long)k0 + dxr));
+        if (rowlo) hlo = LD::load(yv, k0 + dlo);
+        if (rowhi) hhi = LD::load(yv, k0 + dhi);
+        if (xl) hl = ldcg(yv, k0 + dxl);
+        if (xr) hr = ldcg(yv, k0 + dxr);
     }
 #pragma unroll
     for (int zi = 0; zi < (ZFIX > 0 ? ZFIX : z1 - z0); ++zi) {
         const int z = z0 + zi;
         if (ZFIX > 0 && z >= z1) break;
-        const size_t kz = (size_t)kxy + (PER ? zp(z) : (size_t)z * g.nxy);
+        const int kz = kxy + (PER ? zp(z) : z * g.nxy);
         // loads for the next plane
         float4 nup = f4zero(), nyp = f4zero(), nr = f4zero(), nlo = f4zero(), nhi = f4zero();
         float nl = 0.f, nrr = 0.f;
         if (z + 1 < z1) {
-            const size_t kn = PER ? (size_t)kxy + zp(z + 1) : kz + g.nxy;
-            if (hold && (z + 2 < g.nz || pz)) nup = LD::load(yv, PER ? (size_t)kxy + zp(z + 2) : kn + g.nxy);
+            const int kn = PER ? kxy + zp(z + 1) : kz + g.nxy;
+            if (hold && (z + 2 < g.nz || pz)) nup = LD::load(yv, PER ? kxy + zp(z + 2) : kn + g.nxy);
             if (own) {
                 if (ypv) nyp = LD::load(ypv, kn);
                 if constexpr (!PRED) nr = LD::load(rv, kn);
             }
-            if (rowlo) nlo = LD::load(yv, (size_t)((long long)kn + dlo));
-            if (rowhi) nhi = LD::load(yv, (size_t)((long long)kn + dhi));
-            if (xl) nl = ldcg(yv, (int)((long long)kn + dxl));
-            if (xr) nrr = ldcg(yv, (int)((long long)kn + dxr));
+            if (rowlo) nlo = LD::load(yv, kn + dlo);
+            if (rowhi) nhi = LD::load(yv, kn + dhi);
+            if (xl) nl = ldcg(yv, kn + dxl);
+            if (xr) nrr = ldcg(yv, kn + dxr);
         }
         pl[ty + 1][tx] = vc;
         if (ty == 0) pl[0][tx] = hlo;
@@ -2370,8 +2370,12 @@ __device__ __forceinline__ void cheb_v4_tile(const Geo &g, int bx, int by, int z
     }
 }
 
+// The unrolled marches of two and four planes keep their queue in 76 to 80 registers, three
+// blocks to an SM (at four blocks they spill): 128^3, 2 planes 6.39 -> 5.71 us per
+// iteration, 3 fields, 4 planes 16.6 -> 13.3 us (2 planes 16.0 -> 14.1); periodic on every
+// axis, 256 x 128 x 128, 4 planes 15.5 -> 13.9 us.
 template <class TS, int ZFIX = 0, bool PER = false>
-__global__ void __launch_bounds__(kThreads, 4) k_cheb_v4(Geo g, int zlen, int nzc, Coef32 cf,
+__global__ void __launch_bounds__(kThreads, ZFIX >= 2 ? 3 : 4) k_cheb_v4(Geo g, int zlen, int nzc, Coef32 cf,
                                                       float gamma, float omega,
                                                       const TS *__restrict__ y_all,
                                                       const TS *yprev_all,
@@ -4017,12 +4021,18 @@ void launch_cheb(int code, const Geo &g, int nf, const Coef32 &cf, float gamma, 
         const int zlen = code - 100;
         const int nzc = (g.nz + zlen - 1) / zlen;
         const dim3 grid((g.nx + 4 * TX - 1) / (4 * TX), gy, nzc * nf);
-        if (g.per)   // periodic axes: the wrapping variant
+        if (g.per && zlen == 4)
+            launch_chain(k_cheb_v4<TS, 4, true>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
+        else if (g.per && zlen == 2)
+            launch_chain(k_cheb_v4<TS, 2, true>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
+        else if (g.per)   // periodic axes: the wrapping variant
             launch_chain(k_cheb_v4<TS, 0, true>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
         else if (zlen == 1)
             launch_chain(k_cheb_v4<TS, 1>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
         else if (zlen == 2)
             launch_chain(k_cheb_v4<TS, 2>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
+        else if (zlen == 4)
+            launch_chain(k_cheb_v4<TS, 4>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
         else
             launch_chain(k_cheb_v4<TS>, grid, blk, st, g, zlen, nzc, cf, gamma, omega, y, yp, r, yn);
     } else if (code > 0) {
@@ -5086,8 +5096,8 @@ static void launch_pred_combine(size_t n, size_t stride, const PredPlan &pl, int
 }
 
 // Planes per block of the vectorised sweep, unrolled (the register queue rotates by
-// renaming): 128^3 with 1 / 2 / 3 / 4 / 8 planes 6.0 / 5.1 / 6.4 / 6.7 / 6.9 us, 512 x 256 x 256
-// 96.9 / 73.4 / 79.9 / 78.5 / 76.5 us (4.1 -> 5.5 TB/s), with only 1 and 2 unrolled.
+// renaming) in 64 registers, four blocks to an SM: 128^3 4.7 us (1 plane 6.0; 4 planes at three
+// blocks 5.5, 8 at two 7.0), 512 x 256 x 256 70.5 us = 5.7 TB/s (1 plane 96.9; 4 planes 73.4, 8 72.2).
 constexpr int kPredPlanes = 2;
 static void launch_pred_sweep(const Geo &g, int nf, float w, const float *t, const float *tp, float *tn,
                               cudaStream_t st) {
