@@ -3170,7 +3170,9 @@ __device__ __forceinline__ float fld(const TS *p) {
 // +0.0 -- what the other engines add for a wall -- without a test.
 constexpr int kFlatSlots = kFlatCpt * kThreads + 4 * kFlatMaxNx + kFlatCpt * kThreads + 8;
 
-template <class TS, bool COH>
+// PRED: one step of the shared expansion's recurrence in difference form (see k_pred_v4)
+// instead: omega its factor, no r; a wall's neighbour is the cell itself.
+template <class TS, bool COH, bool PRED = false>
 __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk, int z0, int z1,
                                                float ce, float gamma, float omega, const float *sdg,
                                                const TS *yv, const TS *ypv, const TS *rv,
@@ -3195,7 +3197,7 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
     // per cell j (cell qt + j): its segment slot, and (packed) whether it is in the plane
     // and its number of x/y neighbours
     int so[C];
-    unsigned ownm = 0u, nnp = 0u, inl = 0u, inr = 0u;
+    unsigned ownm = 0u, nnp = 0u, inl = 0u, inr = 0u, inu = 0u, ind = 0u;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
         const int q = qt + j;
@@ -3204,6 +3206,8 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
         nnp |= (unsigned)((ix > 0) + (ix + 1 < nx) + (iy > 0) + (iy + 1 < g.ny)) << (3 * j);
         if (ix > 0) inl |= 1u << j;        // x - 1 is in the row (for j > 0: the thread's cell j - 1)
         if (ix + 1 < nx) inr |= 1u << j;   // x + 1 is in the row (for j < 3: its cell j + 1)
+        if (iy > 0) inu |= 1u << j;
+        if (iy + 1 < g.ny) ind |= 1u << j;
         so[j] = slot(q);
     }
     auto own = [&](int j) { return (ownm >> j) & 1u; };
@@ -3219,7 +3223,7 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
     const size_t pz0 = (size_t)z0 * pts;
     const TS *py = yv + pz0 + qt;
     const TS *pp = ypv ? ypv + pz0 + qt : nullptr;
-    const TS *pr = rv + pz0 + qt;
+    const TS *pr = PRED ? nullptr : rv + pz0 + qt;
     TS *po = ynv + pz0 + qt;
     const TS *ph = yv + pz0;
     const int dl0 = lo0 + t, dl1 = lo0 + t + S, dh0 = hi0 + t, dh1 = hi0 + t + S;
@@ -3231,7 +3235,7 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
             vc = LD::load(py, 0);
             if (z0 + 1 < nz) vup = LD::load(py + pts, 0);
             if (pp) yp = LD::load(pp, 0);
-            rc = LD::load(pr, 0);
+            if constexpr (!PRED) rc = LD::load(pr, 0);
         }
         if (hl0) ha0 = fld<TS, COH>(ph + dl0);
         if (hl1) ha1 = fld<TS, COH>(ph + dl1);
@@ -3247,7 +3251,7 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
             if (any) {
                 if (z + 2 < nz) nup = LD::load(py + 2 * pts, 0);
                 if (pp) nyp = LD::load(pp + pts, 0);
-                nrc = LD::load(pr + pts, 0);
+                if constexpr (!PRED) nrc = LD::load(pr + pts, 0);
             }
             if (hl0) na0 = fld<TS, COH>(ph + pts + dl0);
             if (hl1) na1 = fld<TS, COH>(ph + pts + dl1);
@@ -3275,6 +3279,17 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
                 // x neighbours inside the thread's vector come from its registers (the same
                 // values the segment holds; a row end is a wall, zero as its pad slot)
                 const float *c = sp + so[j];
+                if constexpr (PRED) {
+                    const float v = vcs[j];
+                    const float xl = j == 0 ? c[-1] : vcs[j > 0 ? j - 1 : 0];
+                    const float xr = j == C - 1 ? c[1] : vcs[j < C - 1 ? j + 1 : j];
+                    const float dxl = ((inl >> j) & 1u) ? xl - v : 0.0f, dxr = ((inr >> j) & 1u) ? xr - v : 0.0f;
+                    const float dyl = ((inu >> j) & 1u) ? c[-P] - v : 0.0f, dyr = ((ind >> j) & 1u) ? c[P] - v : 0.0f;
+                    const float dzl = z > 0 ? vds[j] - v : 0.0f, dzr = z + 1 < nz ? vus[j] - v : 0.0f;
+                    const float d = (dxl + dxr) + (dyl + dyr) + (dzl + dzr);
+                    o[j] = fmaf(omega, d, pp ? (v - yps[j]) + v : v);
+                    continue;
+                }
                 float sm = j == 0 ? c[-1] : (((inl >> j) & 1u) ? vcs[j - 1] : 0.0f);
                 sm += j == C - 1 ? c[1] : (((inr >> j) & 1u) ? vcs[j + 1] : 0.0f);
                 sm += c[-P];
@@ -3299,7 +3314,7 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
         hb1 = nb1;
         py += pts;
         if (pp) pp += pts;
-        pr += pts;
+        if constexpr (!PRED) pr += pts;
         po += pts;
         ph += pts;
     }
@@ -3317,6 +3332,10 @@ __device__ __forceinline__ void cheb_flat_tile(const Geo &g, int pts, int chunk,
 // rounds alternate X2/X1, and the last round (R >= 2) writes u^{n+1} over u^n in U
 // (read there only at the cell itself).  Per-item residual partials of each step's
 // last pass (and ||b||^2 partials of its first pass) are stored and reduced afterwards.
+// With the shared expansion (pred) a step's first round has no inner solve: its
+// refinement pass takes the expansion's increment, formed by k_bpred* launches before
+// either schedule starts, and reduces ||b||^2; under implicit Euler no pass then starts
+// the next step.
 template <class TS>
 struct SnapDesc {
     Geo g;
@@ -3335,6 +3354,13 @@ struct SnapDesc {
     DF *U, *X1, *X2, *B;
     TS *R, *Ya, *Yb;
     const float *omega;      // omega[k], k = 1 .. m-1
+    // the shared expansion of the steps' first rounds (see k_pred_combine), where the batch
+    // runs it: K steps of the recurrence with factor w, coefficients pc[k * steps + i], the
+    // vectors T_k of one field (nz pts values each) and every step's increment D of all
+    int K;
+    float w;
+    const float *pc;
+    float *T, *D;
 };
 
 struct BItem {
@@ -3369,8 +3395,9 @@ template <bool COH, class TS> __device__ __forceinline__ float bld(const TS *p, 
 // hand, so the next first residual is c L x = (x - A x) / theta (and the Crank-Nicolson
 // right-hand side x + c/2 L x), and that step's ||b||^2 partial goes to part_next.
 template <class TS, bool COH>
-__device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, const BItem &it, bool first,
-                                               int round, int R, double *part, double *part_next) {
+__device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, int nf, const BItem &it, bool first,
+                                               int round, int R, double *part, double *part_next,
+                                               int pstep = -1, double *part_b = nullptr) {
     // the descriptor lives in global memory: copy what the sweep reads into registers
     // (through a reference every store would force the compiler to reload it)
     const Geo g = d.g;
@@ -3423,7 +3450,9 @@ __device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, const BIte
         const DF *b = (scheme == 1 ? d.B : d.U) + off;
         DF *bo = d.B + off;
         const TS *dd = d.Yb + off_ts;
-        const bool next = part_next != nullptr;
+        if constexpr (sizeof(TS) == 4)   // the step's first round: the increment from the expansion
+            if (pstep >= 0) dd = d.D + (size_t)pstep * nf * g.nz * d.pts + off_ts;
+        const bool next = part_next != nullptr, wantb = part_b != nullptr;
         engine(
             [&](int k, int kt) { return DFd{bld_df<COH>(xin, k), bld<COH>(dd, kt)}; },
             [](DFd v) { return df_add_f(v.x, v.d); }, [&](int k) { return bld_df<COH>(b, k); },
@@ -3432,6 +3461,10 @@ __device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, const BIte
                 const DF lx = df_lap(sm, v, (float)nn);
                 float rf = df_f(df_res(bk, v, cf_ce, lx));
                 acc = fmaf(rf, rf, acc);
+                if (wantb) {
+                    const float bf = df_f(bk);
+                    acc_b = fmaf(bf, bf, acc_b);
+                }
                 if (next) {
                     DF cl = df_mul(cf_ce, lx);        // = theta c L v
                     DF bn = v;
@@ -3449,6 +3482,7 @@ __device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, const BIte
             });
         const double tb = block_sum_f(acc_b);
         if (is_thread0() && next) *part_next = tb;
+        if (is_thread0() && wantb) *part_b = tb;
     }
     double tot = block_sum_f(acc);
     if (is_thread0() && part) *part = tot;
@@ -3494,14 +3528,14 @@ template <class TS>
 __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__restrict__ sd, int nsnap,
                                                       int nf, const BItem *__restrict__ ritems,
                                                       int nr, const BItem *__restrict__ citems,
-                                                      int nc, int nsteps, int R, int mmax,
-                                                      double *__restrict__ part_rr,
+                                                      int nc, int nsteps, int R, int mmax, int pred,
+                                                      int cn, double *__restrict__ part_rr,
                                                       double *__restrict__ part_bb, GridBar *gb,
                                                       long long budget) {
-    // phase 0: u^0 -> double-float
+    // phase 0: u^0 -> double-float (with the expansion it has run: k_bconvert)
     const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.y * TX + threadIdx.x;
     const size_t nthr = (size_t)gridDim.x * kThreads;
-    for (int s = 0; s < nsnap; ++s) {
+    for (int s = 0; s < (pred ? 0 : nsnap); ++s) {
         const size_t cnt = (size_t)sd[s].g.n * nf;
         const double *u = sd[s].cells;
         DF *U = sd[s].U;
@@ -3513,15 +3547,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
     }
     if (!grid_sync(gb, gridDim.x, budget)) return;
     for (int step = 0; step < nsteps; ++step) {
-        if (step == 0) {   // later steps were started by the previous step's last pass
+        if (step == 0 && (!pred || cn)) {   // later steps were started by the previous step's last pass
             for (int i = blockIdx.x; i < nr; i += gridDim.x) {
                 const BItem it = ritems[i];
-                batched_refine<TS, true>(sd[it.snap], it, true, 0, R, part_bb + i, nullptr);
+                batched_refine<TS, true>(sd[it.snap], nf, it, true, 0, R, part_bb + i, nullptr);
             }
             if (!grid_sync(gb, gridDim.x, budget)) return;
         }
         for (int round = 1; round <= R; ++round) {
-            for (int k = 1; k < mmax; ++k) {
+            const bool shared = pred && round == 1;
+            for (int k = 1; k < (shared ? 1 : mmax); ++k) {
                 for (int i = blockIdx.x; i < nc; i += gridDim.x) {
                     const BItem it = citems[i];
                     if (k < sd[it.snap].m) batched_cheb<TS, true>(sd[it.snap], it, k);
@@ -3530,10 +3565,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
             }
             for (int i = blockIdx.x; i < nr; i += gridDim.x) {
                 const BItem it = ritems[i];
-                batched_refine<TS, true>(sd[it.snap], it, false, round, R,
+                batched_refine<TS, true>(sd[it.snap], nf, it, false, round, R,
                                    round == R ? part_rr + (size_t)step * nr + i : nullptr,
-                                   round == R && step + 1 < nsteps ? part_bb + (size_t)(step + 1) * nr + i
-                                                                   : nullptr);
+                                   round == R && step + 1 < nsteps && (!pred || cn)
+                                       ? part_bb + (size_t)(step + 1) * nr + i
+                                       : nullptr,
+                                   shared ? step : -1,
+                                   shared && !cn ? part_bb + (size_t)step * nr + i : nullptr);
             }
             if (step + 1 < nsteps || round < R)
                 if (!grid_sync(gb, gridDim.x, budget)) return;
@@ -3571,16 +3609,92 @@ __global__ void __launch_bounds__(kThreads, 3) k_bcheb(const SnapDesc<TS> *__res
 // first: a step's first pass (||b||^2 partial to part[i]); else round `round` of R
 // (||r||^2 partial to part[i] when part, the next step's ||b||^2 to part_next[i]).
 template <class TS>
-__global__ void __launch_bounds__(kThreads, 3) k_brefine(const SnapDesc<TS> *__restrict__ sd,
+__global__ void __launch_bounds__(kThreads, 3) k_brefine(const SnapDesc<TS> *__restrict__ sd, int nf,
                                                       const BItem *__restrict__ ritems, int first,
                                                       int round, int R, double *part,
-                                                      double *part_next) {
+                                                      double *part_next, int pstep, double *part_b) {
     chain_wait();
     chain_release();
     const int i = blockIdx.x;
     const BItem it = ritems[i];
-    batched_refine<TS, false>(sd[it.snap], it, first != 0, round, R, part ? part + i : nullptr,
-                              part_next ? part_next + i : nullptr);
+    batched_refine<TS, false>(sd[it.snap], nf, it, first != 0, round, R, part ? part + i : nullptr,
+                              part_next ? part_next + i : nullptr, pstep, part_b ? part_b + i : nullptr);
+}
+
+// The shared expansion of a batch, one field of every snapshot at a time (so that the
+// vectors T_k take the room of one field): T_0, the recurrence's step k, the combination.
+// 64 snapshots of 32 to 96 cells a side, 5 fields, b = 3 dx, 10 steps: 29 recurrence steps of
+// 80 us per field (3.3 TB/s: the flat tile's barriers and neighbour tests) and 0.9 ms per
+// combination (4.0 TB/s) take the place of 130 k_bcheb launches of 335 us; the call 112 ->
+// 84 ms.
+template <class TS>
+__global__ void __launch_bounds__(kThreads) k_bpred_start(const SnapDesc<TS> *__restrict__ sd, int f) {
+    chain_wait();
+    chain_release();
+    const SnapDesc<TS> &d = sd[blockIdx.y];
+    const int n = d.g.n, nxy = d.g.nxy, pad = d.pts - nxy;
+    const DF *u = d.U + (size_t)f * n;
+    float *t = d.T;
+    for (int i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads)
+        t[i + (pad ? i / nxy * pad : 0)] = u[i].hi;
+}
+
+template <class TS>
+__global__ void __launch_bounds__(kThreads, 4) k_bpred(const SnapDesc<TS> *__restrict__ sd,
+                                                    const BItem *__restrict__ items, int k) {
+    chain_wait();
+    chain_release();
+    const BItem it = items[blockIdx.x];
+    const SnapDesc<TS> &d = sd[it.snap];
+    if (k >= d.K) return;
+    const Geo g = d.g;
+    const int z0 = it.zf * d.zlen, z1 = min(g.nz, z0 + d.zlen);
+    const size_t stride = (size_t)g.nz * d.pts;
+    const float *t = d.T + k * stride;
+    cheb_flat_tile<float, false, true>(g, d.pts, it.bx, z0, z1, 0.f, 0.f, k ? 2.0f * d.w : d.w, nullptr, t,
+                                       k ? t - stride : nullptr, nullptr, d.T + (k + 1) * stride);
+}
+
+// k_pred_combine for one field of every snapshot (blockIdx.y); the coefficients differ per
+// snapshot and come through shared memory.
+template <class TS, int NS>
+__global__ void __launch_bounds__(kThreads) k_bpred_combine(const SnapDesc<TS> *__restrict__ sd, int nf, int f,
+                                                            int steps) {
+    chain_wait();
+    chain_release();
+    __shared__ float a[(kPredMaxK + 1) * NS];
+    const SnapDesc<TS> &d = sd[blockIdx.y];
+    const int K = d.K;
+    const float *pc = d.pc;
+    for (int i = threadIdx.x; i < (K + 1) * NS; i += kThreads) {
+        const int k = i / NS, q = i - k * NS;
+        a[i] = q < steps ? pc[k * steps + q] : 0.0f;
+    }
+    __syncthreads();
+    const size_t stride = (size_t)d.g.nz * d.pts, dstride = stride * nf;
+    const float *t = d.T;
+    float *o = d.D + (size_t)f * stride;
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < stride / 4; i += (size_t)gridDim.x * kThreads) {
+        float2 lo[NS], hi[NS];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) lo[q] = hi[q] = make_float2(0.f, 0.f);
+        const float *tp = t + 4 * i;
+#pragma unroll 4
+        for (int k = 0; k <= K; ++k, tp += stride) {
+            const float4 v = *reinterpret_cast<const float4 *>(tp);
+            const float2 va = make_float2(v.x, v.y), vb = make_float2(v.z, v.w);
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                const float w = a[k * NS + q];
+                lo[q] = fma2(va, make_float2(w, w), lo[q]);
+                hi[q] = fma2(vb, make_float2(w, w), hi[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NS; ++q)
+            if (q < steps)
+                *reinterpret_cast<float4 *>(o + q * dstride + 4 * i) = make_float4(lo[q].x, lo[q].y, hi[q].x, hi[q].y);
+    }
 }
 
 // hist[(step * nsnap + s) * nf + f] = (sum of ||r||^2 partials, sum of ||b||^2 partials)
@@ -5720,6 +5834,11 @@ struct BatchPlan {
     std::vector<float> omegas;
     std::vector<size_t> omega_off;
     std::vector<BItem> ritems, citems;
+    std::vector<BItem> pitems;     // the shared expansion's sweeps (one field)
+    std::vector<float> pcoef;
+    std::vector<size_t> pc_off;
+    bool pred = false;
+    int Kmax = 0;
     std::vector<int> first_item;   // per (snapshot, field), into ritems
     int mmax = 2;
     long long cells_total = 0;
@@ -5728,12 +5847,16 @@ struct BatchPlan {
 template <class TS>
 static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *const *cells,
                             const cg_params *p, const double *bandwidths, int zlen,
-                            BatchPlan<TS> &P) {
+                            bool want_pred, BatchPlan<TS> &P) {
     const bool cn = p->scheme == CG_SCHEME_CRANK_NICOLSON;
     const double eps_inner = sizeof(TS) == 2 ? 2e-3 : 1e-6;
     P = BatchPlan<TS>();
     P.descs.resize((size_t)nsnap);
     P.omega_off.resize((size_t)nsnap);
+    P.pc_off.resize((size_t)nsnap);
+    // the shared expansion serves the batch where it pays for every snapshot: FP32 inner
+    // storage, one run of steps, rows the flat-plane engine takes
+    P.pred = sizeof(TS) == 4 && want_pred && p->nsteps <= kPredMaxSteps;
     for (int s = 0; s < nsnap; ++s) {
         cg_mesh *m = meshes[s];
         SnapDesc<TS> &d = P.descs[s];
@@ -5752,6 +5875,14 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         const double theta = 0.5 * (lmax + 1.0), delta = 0.5 * (lmax - 1.0);
         int mi = cheb_iters(lmax, eps_inner);
         if (mi < 2) mi = 2;
+        const PredPlan *pl = P.pred ? &pred_plan(m, p->scheme, p->nsteps, mi, c, lmax) : nullptr;
+        if (pl && (!pl->use || m->nx > kFlatMaxNx)) P.pred = false;
+        if (!P.pred) pl = nullptr;
+        if (want_pred && sizeof(TS) == 4 && !P.pred && s > 0 && P.Kmax > 0)   // start over without it
+            return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, P);
+        // (counts are even here, so the estimate's last two iterations, below what the fields'
+        // rounding leaves, are given up: 14 instead of 16 at b = 3 dx, errors as before)
+        if (pl) mi = std::max(mi, pl->maxm - 2);
         if (mi & 1) ++mi;
         d.m = mi;
         P.mmax = std::max(P.mmax, mi);
@@ -5784,8 +5915,22 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         // per-snapshot solver vectors, owned by the snapshot's mesh
         const size_t v64 = align_up((size_t)n * nf * 8);
         const size_t vts = align_up((size_t)m->nz * d.pts * nf * sizeof(TS));
+        const size_t t1 = align_up((size_t)m->nz * d.pts * 4);
+        if (pl) {
+            if (m->ws_diffuse.ensure(4 * v64 + 3 * vts + (pl->maxK + 1) * t1 + p->nsteps * vts) != CG_OK)
+                return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, P);
+            d.K = pl->K[0];
+            d.w = (float)(2.0 * ce / (lmax - 1.0));
+            P.Kmax = std::max(P.Kmax, d.K);
+            P.pc_off[s] = P.pcoef.size();
+            P.pcoef.insert(P.pcoef.end(), pl->coef[0].begin(), pl->coef[0].end());
+            for (int zc = 0; zc < d.nzc; ++zc)
+                for (int ch = 0; ch < d.nch; ++ch) P.pitems.push_back(BItem{s, ch, 0, zc});
+        }
         CGK_TRY(m->ws_diffuse.ensure(4 * v64 + 3 * vts));
         char *wb = m->ws_diffuse.as<char>();
+        d.D = (float *)(wb + 4 * v64 + 3 * vts);
+        d.T = d.D + (size_t)m->nz * d.pts * nf * p->nsteps;
         d.U = (DF *)wb;
         d.X1 = (DF *)(wb + v64);
         d.X2 = (DF *)(wb + 2 * v64);
@@ -5822,7 +5967,7 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
 struct BatchArena {
     char *ab = nullptr;
     size_t o_desc = 0, o_om = 0, o_ri = 0, o_ci = 0, o_fi = 0, o_prr = 0, o_pbb = 0, o_hist = 0,
-           o_gb = 0, o_bad = 0, o_out = 0, o_mass = 0, total = 0;
+           o_gb = 0, o_bad = 0, o_out = 0, o_mass = 0, o_pi = 0, o_pc = 0, total = 0;
     size_t nh = 0;
 };
 
@@ -5843,7 +5988,9 @@ static BatchArena batch_layout(const BatchPlan<TS> &P, int nsnap, int nf, int ns
     A.o_bad = align_up(A.o_gb + sizeof(GridBar));
     A.o_out = align_up(A.o_bad + sizeof(unsigned int));
     A.o_mass = align_up(A.o_out + (size_t)nsnap * sizeof(double *));
-    A.total = align_up(A.o_mass + 2 * (size_t)nsnap * nf * 8);
+    A.o_pi = align_up(A.o_mass + 2 * (size_t)nsnap * nf * 8);
+    A.o_pc = align_up(A.o_pi + P.pitems.size() * sizeof(BItem));
+    A.total = align_up(A.o_pc + P.pcoef.size() * sizeof(float));
     return A;
 }
 
@@ -5853,7 +6000,16 @@ template <class TS>
 static cg_status batch_upload(BatchPlan<TS> &P, BatchArena &A, char *ab, int nsnap,
                               double *const *cells, cudaStream_t st) {
     A.ab = ab;
-    for (int s = 0; s < nsnap; ++s) P.descs[s].omega = (const float *)(ab + A.o_om) + P.omega_off[s];
+    for (int s = 0; s < nsnap; ++s) {
+        P.descs[s].omega = (const float *)(ab + A.o_om) + P.omega_off[s];
+        P.descs[s].pc = (const float *)(ab + A.o_pc) + P.pc_off[s];
+    }
+    if (P.pred) {
+        CGK_CUDA(cudaMemcpyAsync(ab + A.o_pi, P.pitems.data(), P.pitems.size() * sizeof(BItem),
+                                 cudaMemcpyHostToDevice, st));
+        CGK_CUDA(cudaMemcpyAsync(ab + A.o_pc, P.pcoef.data(), P.pcoef.size() * sizeof(float),
+                                 cudaMemcpyHostToDevice, st));
+    }
     CGK_CUDA(cudaMemcpyAsync(ab + A.o_desc, P.descs.data(), P.descs.size() * sizeof(SnapDesc<TS>),
                              cudaMemcpyHostToDevice, st));
     CGK_CUDA(cudaMemcpyAsync(ab + A.o_om, P.omegas.data(), P.omegas.size() * sizeof(float),
@@ -5870,6 +6026,34 @@ static cg_status batch_upload(BatchPlan<TS> &P, BatchArena &A, char *ab, int nsn
     return CG_OK;
 }
 
+// The launches of the shared expansion (before either schedule): u^0 -> double-float, then
+// per field the recurrence and the combination.
+template <class TS>
+static cg_status batch_issue_pred(const BatchPlan<TS> &P, const BatchArena &A, int nf, int nsteps,
+                                  cudaStream_t st) {
+    const SnapDesc<TS> *dsd = (const SnapDesc<TS> *)(A.ab + A.o_desc);
+    const BItem *items = (const BItem *)(A.ab + A.o_pi);
+    const int nsnap = (int)P.descs.size();
+    const double cells = (double)P.cells_total;
+    CGK_LAUNCH("bconvert", cells * nf * 16.0, st,
+               launch_chain(k_bconvert<TS>, dim3(num_sms() * 2, nsnap), dim3(TX, TY), st, dsd, nf));
+    for (int f = 0; f < nf; ++f) {
+        CGK_LAUNCH("bpred_start", cells * 12.0, st,
+                   launch_chain(k_bpred_start<TS>, dim3(num_sms(), nsnap), dim3(kThreads), st, dsd, f));
+        for (int k = 0; k < P.Kmax; ++k)
+            CGK_LAUNCH("bpred", cells * 12.0, st,
+                       launch_chain(k_bpred<TS>, dim3((unsigned)P.pitems.size()), dim3(TX, TY), st, dsd, items, k));
+        const dim3 grid(num_sms(), nsnap);
+        CGK_LAUNCH("bpred_combine", cells * 4.0 * (P.Kmax + 1 + nsteps), st, {
+            if (nsteps <= 5) launch_chain(k_bpred_combine<TS, 5>, grid, dim3(kThreads), st, dsd, nf, f, nsteps);
+            else if (nsteps <= 10) launch_chain(k_bpred_combine<TS, 10>, grid, dim3(kThreads), st, dsd, nf, f, nsteps);
+            else launch_chain(k_bpred_combine<TS, kPredMaxSteps>, grid, dim3(kThreads), st, dsd, nf, f, nsteps);
+        });
+    }
+    CGK_CUDA(cudaGetLastError());
+    return CG_OK;
+}
+
 // The phased schedule's launches on stream st (one per phase, in k_batched's order),
 // each with its algorithmic bytes: a Chebyshev iteration reads y_k, y_{k-1} and r and
 // writes y_{k+1} of every snapshot that runs it; a refinement pass reads the double-float
@@ -5877,7 +6061,7 @@ static cg_status batch_upload(BatchPlan<TS> &P, BatchArena &A, char *ab, int nsn
 // and the first Chebyshev iterate.
 template <class TS>
 static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A, int nf,
-                                    int nsteps, int R, cudaStream_t st) {
+                                    int nsteps, int R, bool pred, cudaStream_t st) {
     char *ab = A.ab;
     const SnapDesc<TS> *dsd = (const SnapDesc<TS> *)(ab + A.o_desc);
     const BItem *dri = (const BItem *)(ab + A.o_ri), *dci = (const BItem *)(ab + A.o_ci);
@@ -5891,22 +6075,26 @@ static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A,
     for (const auto &d : P.descs)
         for (int k = 1; k < d.m; ++k) cheb_bytes[(size_t)k] += (double)d.g.n * nf * 4.0 * sizeof(TS);
     const double ref_bytes = cells_f * (24.0 + 3.0 * sizeof(TS));
-    CGK_LAUNCH("bconvert", cells_f * 16.0, st,
-               launch_chain(k_bconvert<TS>, dim3(num_sms() * 2, nsnap), dim3(TX, TY), st, dsd, nf));
+    const bool cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON;
+    if (!pred)
+        CGK_LAUNCH("bconvert", cells_f * 16.0, st,
+                   launch_chain(k_bconvert<TS>, dim3(num_sms() * 2, nsnap), dim3(TX, TY), st, dsd, nf));
     for (int step = 0; step < nsteps; ++step) {
-        if (step == 0)
+        if (step == 0 && (!pred || cn))
             CGK_LAUNCH(rname, cells_f * (8.0 + 2.0 * sizeof(TS)), st,
-                       launch_chain(k_brefine<TS>, dim3(nr), dim3(TX, TY), st, dsd, dri, 1, 0, R, pbb,
-                                    (double *)nullptr));
+                       launch_chain(k_brefine<TS>, dim3(nr), dim3(TX, TY), st, dsd, nf, dri, 1, 0, R, pbb,
+                                    (double *)nullptr, -1, (double *)nullptr));
         for (int round = 1; round <= R; ++round) {
-            for (int k = 1; k < P.mmax; ++k)
+            const bool shared = pred && round == 1;
+            for (int k = 1; k < (shared ? 1 : P.mmax); ++k)
                 CGK_LAUNCH(cname, cheb_bytes[(size_t)k], st,
                            launch_chain(k_bcheb<TS>, dim3(nc), dim3(TX, TY), st, dsd, dci, k));
             double *part = round == R ? prr + (size_t)step * nr : nullptr;
-            double *next = round == R && step + 1 < nsteps ? pbb + (size_t)(step + 1) * nr : nullptr;
+            double *next = round == R && step + 1 < nsteps && (!pred || cn) ? pbb + (size_t)(step + 1) * nr : nullptr;
+            double *partb = shared && !cn ? pbb + (size_t)step * nr : nullptr;
             CGK_LAUNCH(rname, ref_bytes, st,
-                       launch_chain(k_brefine<TS>, dim3(nr), dim3(TX, TY), st, dsd, dri, 0, round, R,
-                                    part, next));
+                       launch_chain(k_brefine<TS>, dim3(nr), dim3(TX, TY), st, dsd, nf, dri, 0, round, R,
+                                    part, next, shared ? step : -1, partb));
         }
     }
     CGK_CUDA(cudaGetLastError());
@@ -5919,8 +6107,8 @@ static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A,
 // when a step missed the tolerance).
 template <class TS>
 static cg_status batch_issue(const BatchPlan<TS> &P, const BatchArena &A, int nsnap, int nf,
-                             int nsteps, int R, int G, long long budget, double tol2, bool final,
-                             cudaStream_t st) {
+                             int nsteps, int R, int G, long long budget, double tol2, bool pred,
+                             bool final, cudaStream_t st) {
     char *ab = A.ab;
     const SnapDesc<TS> *dsd = (const SnapDesc<TS> *)(ab + A.o_desc);
     const BItem *dri = (const BItem *)(ab + A.o_ri), *dci = (const BItem *)(ab + A.o_ci);
@@ -5932,8 +6120,10 @@ static cg_status batch_issue(const BatchPlan<TS> &P, const BatchArena &A, int ns
     CGK_CUDA(cudaMemsetAsync(gb, 0, sizeof(GridBar), st));
     CGK_CUDA(cudaMemsetAsync(bad, 0, sizeof(unsigned int), st));
     int a_ns = nsnap, a_nf = nf, a_nr = nr, a_nc = nc, a_steps = nsteps, a_R = R, a_mm = P.mmax;
+    int a_pred = pred ? 1 : 0, a_cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON ? 1 : 0;
     long long a_budget = budget;
-    void *args[] = {&dsd, &a_ns, &a_nf, &dri, &a_nr, &dci, &a_nc, &a_steps, &a_R, &a_mm,
+    if (pred) CGK_TRY(batch_issue_pred(P, A, nf, nsteps, st));
+    void *args[] = {&dsd, &a_ns, &a_nf, &dri, &a_nr, &dci, &a_nc, &a_steps, &a_R, &a_mm, &a_pred, &a_cn,
                     &prr, &pbb, &gb, &a_budget};
     double bytes = 0.0;
     for (const auto &d : P.descs)
@@ -5945,7 +6135,7 @@ static cg_status batch_issue(const BatchPlan<TS> &P, const BatchArena &A, int ns
                    CGK_CUDA(cudaLaunchCooperativeKernel((const void *)k_batched<TS>, dim3(G),
                                                         dim3(TX, TY), args, 0, st)));
     } else {
-        CGK_TRY(batch_issue_phased(P, A, nf, nsteps, R, st));
+        CGK_TRY(batch_issue_phased(P, A, nf, nsteps, R, pred, st));
     }
     CGK_LAUNCH("batched_hist", 16.0 * nsteps * nr, st,
                k_batched_hist<<<(unsigned)A.nh, kThreads, 0, st>>>(
@@ -6001,7 +6191,7 @@ static cg_status batch_tune(int nsnap, cg_mesh *const *meshes, int nf, double *c
         const int z = code % kPhasedCode;
         const int g = code >= kPhasedCode ? 0 : G;
         BatchPlan<TS> P;
-        rc = batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, z, P);
+        rc = batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, z, true, P);
         if (rc != CG_OK) break;
         BatchArena A = batch_layout(P, nsnap, nf, 1);
         rc = m0->ws_batch.ensure(A.total);
@@ -6011,7 +6201,7 @@ static cg_status batch_tune(int nsnap, cg_mesh *const *meshes, int nf, double *c
         float ms = 0.f;
         for (int rep = 0; rep < 2 && rc == CG_OK; ++rep) {   // the first run warms up
             if (cudaEventRecord(e0, st) != cudaSuccess) rc = fail(CG_ECUDA, "event");
-            if (rc == CG_OK) rc = batch_issue(P, A, nsnap, nf, 1, 2, g, budget, 0.0, false, st);
+            if (rc == CG_OK) rc = batch_issue(P, A, nsnap, nf, 1, 2, g, budget, 0.0, false, false, st);
             if (rc == CG_OK && cudaEventRecord(e1, st) != cudaSuccess) rc = fail(CG_ECUDA, "event");
             if (rc == CG_OK && cudaEventSynchronize(e1) != cudaSuccess) rc = fail(CG_ECUDA, "sync");
             if (rc == CG_OK) cudaEventElapsedTime(&ms, e0, e1);
@@ -6065,7 +6255,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
     const int Gx = code >= kPhasedCode ? 0 : G;
     if (zlen < 1) return fail(CG_EINVAL, "cg_diffuse_batched: bad sweep_shape %d", code);
     BatchPlan<TS> P;
-    CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, P));
+    CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, p->max_rounds <= 0 || p->max_rounds >= 2, P));
     BatchArena A = batch_layout(P, nsnap, nf, p->nsteps);
     CGK_TRY(m0->ws_batch.ensure(A.total));
     CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
@@ -6124,6 +6314,8 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
         key.grid = Gx;
         key.zlen = zlen;
         key.phased = Gx == 0 ? 1 : 0;
+        key.pred = P.pred ? P.Kmax : 0;
+        key.np = (int)P.pitems.size();
         key.tsize = (int)sizeof(TS);
         key.scheme = p->scheme;
         key.budget = budget;
@@ -6151,7 +6343,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
             cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             cg_status is = CG_OK;
             if (ce == cudaSuccess) {
-                is = batch_issue(P, A, nsnap, nf, p->nsteps, R, Gx, budget, tol2, true, cs);
+                is = batch_issue(P, A, nsnap, nf, p->nsteps, R, Gx, budget, tol2, P.pred, true, cs);
                 cudaGraph_t graph = nullptr;
                 ce = cudaStreamEndCapture(cs, &graph);
                 if (ce == cudaSuccess && is == CG_OK) ce = cudaGraphInstantiate(&e.exec, graph, 0);
@@ -6196,6 +6388,9 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
                     // the first pass of the first step, then R rounds of m applications
                     // per step (a step's last pass also starts the next one)
                     long long a = 1 + (long long)p->nsteps * R * d.m;
+                    if (P.pred)   // the expansion, then per step one pass and R - 1 rounds
+                        a = (p->scheme == CG_SCHEME_CRANK_NICOLSON ? 1 : 0) + d.K +
+                            (long long)p->nsteps * (1 + (long long)(R - 1) * d.m);
                     apps += a;
                     upd += a * d.g.n;
                 }

@@ -77,3 +77,36 @@ def test_shared_expansion_saves_applications_and_yields_to_limits():
         mesh.close()
     assert rep["iters"] < 0.8 * tight["iters"]
     assert np.max(np.abs(got - x.cpu().numpy())) <= 2e-12 * 40
+
+
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("nsteps", [2, 6, 20, 21])
+def test_batches_match_single_meshes(nsteps, scheme):
+    """Uneven snapshots (odd and single-cell sides, rows over one tile) with bandwidths of
+    their own: both schedules give the same bits, and each snapshot what its own call gives
+    to the tolerance above (21 steps are more than a batch's one run: own solves)."""
+    import torch
+
+    import paper_1409_0001_gb300 as cg
+    dims = [(33, 20, 17), (5, 1, 1), (64, 9, 3), (1, 30, 4), (130, 6, 5), (40, 40, 12)]
+    cs = [0.1, 0.3, 0.05, 0.2, 0.4, 0.15]
+    rng = np.random.default_rng(nsteps)
+    us = [np.stack([rng.random(a * b * d), rng.standard_normal(a * b * d)]) for a, b, d in dims]
+    bw = [2.0 * np.sqrt(c * nsteps) for c in cs]
+    got = {}
+    for shape in (4, 504, 516):
+        meshes = [cg.StructuredMesh(d, (0, 0, 0), 1.0) for d in dims]
+        x = [torch.from_numpy(u).cuda() for u in us]
+        _, rep = cg.diffuse_batched(meshes, x, cg.Params(nsteps=nsteps, scheme=scheme, sweep_shape=shape,
+                                                         precision=cg.PREC_FP32_DF_REFINE),
+                                    bandwidths=bw, report=True)
+        assert rep["final_rel_residual"] <= 1e-13
+        got[shape] = [t.cpu().numpy() for t in x]
+        for m in meshes:
+            m.close()
+    for s, d in enumerate(dims):
+        assert np.array_equal(got[4][s], got[504][s]) and np.array_equal(got[504][s], got[516][s])
+        lone, _ = solve(cg, d, us[s], cs[s], nsteps, scheme, (0, 0, 0))
+        for f in (0, 1):
+            bound = 2e-13 * nsteps * np.sqrt(np.mean(us[s][f] ** 2)) * 40
+            assert np.max(np.abs(got[504][s][f] - lone[f])) <= bound
