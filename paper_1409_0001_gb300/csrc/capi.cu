@@ -466,6 +466,10 @@ cg_status cg_destroy_mesh(cg_mesh *m) {
     m->h_small.release();
     for (auto &e : m->graphs) graph_release(e);
     m->graphs.clear();
+    for (cudaEvent_t e : m->dep_ev)
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : m->dif_ev)
+        if (e) cudaEventDestroy(e);
     if (m->capture_stream) cudaStreamDestroy(m->capture_stream);
     for (cudaStream_t a : m->aux_streams) cudaStreamDestroy(a);
     if (m->kind != MESH_STRUCTURED) tet_release(m);
@@ -565,12 +569,16 @@ cg_status cg_deposit(cg_mesh *m, int64_t n, const double *pos, int nfields, cons
 
 static cg_status diffuse_impl(cg_mesh *m, int nf, double *cells, const cg_params *p,
                               cg_report *rep, cudaStream_t st) {
+    // the events are kept with the mesh; the masses before the smoothing are read with
+    // those after it
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    const int nm = nf < CG_REPORT_MAX_FIELDS ? nf : CG_REPORT_MAX_FIELDS;
     if (rep) {
-        CGK_TRY(field_mass(m, nf < CG_REPORT_MAX_FIELDS ? nf : CG_REPORT_MAX_FIELDS, cells,
-                           rep->mass_in, st));
-        CGK_CUDA(cudaEventCreate(&e0));
-        CGK_CUDA(cudaEventCreate(&e1));
+        CGK_TRY(field_mass_keep(m, nm, cells, 0, st));
+        for (int i = 0; i < 2; ++i)
+            if (!m->dif_ev[i]) CGK_CUDA(cudaEventCreate(&m->dif_ev[i]));
+        e0 = m->dif_ev[0];
+        e1 = m->dif_ev[1];
         CGK_CUDA(cudaEventRecord(e0, st));
     }
     cg_status s;
@@ -584,17 +592,14 @@ static cg_status diffuse_impl(cg_mesh *m, int nf, double *cells, const cg_params
     }
     if (rep) {
         cudaEventRecord(e1, st);
-        cudaEventSynchronize(e1);
+        const bool after = s == CG_OK || s == CG_ENOCONV;
+        cg_status s2 = after ? field_mass_keep(m, nm, cells, 1, st) : CG_OK;
+        if (s2 == CG_OK) s2 = field_mass_read(m, nm, rep->mass_in, after ? rep->mass_out : nullptr, st);
+        else cudaEventSynchronize(e1);
         float ms = 0;
         cudaEventElapsedTime(&ms, e0, e1);
         rep->ms_diffuse = ms;
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        if (s == CG_OK || s == CG_ENOCONV) {
-            cg_status s2 = field_mass(m, nf < CG_REPORT_MAX_FIELDS ? nf : CG_REPORT_MAX_FIELDS,
-                                      cells, rep->mass_out, st);
-            if (s == CG_OK) s = s2;
-        }
+        if (s == CG_OK) s = s2;
     }
     return s;
 }

@@ -197,10 +197,20 @@ __global__ void k_scan_top(uint32_t *__restrict__ sums, int64_t nb) {
     }
 }
 
+// sums_raw: block_off holds the chunks' sums, not yet scanned, and every block adds those of
+// the chunks before it (at most kScanInline, from L2): one launch of 5 to 7 us less
+constexpr int kScanInline = 2048;
 __global__ void k_scan_down(const uint32_t *in, uint32_t *out, int64_t n,
-                            const uint32_t *__restrict__ block_off) {
+                            const uint32_t *__restrict__ block_off, bool sums_raw) {
     __shared__ uint32_t tile[kScanChunk + kScanChunk / 32];
+    __shared__ uint32_t before[kThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanChunk;
+    if (sums_raw) {
+        uint32_t b = 0;
+        for (int j = threadIdx.x; j < (int)blockIdx.x; j += kThreads) b += block_off[j];
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_down_sync(0xffffffffu, b, o);
+        if ((threadIdx.x & 31) == 0) before[threadIdx.x >> 5] = b;
+    }
     for (int j = threadIdx.x; j < kScanChunk; j += kThreads) {
         int64_t i = base + j;
         tile[j + (j >> 5)] = i < n ? in[i] : 0;
@@ -216,7 +226,13 @@ __global__ void k_scan_down(const uint32_t *in, uint32_t *out, int64_t n,
         s += v[q];
     }
     __syncthreads();
-    uint32_t ex = block_exclusive_scan(s, nullptr) + block_off[blockIdx.x];
+    uint32_t ex = block_exclusive_scan(s, nullptr);
+    if (sums_raw) {
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) ex += before[w];
+    } else {
+        ex += block_off[blockIdx.x];
+    }
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
         int j = t0 + q;
@@ -354,17 +370,24 @@ __global__ void k_scatter_cells(int64_t n, const int32_t *__restrict__ cell,
                                 const uint32_t *__restrict__ off, const uint32_t *__restrict__ ranks,
                                 uint32_t *__restrict__ idx) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        idx[off[cell[i]] + ranks[i]] = (uint32_t)i;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t c = cell[i];   // -1: outside (the call is about to fail)
+        if (c >= 0) idx[off[c] + ranks[i]] = (uint32_t)i;
+    }
 }
 
 // eps_c = (sum of the cell's weights in ascending particle index, FP64 from +0.0) / V_c;
-// an empty cell gets +0.0.
+// an empty cell gets +0.0.  Bound by the random gathers of the weights (a 32-byte sector per
+// particle and field; ids in registers and a cell's loads in flight together gained nothing
+// with one field, and four fields took 553 instead of 447 us).  check != nullptr: the
+// location's counters -- nothing is written where a particle lies outside, a weight is not
+// finite or a cell is too full, so the launch may precede the host's look at them.
 __global__ void k_cell_sums(int64_t ncells, const uint32_t *__restrict__ off,
                             const uint32_t *__restrict__ idx, int nf,
                             const double *__restrict__ w, int64_t n,
                             const double *__restrict__ vc, double vc_uniform, double inv_pow2,
-                            double *__restrict__ out) {
+                            double *__restrict__ out, const unsigned long long *__restrict__ check) {
+    if (check && (check[0] | check[1] || check[2] > (unsigned long long)kSegMax)) return;
     uint32_t s[kSegMax];
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncells;
          c += (int64_t)gridDim.x * blockDim.x) {
@@ -457,9 +480,10 @@ cg_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint3
     int64_t nb = (n + kScanChunk - 1) / kScanChunk;
     CGK_LAUNCH("scan_reduce", (double)n * 4, st,
                k_scan_reduce<<<(unsigned)nb, kThreads, 0, st>>>(in, n, tmp));
-    CGK_LAUNCH("scan_top", (double)nb * 8, st, k_scan_top<<<1, kThreads, 0, st>>>(tmp, nb));
+    const bool raw = nb <= kScanInline;
+    if (!raw) CGK_LAUNCH("scan_top", (double)nb * 8, st, k_scan_top<<<1, kThreads, 0, st>>>(tmp, nb));
     CGK_LAUNCH("scan_down", (double)n * 8, st,
-               k_scan_down<<<(unsigned)nb, kThreads, 0, st>>>(in, out, n, tmp));
+               k_scan_down<<<(unsigned)nb, kThreads, 0, st>>>(in, out, n, tmp, raw));
     CGK_CUDA(cudaGetLastError());
     return CG_OK;
 }
@@ -472,12 +496,14 @@ cg_status tet_locate_launch(cg_mesh *m, int64_t n, const double *pos, int nf, co
 // The point location and its counters (outside particles, non-finite weights, the most
 // particles in one cell), copied to the mesh's pinned readback buffer; nothing is waited
 // for (locate_read takes the counters once the stream has synchronised).
+// bad_zeroed: the counters' place where the caller has one, cleared already.
 static cg_status locate_launch(cg_mesh *m, int64_t n, const double *pos, int nf, const double *w,
-                               int32_t *cell_out, uint32_t *counts, uint32_t *ranks, cudaStream_t st) {
+                               int32_t *cell_out, uint32_t *counts, uint32_t *ranks, cudaStream_t st,
+                               unsigned long long *bad_zeroed = nullptr) {
     CGK_TRY(m->ws_small.ensure(4096));
     CGK_TRY(m->h_small.ensure(4096));
-    unsigned long long *bad = m->ws_small.as<unsigned long long>();
-    CGK_CUDA(cudaMemsetAsync(bad, 0, 3 * sizeof(unsigned long long), st));
+    unsigned long long *bad = bad_zeroed ? bad_zeroed : m->ws_small.as<unsigned long long>();
+    if (!bad_zeroed) CGK_CUDA(cudaMemsetAsync(bad, 0, 3 * sizeof(unsigned long long), st));
     if (n > 0) {
         if (m->kind == MESH_STRUCTURED) {
             double hi[3];
@@ -541,6 +567,9 @@ struct DepositPlan {
     size_t s_cell, s_cnt;
     int32_t *cell;
     uint32_t *counts, *ranks;
+    const unsigned long long *bad;   // the location's counters on the device
+    uint32_t *off, *idx;             // the counting sort's offsets and ids (deposit_sort)
+    cg_status sorted;                // what deposit_sort returned
 };
 
 // Phase 1 of a deposition: the workspace, the cleared per-cell counters and the point
@@ -564,29 +593,66 @@ static cg_status deposit_begin(cg_mesh *m, int64_t n, const double *pos, int nf,
     // (ncells + 1 counters, the last one staying 0 for the exclusive scan)
     // and keeps each particle's arrival rank at its cell's counter
     const bool ordered = mode == CG_DEPOSIT_ORDERED;
+    // (the location's counters sit in front of the per-cell ones: one clear for both)
+    const size_t s_bad = 256;
     const size_t s_cell = align_up((size_t)(n > 0 ? n : 1) * 4);
     const size_t s_cnt = align_up((size_t)(ncells + 1) * 4);
-    CGK_TRY(m->ws_locate.ensure(s_cell + (ordered ? s_cnt + s_cell : 0)));
+    CGK_TRY(m->ws_locate.ensure(s_cell + s_bad + (ordered ? s_cnt + s_cell : 0)));
     int32_t *cell = m->ws_locate.as<int32_t>();
-    uint32_t *counts = ordered ? (uint32_t *)(m->ws_locate.as<char>() + s_cell) : nullptr;
-    uint32_t *ranks = ordered ? (uint32_t *)(m->ws_locate.as<char>() + s_cell + s_cnt) : nullptr;
-    if (counts) CGK_CUDA(cudaMemsetAsync(counts, 0, (size_t)(ncells + 1) * 4, st));
-    dp = DepositPlan{ncells, mode, vc, vcu, inv_pow2, ordered, s_cell, s_cnt, cell, counts, ranks};
-    return locate_launch(m, n, pos, nf, w, cell, counts, ranks, st);
+    unsigned long long *bad = (unsigned long long *)(m->ws_locate.as<char>() + s_cell);
+    uint32_t *counts = ordered ? (uint32_t *)(m->ws_locate.as<char>() + s_cell + s_bad) : nullptr;
+    uint32_t *ranks = ordered ? (uint32_t *)(m->ws_locate.as<char>() + s_cell + s_bad + s_cnt) : nullptr;
+    CGK_CUDA(cudaMemsetAsync(bad, 0, s_bad + (ordered ? (size_t)(ncells + 1) * 4 : 0), st));
+    dp = DepositPlan{ncells, mode, vc, vcu, inv_pow2, ordered, s_cell, s_cnt, cell, counts, ranks, bad,
+                     nullptr, nullptr, CG_OK};
+    return locate_launch(m, n, pos, nf, w, cell, counts, ranks, st, bad);
+}
+
+// The counting sort by cell of the ordered sums: offsets = exclusive scan of the counts,
+// then a scatter of the ids into the segments.  It writes workspace only, so it runs
+// before the host has seen the location's counters; a workspace that cannot grow is
+// reported (dp.sorted) after them.
+static void deposit_sort(cg_mesh *m, int64_t n, cudaStream_t st, DepositPlan &dp) {
+    if (!dp.ordered) return;
+    const size_t s_off = dp.s_cnt, s_idx = align_up((size_t)(n > 0 ? n : 1) * 4);
+    const size_t s_tmp = align_up(scan_tmp_words(dp.ncells + 1) * 4);
+    dp.sorted = m->ws_sort.ensure(s_off + s_idx + s_tmp);
+    if (dp.sorted != CG_OK) return;
+    char *sb = m->ws_sort.as<char>();
+    dp.off = (uint32_t *)sb;
+    dp.idx = (uint32_t *)(sb + s_off);
+    dp.sorted = exclusive_scan_u32(dp.counts, dp.off, dp.ncells + 1, (uint32_t *)(sb + s_off + s_idx), st);
+    if (dp.sorted == CG_OK && n > 0) {
+        CGK_LAUNCH("scatter_cells", (double)n * 16, st,
+                   k_scatter_cells<<<grid_for(n), kThreads, 0, st>>>(n, dp.cell, dp.off, dp.ranks, dp.idx));
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) dp.sorted = cuda_fail(e, "scatter", __FILE__, __LINE__);
+    }
+}
+
+// The ordered sums from the counting sort; checked: guarded on the device by the
+// location's counters.
+static cg_status deposit_sums(int64_t n, int nf, const double *w, double *out, cudaStream_t st,
+                              const DepositPlan &dp, bool checked) {
+    CGK_LAUNCH("cell_sums", (double)n * (4 + 8 * nf) + (double)dp.ncells * (4 + 8 * nf), st,
+               k_cell_sums<<<grid_for(dp.ncells), kThreads, 0, st>>>(dp.ncells, dp.off, dp.idx, nf, w, n, dp.vc, dp.vcu,
+                                                                  dp.inv_pow2, out, checked ? dp.bad : nullptr));
+    CGK_CUDA(cudaGetLastError());
+    return CG_OK;
 }
 
 // Phase 2, once the stream has synchronised after phase 1: the location's counters are
 // checked (CG_EINVAL for non-finite weights, CG_EDOMAIN for particles outside the mesh,
-// before anything is written to out), then the per-cell sums run.
+// before anything is written to out), then the per-cell sums run (summed: they have run,
+// guarded on the device by the same counters).
 static cg_status deposit_end(cg_mesh *m, int64_t n, int nf, const double *w, double *out,
-                             cg_report *rep, cudaStream_t st, const DepositPlan &dp) {
+                             cg_report *rep, cudaStream_t st, const DepositPlan &dp, bool summed) {
     const int64_t ncells = dp.ncells;
     const double *vc = dp.vc;
     const double vcu = dp.vcu, inv_pow2 = dp.inv_pow2;
     const bool ordered = dp.ordered;
-    const size_t s_cnt = dp.s_cnt;
     int32_t *cell = dp.cell;
-    uint32_t *counts = dp.counts, *ranks = dp.ranks;
+    uint32_t *counts = dp.counts;
     int64_t n_out = 0, n_bad = 0;
     uint32_t max_count = 0;
     locate_read(m, &n_out, &n_bad, counts ? &max_count : nullptr);
@@ -596,25 +662,8 @@ static cg_status deposit_end(cg_mesh *m, int64_t n, int nf, const double *w, dou
         return fail(CG_EDOMAIN, "cg_deposit: %lld particles outside the mesh", (long long)n_out);
 
     if (ordered && max_count <= (uint32_t)kSegMax) {
-        // counting sort by cell: offsets = exclusive scan of the counts, a scatter into the
-        // segments, then per cell the segment's ids in ascending order and the ordered sum
-        const size_t s_off = s_cnt;
-        const size_t s_idx = align_up((size_t)(n > 0 ? n : 1) * 4);
-        const size_t s_tmp = align_up(scan_tmp_words(ncells + 1) * 4);
-        CGK_TRY(m->ws_sort.ensure(s_off + s_idx + s_tmp));
-        char *sb = m->ws_sort.as<char>();
-        uint32_t *off = (uint32_t *)sb, *idx = (uint32_t *)(sb + s_off);
-        uint32_t *tmp = (uint32_t *)(sb + s_off + s_idx);
-        CGK_TRY(exclusive_scan_u32(counts, off, ncells + 1, tmp, st));
-        if (n > 0) {
-            CGK_LAUNCH("scatter_cells", (double)n * 16, st,
-                       k_scatter_cells<<<grid_for(n), kThreads, 0, st>>>(n, cell, off, ranks, idx));
-            CGK_CUDA(cudaGetLastError());
-        }
-        CGK_LAUNCH("cell_sums", (double)n * (4 + 8 * nf) + (double)ncells * (4 + 8 * nf), st,
-                   k_cell_sums<<<grid_for(ncells), kThreads, 0, st>>>(ncells, off, idx, nf, w, n,
-                                                                      vc, vcu, inv_pow2, out));
-        CGK_CUDA(cudaGetLastError());
+        CGK_TRY(dp.sorted);
+        if (!summed) CGK_TRY(deposit_sums(n, nf, w, out, st, dp, false));
         if (rep)
             for (int f = 0; f < nf && f < CG_REPORT_MAX_FIELDS; ++f) rep->fixed_point_bits[f] = 0;
     } else if (ordered) {
@@ -710,23 +759,36 @@ static cg_status deposit_end(cg_mesh *m, int64_t n, int nf, const double *w, dou
 
 cg_status deposit_run(cg_mesh *m, int64_t n, const double *pos, int nf, const double *w,
                       double *out, const cg_params *p, cg_report *rep, cudaStream_t st) {
-    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
-    auto drop = [&]() {
-        for (auto &e : ev)
-            if (e) cudaEventDestroy(e);
-    };
+    cudaEvent_t *ev = m->dep_ev;   // phase times, kept with the mesh
     if (rep) {
-        for (auto &e : ev) CGK_CUDA(cudaEventCreate(&e));
+        for (int i = 0; i < 3; ++i)
+            if (!ev[i]) CGK_CUDA(cudaEventCreate(&ev[i]));
         CGK_CUDA(cudaEventRecord(ev[0], st));
     }
     DepositPlan dp;
     cg_status s = deposit_begin(m, n, pos, nf, w, p, st, dp);
+    if (s == CG_OK && rep) cudaEventRecord(ev[1], st);
+    // the ordered sums are launched behind the location, guarded on the device by its
+    // counters, and the host waits once for all of it
+    bool summed = false;
+    if (s == CG_OK && dp.ordered) {
+        deposit_sort(m, n, st, dp);
+        if (dp.sorted == CG_OK) {
+            s = deposit_sums(n, nf, w, out, st, dp, true);
+            summed = s == CG_OK;
+            if (summed && rep) cudaEventRecord(ev[2], st);
+        }
+    }
     if (s == CG_OK && cudaStreamSynchronize(st) != cudaSuccess)
         s = cuda_fail(cudaGetLastError(), "deposition", __FILE__, __LINE__);
-    if (s == CG_OK && rep) cudaEventRecord(ev[1], st);
-    if (s == CG_OK) s = deposit_end(m, n, nf, w, out, rep, st, dp);
+    if (s == CG_OK) {
+        uint32_t most = 0;
+        locate_read(m, nullptr, nullptr, &most);
+        summed = summed && most <= (uint32_t)kSegMax;
+        s = deposit_end(m, n, nf, w, out, rep, st, dp, summed);
+    }
     if (s == CG_OK && rep) {
-        cudaEventRecord(ev[2], st);
+        if (!summed) cudaEventRecord(ev[2], st);
         cudaEventSynchronize(ev[2]);
         float a = 0, b = 0;
         cudaEventElapsedTime(&a, ev[0], ev[1]);
@@ -734,7 +796,6 @@ cg_status deposit_run(cg_mesh *m, int64_t n, const double *pos, int nf, const do
         rep->ms_locate = a;
         rep->ms_deposit = b;
     }
-    drop();
     return s;
 }
 
@@ -794,6 +855,8 @@ cg_status deposit_many(int nsnap, cg_mesh *const *meshes, const int64_t *n, cons
     if (s == CG_OK) s = fork();
     for (int q = 0; q < nsnap && s == CG_OK; ++q)
         s = deposit_begin(meshes[q], n[q], pos[q], nf, w[q], p, m0->aux_streams[q % na], dps[q]);
+    for (int q = 0; q < nsnap && s == CG_OK; ++q)
+        deposit_sort(meshes[q], n[q], m0->aux_streams[q % na], dps[q]);
     if (s == CG_OK) s = join();
     if (s == CG_OK && cudaStreamSynchronize(st) != cudaSuccess)
         s = cuda_fail(cudaGetLastError(), "deposition", __FILE__, __LINE__);
@@ -809,7 +872,7 @@ cg_status deposit_many(int nsnap, cg_mesh *const *meshes, const int64_t *n, cons
     if (rep) rep->n_out_of_domain = n_out_total;
     if (s == CG_OK) s = fork();
     for (int q = 0; q < nsnap && s == CG_OK; ++q)
-        s = deposit_end(meshes[q], n[q], nf, w[q], out[q], nullptr, m0->aux_streams[q % na], dps[q]);
+        s = deposit_end(meshes[q], n[q], nf, w[q], out[q], nullptr, m0->aux_streams[q % na], dps[q], false);
     if (s == CG_OK) s = join();
     if (s == CG_OK && rep) {
         cudaEventRecord(ev[2], st);

@@ -181,6 +181,8 @@ struct cg_mesh {
     std::vector<cgk::PredPlan> preds;         // shared expansions per (scheme, steps, c)
     std::vector<std::pair<double, double>> spectrum;   // unstructured: lower end of the
                                                        // Chebyshev interval per dte
+    cudaEvent_t dep_ev[3] = {nullptr, nullptr, nullptr};   // a deposition's phase times
+    cudaEvent_t dif_ev[2] = {nullptr, nullptr};            // a diffusion's
     cudaStream_t capture_stream = nullptr;    // private stream used only for capture
     std::vector<cudaStream_t> aux_streams;    // batched depositions: snapshots in parallel
 };
@@ -273,9 +275,9 @@ cg_status diffuse_batched_run(int nsnap, cg_mesh *const *meshes, int nf, double 
 cg_status diffuse_tet_run(cg_mesh *m, int nf, double *cells, const cg_params *p,
                           cg_report *rep, cudaStream_t st);
 
-// sum_k V_c,k u_f,k for each field (FP64, deterministic order), written to host.
-cg_status field_mass(cg_mesh *m, int nf, const double *cells, double *mass_host,
-                     cudaStream_t st);
+// sum_k V_c,k u_f,k for each field (FP64, deterministic order).
+cg_status field_mass_keep(cg_mesh *m, int nf, const double *cells, int slot, cudaStream_t st);
+cg_status field_mass_read(cg_mesh *m, int nf, double *slot0, double *slot1, cudaStream_t st);
 cg_status field_mass_many(int nmesh, cg_mesh *const *ms, int nf, const double *const *cells,
                           double *mass_host, cudaStream_t st);
 

@@ -4651,7 +4651,9 @@ cg_status solid_velocity_run(int64_t n, int ncomp, const double *eps, const doub
 
 // Launches the mass reduction of one mesh's fields and the copy of its result into the
 // mesh's pinned readback buffer (complete once the stream has synchronised).
-static cg_status field_mass_launch(cg_mesh *m, int nf, const double *cells, cudaStream_t st) {
+// keep: device doubles that take the masses instead of the pinned readback buffer.
+static cg_status field_mass_launch(cg_mesh *m, int nf, const double *cells, cudaStream_t st,
+                                   double *keep = nullptr) {
     int n = (int)m->ncells;
     int G = stencil_grid(n);
     size_t need = align_up((size_t)nf * G * 8) + 64 * 8 + 64 * 4;
@@ -4660,19 +4662,35 @@ static cg_status field_mass_launch(cg_mesh *m, int nf, const double *cells, cuda
     double *partials = (double *)base;
     double *out = (double *)(base + align_up((size_t)nf * G * 8));
     unsigned int *tickets = (unsigned int *)(out + 64);
+    if (keep) out = keep;
     CGK_CUDA(cudaMemsetAsync(tickets, 0, 64 * 4, st));
     const double *vc = m->kind != MESH_STRUCTURED ? m->tet.vc : nullptr;
     double vcu = (m->dx * m->dx) * m->dx;
     CGK_LAUNCH("mass", (double)n * nf * 8, st,
                k_mass<<<dim3(G, nf), kThreads, 0, st>>>(n, cells, vc, vcu, partials, tickets, out));
     CGK_CUDA(cudaGetLastError());
+    if (keep) return CG_OK;
     CGK_TRY(m->h_small.ensure(4096));
     CGK_CUDA(cudaMemcpyAsync(m->h_small.as<char>() + 2048, out, nf * 8, cudaMemcpyDeviceToHost, st));
     return CG_OK;
 }
 
-cg_status field_mass(cg_mesh *m, int nf, const double *cells, double *mass_host, cudaStream_t st) {
-    return field_mass_many(1, &m, nf, &cells, mass_host, st);
+// Without waiting or copying: the masses stay in device memory (the mesh's location
+// workspace, which no diffusion touches), slot 0 or 1; field_mass_read waits and copies.
+cg_status field_mass_keep(cg_mesh *m, int nf, const double *cells, int slot, cudaStream_t st) {
+    CGK_TRY(m->ws_locate.ensure(4096));
+    return field_mass_launch(m, nf, cells, st, m->ws_locate.as<double>() + 64 * slot);
+}
+cg_status field_mass_read(cg_mesh *m, int nf, double *slot0, double *slot1, cudaStream_t st) {
+    CGK_TRY(m->h_small.ensure(4096));
+    double *h = (double *)(m->h_small.as<char>() + 2048);
+    CGK_CUDA(cudaMemcpyAsync(h, m->ws_locate.as<double>(), 128 * 8, cudaMemcpyDeviceToHost, st));
+    CGK_CUDA(cudaStreamSynchronize(st));
+    for (int f = 0; f < nf; ++f) {
+        slot0[f] = h[f];
+        if (slot1) slot1[f] = h[64 + f];
+    }
+    return CG_OK;
 }
 
 // The masses of several meshes' fields (distinct meshes: each uses its own buffers): every
