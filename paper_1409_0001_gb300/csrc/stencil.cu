@@ -2037,6 +2037,347 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     }
 }
 
+// ---------------------------------------------------------------- merged step pass
+// With the shared expansion a step ends with x = (u_s + e_s) + d (e_s its increment, d its
+// round's correction; u_{s+1} = x) and the next one starts from u_{s+1} + e_{s+1}: two
+// passes that read the same cells one after the other.  Here they are one: per cell and
+// neighbour the pass forms x and takes e' = e_{s+1}, and from the two neighbour sums it has
+// both the finished step's residual b - A x (reduced) and the next step's first one,
+//   r' = b' - A (x + e') = theta ce L x - e' + ce L e',
+// b' = x (implicit Euler, theta = 1) or x + ce L x (Crank-Nicolson, theta = 2), all in
+// double-float arithmetic (e' is exact in FP32).  36 B per cell instead of 60 for the two
+// (x + e' is never stored), one launch instead of two; bound by instruction issue and
+// latency like k_refine_df2.  Per step (one merged pass for two): 128^3 53.5 -> 32.9 us,
+// 256 x 128 x 128 x 4 fields 276 -> 193 us, 512 x 256 x 256 520 -> 352 us (3.4 TB/s), and in the scalar
+// form 97 x 61 x 45 x 3 fields 47 -> 37 us.  kEnd: the last step's pass, without a next step.
+// the value pair of the scalar form: += is the double-float cascade on both parts
+struct DFe {
+    DF x, e;
+};
+__device__ __forceinline__ DFe &operator+=(DFe &a, DFe b) {
+    a.x += b.x;
+    a.e += b.e;
+    return a;
+}
+struct DFeRaw {
+    DF u;
+    float e, d, en;
+};
+
+template <bool kEnd>
+__global__ void __launch_bounds__(kThreads) k_refine_mid(Geo g, int zlen, int nzc, CoefDF cf, int scheme,
+                                                         const DF *__restrict__ u_all,
+                                                         const float *__restrict__ e_all,
+                                                         const float *__restrict__ d_all,
+                                                         const float *__restrict__ en_all, const DF *b_all,
+                                                         DF *__restrict__ xout_all, DF *bout_all,
+                                                         float *__restrict__ r_all, float *__restrict__ y1_all,
+                                                         float gamma, double *__restrict__ partials_all,
+                                                         RefScal *__restrict__ sc, RefScal *__restrict__ sc_next) {
+    chain_wait();
+    chain_release();
+    const BlockPos bp = block_pos(g, zlen, nzc);
+    const size_t off = (size_t)bp.f * g.n;
+    const DF *u = u_all + off, *b = b_all + off;
+    const float *e = e_all + off, *d = d_all + off, *en = kEnd ? nullptr : en_all + off;
+    DF *xout = xout_all + off;
+    float *r = r_all + off, *y1 = y1_all + off;
+    float rr = 0.0f, bb = 0.0f;
+    sweep25_lf<DFe>(
+        g, blockIdx.x, blockIdx.y, bp.z0, bp.z1,
+        [&](int k) { return DFeRaw{u[k], e[k], d[k], kEnd ? 0.0f : en[k]}; },
+        [](DFeRaw v) { return DFe{df_add_f(df_add_f(v.u, v.e), v.d), DF{v.en, 0.0f}}; },
+        [&](int k) { return b[k]; },
+        [&](int k, DFe v, DFe s, int nn, DF bk) {
+            xout[k] = v.x;
+            const DF lx = df_lap(s.x, v.x, (float)nn);
+            const float rf = df_f(df_res(bk, v.x, cf.ce, lx));
+            rr = fmaf(rf, rf, rr);
+            if constexpr (!kEnd) {
+                const DF le = df_lap(s.e, v.e, (float)nn);
+                DF bn = v.x, m = lx;
+                if (scheme == 1) {
+                    bn = v.x + df_mul(cf.ce, lx);
+                    bout_all[off + k] = bn;
+                    m = DF{2.0f * lx.hi, 2.0f * lx.lo};
+                }
+                const float bf = df_f(bn);
+                bb = fmaf(bf, bf, bb);
+                const DF t = df_two_sum(m.hi, le.hi);
+                const DF q = df_mul_un(cf.ce, DF{t.hi, (m.lo + le.lo) + t.lo});
+                const DF w = df_two_sum(-v.e.hi, q.hi);
+                const float rn = w.hi + (q.lo + w.lo);
+                r[k] = rn;
+                y1[k] = gamma * rn;
+            }
+        });
+    double vals[2] = {block_sum_f(rr), kEnd ? 0.0 : block_sum_f(bb)};
+    double *partials = partials_all + (size_t)bp.f * 2 * bp.nb;
+    if (arrive(partials, kEnd ? 1 : 2, vals, bp.bid, bp.nb, &sc[bp.f].ticket)) {
+        double RR = finish_sum(partials, 0, bp.nb);
+        double BB = kEnd ? 0.0 : finish_sum(partials, 1, bp.nb);
+        if (is_thread0()) {
+            sc[bp.f].rr = RR;
+            if (!kEnd) sc_next[bp.f].bb = BB;
+            sc[bp.f].ticket = 0;
+        }
+    }
+}
+
+// The same pass with two x-cells per thread in packed arithmetic, implicit Euler, built as
+// k_refine_df2: the planes ahead come through a per-thread cp.async ring, the march is
+// unrolled by its three slots.  The finished step's b is u_s, which the x of a cell is
+// formed from: it stays in registers from when its plane arrives until it is the centre.
+template <bool kEnd>
+__global__ void __launch_bounds__(kThreads, 3) k_refine_mid2(Geo g, int zlen, int nzc, CoefDF cf,
+                                                          const DF *__restrict__ u_all,
+                                                          const float *__restrict__ e_all,
+                                                          const float *__restrict__ d_all,
+                                                          const float *__restrict__ en_all,
+                                                          DF *__restrict__ xout_all, float *__restrict__ r_all,
+                                                          float *__restrict__ y1_all, float gamma,
+                                                          double *__restrict__ partials_all,
+                                                          RefScal *__restrict__ sc, RefScal *__restrict__ sc_next) {
+    chain_wait();
+    chain_release();
+    using PR = Pair<float>;
+    constexpr int RS = kRefRing;
+    const int f = blockIdx.z / nzc;
+    const int zc = blockIdx.z - f * nzc;
+    const int z0 = zc * zlen, z1 = min(g.nz, z0 + zlen);
+    const int bid = (zc * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const int nb = gridDim.x * gridDim.y * nzc;
+    const size_t off = (size_t)f * g.n;
+    const float4 *U = reinterpret_cast<const float4 *>(u_all + off);   // cell pairs
+    const float *E = e_all + off, *D = d_all + off, *F = kEnd ? nullptr : en_all + off;
+    float4 *XO = reinterpret_cast<float4 *>(xout_all + off);
+    float *r = r_all + off, *y1 = y1_all + off;
+    const DFc2 ce2 = dfc2(cf.ce);
+    __shared__ float4 pl[TY + 2][TX];   // the plane's x with its y halo rows
+    __shared__ float2 pf[kEnd ? 1 : TY + 2][TX];   // and its e'
+    __shared__ float4 rU[RS][kThreads];    // own pair (plane q + 2): u, e, d, e'
+    __shared__ float2 rE[RS][kThreads], rD[RS][kThreads], rF[kEnd ? 1 : RS][kEnd ? 1 : kThreads];
+    __shared__ float4 rhU[RS][2][TX];      // halo rows (plane q + 1)
+    __shared__ float2 rhE[RS][2][TX], rhD[RS][2][TX], rhF[kEnd ? 1 : RS][2][TX];
+    __shared__ float4 rcU[RS][TY][2];      // halo columns (plane q + 1): the pairs holding x - 1, x + 2
+    __shared__ float rcE[RS][TY][2], rcD[RS][TY][2], rcF[kEnd ? 1 : RS][TY][2];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int x0 = blockIdx.x * (2 * TX);
+    const int x = x0 + 2 * tx, y = blockIdx.y * TY + ty;
+    const bool own = (x < g.nx) && (y < g.ny);
+    const bool rowlo = (ty == 0) && (y > 0) && (x < g.nx);
+    const bool rowhi = (ty == TY - 1) && (y + 1 < g.ny) && (x < g.nx);
+    const bool row = rowlo || rowhi;
+    const bool px = (g.per & 1) != 0;   // a periodic x axis (the only one this kernel takes)
+    const bool xl = (tx == 0) && (x > 0 || px) && (y < g.ny);
+    const int xlast = min(g.nx, x0 + 2 * TX) - 2;
+    const bool xr = (x == xlast) && (x + 2 < g.nx || px) && (y < g.ny);
+    const int dxl = (px && x == 0) ? g.nx - 1 : -1;
+    const int dxr = (px && x + 2 >= g.nx) ? 2 - g.nx : 2;
+    const int dro = rowlo ? -g.nx : g.nx;
+    const int nyb = (y > 0) + (y + 1 < g.ny);
+    const int n0 = nyb + ((x > 0 || px) ? 1 : 0) + 1, n1 = nyb + 1 + ((x + 2 < g.nx || px) ? 1 : 0);
+    const float2 nn_mid = make_float2((float)(n0 + 2), (float)(n1 + 2));
+    const int kxy = y * g.nx + x;
+    auto value = [](float4 u, float2 e, float2 d) { return pair_add(pair_add(u, e), d); };
+    auto value1 = [](float4 p, bool odd, float e, float d) {   // one cell of a pair
+        return df_add_f(df_add_f(odd ? DF{p.y, p.w} : DF{p.x, p.z}, e), d);
+    };
+    const float2 z2 = make_float2(0.f, 0.f);
+    const int tid = ty * TX + tx, hrow = ty == 0 ? 0 : 1;
+    auto stage = [&](int q, int sl) {
+        if (q + 1 < z1) {
+            const int kn = kxy + (q + 1) * g.nxy;
+            if (own && q + 2 < g.nz) {
+                const int k2 = kn + g.nxy;
+                cp_async16(&rU[sl][tid], U + (k2 >> 1));
+                cp_async8(&rE[sl][tid], E + k2);
+                cp_async8(&rD[sl][tid], D + k2);
+                if constexpr (!kEnd) cp_async8(&rF[sl][tid], F + k2);
+            }
+            if (row) {
+                const int kh = kn + dro;
+                cp_async16(&rhU[sl][hrow][tx], U + (kh >> 1));
+                cp_async8(&rhE[sl][hrow][tx], E + kh);
+                cp_async8(&rhD[sl][hrow][tx], D + kh);
+                if constexpr (!kEnd) cp_async8(&rhF[sl][hrow][tx], F + kh);
+            }
+            if (xl) {
+                const int kl = kn + dxl;
+                cp_async16(&rcU[sl][ty][0], U + (kl >> 1));
+                cp_async4(&rcE[sl][ty][0], E + kl);
+                cp_async4(&rcD[sl][ty][0], D + kl);
+                if constexpr (!kEnd) cp_async4(&rcF[sl][ty][0], F + kl);
+            }
+            if (xr) {
+                const int kr = kn + dxr;
+                cp_async16(&rcU[sl][ty][1], U + (kr >> 1));
+                cp_async4(&rcE[sl][ty][1], E + kr);
+                cp_async4(&rcD[sl][ty][1], D + kr);
+                if constexpr (!kEnd) cp_async4(&rcF[sl][ty][1], F + kr);
+            }
+        }
+        cp_async_commit();
+    };
+    // register state: the plane queues (rotating by renaming), u of planes z and z + 1, the
+    // halo values of plane z
+    float4 qa = f4z(), qb = f4z(), qc = f4z(), bc = f4z(), bn = f4z(), hv = f4z();
+    float2 fa = z2, fb = z2, fc = z2, hf = z2;
+    DF hl{0.f, 0.f}, hr{0.f, 0.f};
+    float hfl = 0.f, hfr = 0.f;
+    float rr = 0.0f, bb = 0.0f;
+    if (z0 < z1) {
+        const int k0 = kxy + z0 * g.nxy;
+        auto at = [&](int k) { return value(U[k >> 1], PR::load(E, k), PR::load(D, k)); };
+        auto at1 = [&](int k) { return value1(U[k >> 1], k & 1, E[k], D[k]); };
+        if (own) {
+            if (z0 > 0) {
+                qa = at(k0 - g.nxy);
+                if constexpr (!kEnd) fa = PR::load(F, k0 - g.nxy);
+            }
+            qb = at(k0);
+            bc = U[k0 >> 1];
+            if constexpr (!kEnd) fb = PR::load(F, k0);
+            if (z0 + 1 < g.nz) {
+                qc = at(k0 + g.nxy);
+                bn = U[(k0 + g.nxy) >> 1];
+                if constexpr (!kEnd) fc = PR::load(F, k0 + g.nxy);
+            }
+        }
+        if (row) {
+            hv = at(k0 + dro);
+            if constexpr (!kEnd) hf = PR::load(F, k0 + dro);
+        }
+        if (xl) {
+            hl = at1(k0 + dxl);
+            if constexpr (!kEnd) hfl = F[k0 + dxl];
+        }
+        if (xr) {
+            hr = at1(k0 + dxr);
+            if constexpr (!kEnd) hfr = F[k0 + dxr];
+        }
+    }
+    stage(z0, 0);
+    stage(z0 + 1, 1);
+    // one plane: planes z - 1, z, z + 1 of x (vdn, vc, vup) and e' (gdn, gc, gup);
+    // j = (z - z0) % 3.  After the stencils vdn and gdn take plane z + 2.
+    auto step = [&](const int z, const int j, float4 &vdn, const float4 &vc, const float4 &vup, float2 &gdn,
+                    const float2 &gc, const float2 &gup) {
+        stage(z + RS - 1, (j + RS - 1) % RS);
+        const int kz = kxy + z * g.nxy;
+        pl[ty + 1][tx] = vc;
+        if constexpr (!kEnd) pf[ty + 1][tx] = gc;
+        if (ty == 0 || ty == TY - 1) {   // (zero where the row lies outside the mesh)
+            const int hr_ = ty == 0 ? 0 : TY + 1;
+            pl[hr_][tx] = hv;
+            if constexpr (!kEnd) pf[hr_][tx] = hf;
+        }
+        DF left{__shfl_up_sync(0xffffffffu, vc.y, 1), __shfl_up_sync(0xffffffffu, vc.w, 1)};
+        DF right{__shfl_down_sync(0xffffffffu, vc.x, 1), __shfl_down_sync(0xffffffffu, vc.z, 1)};
+        float fl = 0.f, fr = 0.f;
+        if constexpr (!kEnd) {
+            fl = __shfl_up_sync(0xffffffffu, gc.y, 1);
+            fr = __shfl_down_sync(0xffffffffu, gc.x, 1);
+        }
+        if (tx == 0) {
+            left = hl;
+            fl = hfl;
+        }
+        if (x == xlast) {
+            right = hr;
+            fr = hfr;
+        }
+        __syncthreads();
+        if (own) {
+            const DF2 V = df2_of(vc);
+            float2 nn = nn_mid;
+            if (z == 0 || z + 1 == g.nz) {   // a z wall: fewer neighbours
+                const int nz_ = (z > 0) + (z + 1 < g.nz);
+                nn = make_float2((float)(n0 + nz_), (float)(n1 + nz_));
+            }
+            const float2 nnn = make_float2(-nn.x, -nn.y);
+            DF2 S{make_float2(left.hi, vc.x), make_float2(left.lo, vc.z)};
+            df2_acc(S, DF2{make_float2(vc.y, right.hi), make_float2(vc.w, right.lo)});
+            df2_acc(S, df2_of(pl[ty][tx]));
+            df2_acc(S, df2_of(pl[ty + 2][tx]));
+            df2_acc(S, df2_of(vdn));
+            df2_acc(S, df2_of(vup));
+            const DF2 L = df2_lap(S, V, nn, nnn);
+            XO[kz >> 1] = vc;
+            const float2 rf = df2_f(df2_res(df2_of(bc), V, ce2, L));
+            rr = fmaf(rf.x, rf.x, fmaf(rf.y, rf.y, rr));
+            if constexpr (!kEnd) {
+                // the neighbour sum of e' as a pair: the TwoSum cascade's errors
+                DF2 G{make_float2(fl, gc.x), z2};
+                auto acc = [&](float2 v) {
+                    const DF2 t = df2_two_sum(G.hi, v);
+                    G.hi = t.hi;
+                    G.lo = add2(G.lo, t.lo);
+                };
+                acc(make_float2(gc.y, fr));
+                acc(pf[ty][tx]);
+                acc(pf[ty + 2][tx]);
+                acc(gdn);
+                acc(gup);
+                const DF2 LE = df2_lap(G, DF2{gc, z2}, nn, nnn);
+                const DF2 t = df2_two_sum(L.hi, LE.hi);
+                const DF2n q = df2_mul_un(ce2, DF2{t.hi, add2(add2(L.lo, LE.lo), t.lo)});
+                const DF2 w = df2_two_sum(q.hi, make_float2(-gc.x, -gc.y));
+                const float2 rn = add2(w.hi, sub2(w.lo, q.nlo));
+                const float2 fb2 = df2_f(V);
+                bb = fmaf(fb2.x, fb2.x, fmaf(fb2.y, fb2.y, bb));
+                PR::store(r, kz, rn.x, rn.y);
+                const float2 g1 = mul2(make_float2(gamma, gamma), rn);
+                PR::store(y1, kz, g1.x, g1.y);
+            }
+        }
+        __syncthreads();   // the plane buffers are rewritten by the next step
+        cp_async_wait<RS - 1>();
+        if (z + 1 < z1) {
+            if (own) {
+                bc = bn;
+                vdn = f4z();
+                gdn = z2;
+                if (z + 2 < g.nz) {
+                    bn = rU[j][tid];
+                    vdn = value(bn, rE[j][tid], rD[j][tid]);
+                    if constexpr (!kEnd) gdn = rF[j][tid];
+                }
+            }
+            if (row) {
+                hv = value(rhU[j][hrow][tx], rhE[j][hrow][tx], rhD[j][hrow][tx]);
+                if constexpr (!kEnd) hf = rhF[j][hrow][tx];
+            }
+            if (xl) {   // x - 1 is the odd cell of its pair, x + 2 the even one
+                hl = value1(rcU[j][ty][0], true, rcE[j][ty][0], rcD[j][ty][0]);
+                if constexpr (!kEnd) hfl = rcF[j][ty][0];
+            }
+            if (xr) {
+                hr = value1(rcU[j][ty][1], false, rcE[j][ty][1], rcD[j][ty][1]);
+                if constexpr (!kEnd) hfr = rcF[j][ty][1];
+            }
+        }
+    };
+    static_assert(RS == 3, "the march below is unrolled for three ring slots");
+    for (int z = z0; z < z1; z += RS) {
+        step(z, 0, qa, qb, qc, fa, fb, fc);
+        if (z + 1 < z1) step(z + 1, 1, qb, qc, qa, fb, fc, fa);
+        if (z + 2 < z1) step(z + 2, 2, qc, qa, qb, fc, fa, fb);
+    }
+    cp_async_wait<0>();   // no copy outlives the block
+    double vals[2] = {block_sum_f(rr), kEnd ? 0.0 : block_sum_f(bb)};
+    double *partials = partials_all + (size_t)f * 2 * nb;
+    if (arrive(partials, kEnd ? 1 : 2, vals, bid, nb, &sc[f].ticket)) {
+        double RR = finish_sum(partials, 0, nb);
+        double BB = kEnd ? 0.0 : finish_sum(partials, 1, nb);
+        if (is_thread0()) {
+            sc[f].rr = RR;
+            if (!kEnd) sc_next[f].bb = BB;
+            sc[f].ticket = 0;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- grid barrier
 // A barrier over all blocks of a cooperative launch (all blocks co-resident).  The
 // wait is bounded: a block that spins longer than `budget` clock cycles raises err and
@@ -4281,6 +4622,47 @@ void launch_refine_df(const Geo &g, const Sweep &sw, int nf, const CoefDF &cf, i
     }
 }
 
+// Whether the merged pass has a form for the call: the packed form is implicit Euler only.
+inline bool mid_fits(const Geo &g, int scheme) { return scheme == 0 || !df_pairs(g); }
+
+// Its launch geometry: three blocks to an SM, and a block pays about two planes besides its
+// own (the planes either side and its start), so the chunk of at most 16 planes that minimises
+// waves x (planes + 2): longer ones leave SMs idle at the end (3 fields of 128^3 in one wave of
+// 32 planes 81.7 us, in two or more 76).
+inline Sweep mid_sweep(const Geo &g, int nf) {
+    const long long slots = 3LL * num_sms();
+    const int w = df_pairs(g) ? 2 * TX : TX;
+    const long long cols = (long long)((g.nx + w - 1) / w) * ((g.ny + TY - 1) / TY) * nf;
+    int best = 1;
+    long long cost = -1;
+    for (int nzc = 1; nzc <= g.nz; ++nzc) {
+        const int z = (g.nz + nzc - 1) / nzc;
+        if (z > 16) continue;
+        const long long c = (cols * ((g.nz + z - 1) / z) + slots - 1) / slots * (z + 2);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = z;
+        }
+    }
+    return make_sweep_z(g, nf, best);
+}
+
+// One merged pass (en == nullptr: the call's last).
+inline void launch_refine_mid(const Geo &g, const Sweep &sw, const CoefDF &cf, int scheme, const DF *u,
+                              const float *e, const float *d, const float *en, const DF *b, DF *xout, DF *bout,
+                              float *r, float *y1, float gamma, double *partials, RefScal *sc, RefScal *sc_next,
+                              cudaStream_t st) {
+    const dim3 blk(TX, TY);
+    if (df_pairs(g)) {
+        const dim3 grid((g.nx + 2 * TX - 1) / (2 * TX), sw.grid.y, sw.grid.z);
+        launch_chain(en ? k_refine_mid2<false> : k_refine_mid2<true>, grid, blk, st, g, sw.zlen, sw.nzc, cf, u, e, d,
+                     en, xout, r, y1, gamma, partials, sc, sc_next);
+    } else {
+        launch_chain(en ? k_refine_mid<false> : k_refine_mid<true>, sw.grid, blk, st, g, sw.zlen, sw.nzc, cf, scheme,
+                     u, e, d, en, b, xout, bout, r, y1, gamma, partials, sc, sc_next);
+    }
+}
+
 // Brick decomposition for k_cheb_resident: the smallest brick (rows x planes) such that
 // the bricks fit on the SMs one per SM and two padded brick arrays fit in one block's
 // shared memory.  Not available (ok = false) for several fields, nx % 4 != 0, more
@@ -5298,7 +5680,8 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     const double ce = cn ? 0.5 * c : c;
     const double tol2 = p->tol * p->tol;
     const Sweep sw = make_sweep(g, nf);
-    const int G = sw.nb;
+    const Sweep sw_mid = mid_sweep(g, nf);
+    const int G = std::max(sw.nb, sw_mid.nb);
     const dim3 blk(TX, TY);
     const Coef64 cf64 = coef64(ce);
     const Coef32 cf32 = coef32(ce);
@@ -5484,13 +5867,18 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                     XT *u = X0, *f1 = X1, *f2 = X2;
                     TS *y1_start = Ya;
                     int run = -1;   // the current run of the shared expansion
+                    // merged passes between the steps of a run (one inner solve per step)
+                    const bool mid = pred && R == 2 && mid_fits(g, p->scheme);
+                    bool merged_in = false;   // the step was started by a merged pass
                     for (int s2 = 0; s2 < p->nsteps; ++s2) {
                         RefScal *slot = hist + (size_t)s2 * nf;
                         const XT *bp_ = cn ? B : u;
                         TS *y1 = y1_start;
                         // the first step starts with its own pass; later steps were started
                         // by the previous step's last pass
-                        if (s2 == 0 && (!pred || cn))
+                        const bool run_start = pred && run + 1 < (int)pred->start.size() &&
+                                               pred->start[run + 1] == s2;
+                        if ((s2 == 0 || (mid && run_start)) && (!pred || cn))
                             CGK_LAUNCH("refine_df_first", (double)n * nf * (8 + (cn ? 8 : 0) + 2 * sizeof(TS)), cs,
                                        launch_refine_df<TS, 0>(g, sw, nf, cfdf, p->scheme,
                                                                (const DF *)u, (const TS *)nullptr,
@@ -5500,10 +5888,12 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                         XT *xc = u;
                         if constexpr (sizeof(TS) == 4)
                             if (pred) {   // the step's first round
-                                if (run + 1 < (int)pred->start.size() && pred->start[run + 1] == s2)
-                                    launch_pred(*pred, ++run, g, nf, (const DF *)u, PT, PD, vts / 4, cs);
+                                if (run_start) launch_pred(*pred, ++run, g, nf, (const DF *)u, PT, PD, vts / 4, cs);
                                 const float *d0 = PD + (size_t)(s2 - pred->start[run]) * (vts / 4);
-                                if (cn)
+                                // (a merged pass at the end of the step before has left this
+                                // step's first residual, and u + d0 is formed where it is read)
+                                if (merged_in) {
+                                } else if (cn)
                                     CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
                                                launch_refine_df<TS, 1>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
                                                                        (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
@@ -5513,7 +5903,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                launch_refine_df<TS, 4>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
                                                                        (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
                                                                        (float)gamma, partials, slot, slot, cs));
-                                xc = f1;
+                                if (!merged_in) xc = f1;
                             }
                         const int mi = pred ? pred->m[s2] : m_it;   // inner iterations of a round
                         for (int r = pred ? 1 : 0; r < R; ++r) {
@@ -5560,6 +5950,23 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                             // the next step's first Chebyshev iterate goes to Ya: it must not
                             // be the buffer holding this round's correction
                             const bool last = r == R - 1;
+                            if constexpr (sizeof(TS) == 4)
+                                if (last && mid) {
+                                    const int i = s2 - pred->start[run];
+                                    const float *e0 = PD + (size_t)i * (vts / 4);
+                                    merged_in = i + 1 < pred->len[run];
+                                    y1 = (yc == Ya) ? Yb : Ya;
+                                    if (merged_in) y1_start = y1;
+                                    CGK_LAUNCH(merged_in ? "refine_mid" : "refine_mid_end",
+                                               (double)n * nf * ((merged_in ? 36 : 24) + (cn ? 16 : 0)), cs,
+                                               launch_refine_mid(g, sw_mid, cfdf, p->scheme, (const DF *)u, e0,
+                                                                 (const float *)yc,
+                                                                 merged_in ? e0 + vts / 4 : nullptr, (const DF *)bp_,
+                                                                 (DF *)xn, (DF *)B, (float *)R_, (float *)y1,
+                                                                 (float)gamma, partials, slot, slot + nf, cs));
+                                    xc = xn;
+                                    break;
+                                }
                             const bool emit = last && (s2 + 1 < p->nsteps) && (!pred || cn);
                             y1 = (yc == Ya) ? Yb : Ya;
                             if (emit) y1_start = y1;    // where the next step's y1 is
