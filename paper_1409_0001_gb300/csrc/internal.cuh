@@ -102,6 +102,7 @@ struct RoundsEntry {
     int nf, precision, scheme, nsteps;
     double T, tol;
     int rounds;
+    bool predicted;   // with the shared expansion
 };
 
 // The increments of a run of implicit steps as Chebyshev expansions of the run's first

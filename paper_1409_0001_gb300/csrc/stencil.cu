@@ -1643,10 +1643,11 @@ __global__ void k_from_df_pairs(size_t npairs, const float4 *__restrict__ x, dou
 // also reduces ||b||^2 (the first pass of a step whose correction comes from the shared
 // expansion); 5: a step's last refinement pass when nothing follows from its r (no r and
 // y1 written).
-template <class TS, int kMode>
+// TD: the stored type of the correction d (FP32 for the shared expansion's increments).
+template <class TS, int kMode, class TD = TS>
 __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc, CoefDF cf,
                                                         int scheme, const DF *__restrict__ xin_all,
-                                                        const TS *__restrict__ d_all,
+                                                        const TD *__restrict__ d_all,
                                                         const DF *b_all, DF *__restrict__ xout_all,
                                                         DF *bout_all, TS *__restrict__ r_all,
                                                         TS *__restrict__ y1_all, float gamma,
@@ -1679,7 +1680,7 @@ __global__ void __launch_bounds__(kThreads) k_refine_df(Geo g, int zlen, int nzc
                 rr = fmaf(rf, rf, rr);
             });
     } else {
-        const TS *d = d_all + off;
+        const TD *d = d_all + off;
         const DF *b = b_all + off;
         DF *xout = xout_all + off;
         sweep25_lf<DF>(
@@ -1771,10 +1772,10 @@ __device__ __forceinline__ float4 pair_add(float4 xv, float2 dv) { return f4_of(
 // shared footprint cost ~8 ms over the 80 passes of the channel case.)
 constexpr int kRefRing = 3;   // ring slots: two planes in flight beyond the one consumed
 
-template <class TS, int kMode>
+template <class TS, int kMode, class TD = TS>
 __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int nzc, CoefDF cf,
                                                          int scheme, const DF *__restrict__ xin_all,
-                                                         const TS *__restrict__ d_all,
+                                                         const TD *__restrict__ d_all,
                                                          const DF *b_all, DF *__restrict__ xout_all,
                                                          DF *bout_all, TS *__restrict__ r_all,
                                                          TS *__restrict__ y1_all, float gamma,
@@ -1784,6 +1785,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     chain_wait();
     chain_release();
     using PR = Pair<TS>;
+    using PD = Pair<TD>;
     const int f = blockIdx.z / nzc;
     const int zc = blockIdx.z - f * nzc;
     const int z0 = zc * zlen, z1 = min(g.nz, z0 + zlen);
@@ -1792,7 +1794,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     const size_t off = (size_t)f * g.n;
     const float4 *X = reinterpret_cast<const float4 *>(xin_all + off);   // cell pairs
     constexpr bool kPlain = kMode == 0 || kMode == 3;   // the stencil of x itself (no d)
-    const TS *D = kPlain ? nullptr : d_all + off;
+    const TD *D = kPlain ? nullptr : d_all + off;
     const float4 *Bp = reinterpret_cast<const float4 *>(kPlain ? nullptr : b_all + off);
     float4 *XO = reinterpret_cast<float4 *>(xout_all + off);
     float4 *BO = reinterpret_cast<float4 *>(bout_all ? bout_all + off : nullptr);
@@ -1825,7 +1827,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     auto val2 = [&](int k) -> float4 {
         const float4 xv = X[k >> 1];
         if (kPlain) return xv;
-        return pair_add(xv, PR::load(D, k));
+        return pair_add(xv, PD::load(D, k));
     };
     auto val1 = [&](int k) -> DF {
         const float4 pv = X[k >> 1];
@@ -1835,20 +1837,20 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
     };
     // d of a cell pair as stored (FP32: 8 bytes; BF16: 4 bytes); a halo column's d is
     // staged as the aligned pair that holds it (BF16 has no 2-byte asynchronous copy)
-    using DPair = typename std::conditional<sizeof(TS) == 4, float2, __nv_bfloat162>::type;
+    using DPair = typename std::conditional<sizeof(TD) == 4, float2, __nv_bfloat162>::type;
     __shared__ float4 rX[RS][kThreads];    // own pair's x (plane q + 2)
     __shared__ DPair rD[RS][kThreads];     // own pair's d (plane q + 2)
     __shared__ float4 rB[RS][kThreads];    // own pair's b (plane q + 1)
     __shared__ float4 rhX[RS][2][TX];      // halo rows (plane q + 1): y - 1 (ty 0), y + 1 (ty TY-1)
     __shared__ DPair rhD[RS][2][TX];
     __shared__ float4 rcX[RS][TY][2];      // the pairs holding the halo columns (plane q + 1): x - 1, x + 2
-    __shared__ typename std::conditional<sizeof(TS) == 4, float, __nv_bfloat162>::type rcD[RS][TY][2];
-    auto cp_dpair = [&](void *dst, const TS *src) {
-        if constexpr (sizeof(TS) == 4) cp_async8(dst, src);
+    __shared__ typename std::conditional<sizeof(TD) == 4, float, __nv_bfloat162>::type rcD[RS][TY][2];
+    auto cp_dpair = [&](void *dst, const TD *src) {
+        if constexpr (sizeof(TD) == 4) cp_async8(dst, src);
         else cp_async4(dst, src);
     };
     auto dpair = [&](const DPair &v) -> float2 {
-        if constexpr (sizeof(TS) == 4) return v;
+        if constexpr (sizeof(TD) == 4) return v;
         else return __bfloat1622float2(v);
     };
     const int tid = ty * TX + tx, hrow = ty == 0 ? 0 : 1;
@@ -1873,7 +1875,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
             if (xl) {
                 const int kl = kn + dxl;
                 cp_async16(&rcX[sl][ty][0], X + (kl >> 1));
-                if (!kPlain) cp_async4(&rcD[sl][ty][0], D + (sizeof(TS) == 4 ? kl : kl - 1));
+                if (!kPlain) cp_async4(&rcD[sl][ty][0], D + (sizeof(TD) == 4 ? kl : kl - 1));
             }
             if (xr) {
                 const int kr = kn + dxr;
@@ -1999,7 +2001,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
             if (xl) {
                 const float4 pv = rcX[j][ty][0];
                 const DF xv{pv.y, pv.w};
-                if constexpr (sizeof(TS) == 4)
+                if constexpr (sizeof(TD) == 4)
                     hl = kPlain ? xv : df_add_f(xv, rcD[j][ty][0]);
                 else
                     hl = kPlain ? xv : df_add_f(xv, __high2float(rcD[j][ty][0]));
@@ -2007,7 +2009,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine_df2(Geo g, int zlen, int
             if (xr) {
                 const float4 pv = rcX[j][ty][1];
                 const DF xv{pv.x, pv.z};
-                if constexpr (sizeof(TS) == 4)
+                if constexpr (sizeof(TD) == 4)
                     hr = kPlain ? xv : df_add_f(xv, rcD[j][ty][1]);
                 else
                     hr = kPlain ? xv : df_add_f(xv, __low2float(rcD[j][ty][1]));
@@ -4606,18 +4608,18 @@ TS *cheb_pairs(int zlen, const Geo &g, int nf, const Coef32 &cf, float gamma, do
 // A double-float refinement pass of mode kMode: the two-cells-per-thread kernel when nx
 // is even (and no axis but x is periodic), the scalar one otherwise; both use the z-chunks
 // of sw (same partial slots).
-template <class TS, int kMode>
+template <class TS, int kMode, class TD = TS>
 void launch_refine_df(const Geo &g, const Sweep &sw, int nf, const CoefDF &cf, int scheme,
-                      const DF *xin, const TS *d, const DF *b, DF *xout, DF *bout, TS *r, TS *y1,
+                      const DF *xin, const TD *d, const DF *b, DF *xout, DF *bout, TS *r, TS *y1,
                       float gamma, double *partials, RefScal *sc, RefScal *sc_next,
                       cudaStream_t st) {
     const dim3 blk(TX, TY);
     if (df_pairs(g)) {
         const dim3 grid((g.nx + 2 * TX - 1) / (2 * TX), sw.grid.y, sw.grid.z);
-        launch_chain(k_refine_df2<TS, kMode>, grid, blk, st, g, sw.zlen, sw.nzc, cf,
+        launch_chain(k_refine_df2<TS, kMode, TD>, grid, blk, st, g, sw.zlen, sw.nzc, cf,
                      scheme, xin, d, b, xout, bout, r, y1, gamma, partials, sc, sc_next);
     } else {
-        launch_chain(k_refine_df<TS, kMode>, sw.grid, blk, st, g, sw.zlen, sw.nzc, cf, scheme, xin,
+        launch_chain(k_refine_df<TS, kMode, TD>, sw.grid, blk, st, g, sw.zlen, sw.nzc, cf, scheme, xin,
                      d, b, xout, bout, r, y1, gamma, partials, sc, sc_next);
     }
 }
@@ -5718,16 +5720,19 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     // solve's), where it pays, nothing caps the iterations, and its vectors may be held
     const PredPlan *pred = nullptr;
     const size_t base_b = 4 * v64 + 5 * vts + align_up(rp.ok ? rp.ws_bytes : 0);
-    if (kDF && sizeof(TS) == 4 && !persistent) {
-        const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, m_it, c, lmax);
+    const size_t vpd = align_up((size_t)n * nf * 4);   // one FP32 vector of the expansion
+    if (kDF && !persistent) {
+        const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, cheb_iters(lmax, 1e-6), c, lmax);
+        // (a round cap that the own rounds' start would exceed is refused as ever)
         if (q.use && p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
-            m->ws_diffuse.ensure(base_b + (size_t)(q.maxK + 1 + pred_vectors(q.maxlen)) * vts) == CG_OK)
+            (p->max_rounds <= 0 || p->max_rounds >= (sizeof(TS) == 2 ? 5 : 2)) &&
+            m->ws_diffuse.ensure(base_b + (size_t)(q.maxK + 1 + pred_vectors(q.maxlen)) * vpd) == CG_OK)
             pred = &q;
     }
     if (!pred) CGK_TRY(m->ws_diffuse.ensure(base_b));
     char *wb = m->ws_diffuse.as<char>();
     char *rws = wb + 4 * v64 + 5 * vts;
-    float *PT = (float *)(wb + base_b), *PD = pred ? PT + (size_t)(pred->maxK + 1) * (vts / 4) : nullptr;
+    float *PT = (float *)(wb + base_b), *PD = pred ? PT + (size_t)(pred->maxK + 1) * (vpd / 4) : nullptr;
     XT *X1 = (XT *)wb, *X2 = (XT *)(wb + v64), *B = (XT *)(wb + 2 * v64), *X0 = (XT *)(wb + 3 * v64);
     TS *R = (TS *)(wb + 4 * v64), *Ya = (TS *)(wb + 4 * v64 + vts), *Yb = (TS *)(wb + 4 * v64 + 2 * vts);
     // two more iterate buffers for two-iterations-per-launch sweeps
@@ -5802,16 +5807,18 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
         // rounds per step: remembered for this signature, else an a-priori start (two
         // FP32 inner solves of ~1e-6 each reach 1e-13 from a residual below |b|)
         const int max_r = p->max_rounds > 0 ? p->max_rounds : 12;
-        int R = sizeof(TS) == 2 ? 5 : 2;
+        // (BF16 rounds gain about 2.5 digits each: five from r = c L u, three and the shared
+        // expansion's from there)
+        int R = sizeof(TS) == 2 ? (pred ? 4 : 5) : 2;
         RoundsEntry *remembered = nullptr;
         for (RoundsEntry &re : m->rounds)
             if (re.nf == nf && re.precision == p->precision && re.scheme == p->scheme &&
-                re.nsteps == p->nsteps && re.T == T && re.tol == p->tol) {
+                re.nsteps == p->nsteps && re.T == T && re.tol == p->tol && re.predicted == (pred != nullptr)) {
                 R = re.rounds;
                 remembered = &re;
             }
         if (!remembered) {
-            m->rounds.push_back(RoundsEntry{nf, p->precision, p->scheme, p->nsteps, T, p->tol, R});
+            m->rounds.push_back(RoundsEntry{nf, p->precision, p->scheme, p->nsteps, T, p->tol, R, pred != nullptr});
             remembered = &m->rounds.back();
         }
         XT *last_result = nullptr;
@@ -5868,7 +5875,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                     TS *y1_start = Ya;
                     int run = -1;   // the current run of the shared expansion
                     // merged passes between the steps of a run (one inner solve per step)
-                    const bool mid = pred && R == 2 && mid_fits(g, p->scheme);
+                    const bool mid = sizeof(TS) == 4 && pred && R == 2 && mid_fits(g, p->scheme);
                     bool merged_in = false;   // the step was started by a merged pass
                     for (int s2 = 0; s2 < p->nsteps; ++s2) {
                         RefScal *slot = hist + (size_t)s2 * nf;
@@ -5886,26 +5893,25 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                                (DF *)B, R_, y1, (float)gamma,
                                                                partials, slot, slot, cs));
                         XT *xc = u;
-                        if constexpr (sizeof(TS) == 4)
-                            if (pred) {   // the step's first round
-                                if (run_start) launch_pred(*pred, ++run, g, nf, (const DF *)u, PT, PD, vts / 4, cs);
-                                const float *d0 = PD + (size_t)(s2 - pred->start[run]) * (vts / 4);
-                                // (a merged pass at the end of the step before has left this
-                                // step's first residual, and u + d0 is formed where it is read)
-                                if (merged_in) {
-                                } else if (cn)
-                                    CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
-                                               launch_refine_df<TS, 1>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
-                                                                       (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
-                                                                       (float)gamma, partials, slot, slot, cs));
-                                else
-                                    CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
-                                               launch_refine_df<TS, 4>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
-                                                                       (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
-                                                                       (float)gamma, partials, slot, slot, cs));
-                                if (!merged_in) xc = f1;
-                            }
-                        const int mi = pred ? pred->m[s2] : m_it;   // inner iterations of a round
+                        if (pred) {   // the step's first round
+                            if (run_start) launch_pred(*pred, ++run, g, nf, (const DF *)u, PT, PD, vpd / 4, cs);
+                            const float *d0 = PD + (size_t)(s2 - pred->start[run]) * (vpd / 4);
+                            // (a merged pass at the end of the step before has left this
+                            // step's first residual, and u + d0 is formed where it is read)
+                            if (merged_in) {
+                            } else if (cn)
+                                CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
+                                           launch_refine_df<TS, 1, float>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
+                                                                   (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
+                                                                   (float)gamma, partials, slot, slot, cs));
+                            else
+                                CGK_LAUNCH("refine_df", (double)n * nf * (24 + 3 * sizeof(TS)), cs,
+                                           launch_refine_df<TS, 4, float>(g, sw, nf, cfdf, p->scheme, (const DF *)u, d0,
+                                                                   (const DF *)bp_, (DF *)f1, (DF *)nullptr, R_, y1,
+                                                                   (float)gamma, partials, slot, slot, cs));
+                            if (!merged_in) xc = f1;
+                        }
+                        const int mi = pred && sizeof(TS) == 4 ? pred->m[s2] : m_it;   // inner iterations of a round
                         for (int r = pred ? 1 : 0; r < R; ++r) {
                             TS *yc = y1, *yp = nullptr, *yo = (y1 == Ya) ? Yb : Ya;
                             double om = 1.0;
@@ -5953,7 +5959,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                             if constexpr (sizeof(TS) == 4)
                                 if (last && mid) {
                                     const int i = s2 - pred->start[run];
-                                    const float *e0 = PD + (size_t)i * (vts / 4);
+                                    const float *e0 = PD + (size_t)i * (vpd / 4);
                                     merged_in = i + 1 < pred->len[run];
                                     y1 = (yc == Ya) ? Yb : Ya;
                                     if (merged_in) y1_start = y1;
@@ -5961,7 +5967,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                (double)n * nf * ((merged_in ? 36 : 24) + (cn ? 16 : 0)), cs,
                                                launch_refine_mid(g, sw_mid, cfdf, p->scheme, (const DF *)u, e0,
                                                                  (const float *)yc,
-                                                                 merged_in ? e0 + vts / 4 : nullptr, (const DF *)bp_,
+                                                                 merged_in ? e0 + vpd / 4 : nullptr, (const DF *)bp_,
                                                                  (DF *)xn, (DF *)B, (float *)R_, (float *)y1,
                                                                  (float)gamma, partials, slot, slot + nf, cs));
                                     xc = xn;
@@ -6048,13 +6054,13 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                     if (pred) {   // expansions, then per step one pass and R - 1 rounds
                         apps = (cn ? 1 : 0) + p->nsteps;
                         for (int K : pred->K) apps += K;
-                        for (int mi : pred->m) apps += (long long)(R - 1) * mi;
+                        for (int mi : pred->m) apps += (long long)(R - 1) * (sizeof(TS) == 4 ? mi : m_it);
                     }
                     rep->iters = apps * nf;
                     rep->refine_rounds = (long long)p->nsteps * R;
                     rep->cell_updates = apps * nf * (long long)n;
                     rep->final_rel_residual = worst_g;
-                    rep->inner_iters_per_round = pred ? pred->maxm : m_it;
+                    rep->inner_iters_per_round = pred && sizeof(TS) == 4 ? pred->maxm : m_it;
                     rep->sweep_shape_used = shape_used;
                 }
                 return CG_OK;

@@ -110,3 +110,28 @@ def test_batches_match_single_meshes(nsteps, scheme):
         for f in (0, 1):
             bound = 2e-13 * nsteps * np.sqrt(np.mean(us[s][f] ** 2)) * 40
             assert np.max(np.abs(got[504][s][f] - lone[f])) <= bound
+
+
+@pytest.mark.parametrize("dims,period", [((32, 24, 16), (0, 0, 0)), ((33, 20, 17), (0, 0, 0)),
+                                         ((64, 10, 9), (1, 0, 0)), ((30, 12, 7), (1, 1, 1))])
+@pytest.mark.parametrize("scheme", [0, 1])
+def test_bf16_inner_storage_takes_the_fp32_increments(dims, period, scheme):
+    """BF16 inner storage: the expansion's FP32 increments, then BF16 rounds; against FP32
+    storage to the tolerance above.  A round cap below its five own rounds stays refused."""
+    import torch
+
+    import paper_1409_0001_gb300 as cg
+    n = dims[0] * dims[1] * dims[2]
+    rng = np.random.default_rng(n)
+    u = np.stack([rng.random(n), rng.standard_normal(n)])
+    ref, _ = solve(cg, dims, u, 0.2, 8, scheme, period)
+    mesh = cg.StructuredMesh(dims, (0, 0, 0), 1.0, periodic=period)
+    par = dict(T=1.6, nsteps=8, scheme=scheme, precision=cg.PREC_BF16_DF_REFINE)
+    x = torch.from_numpy(u).cuda()
+    _, rep = cg.diffuse(mesh, x, cg.Params(**par), report=True)
+    assert rep["final_rel_residual"] <= 1e-13
+    for f in (0, 1):
+        assert np.max(np.abs(x[f].cpu().numpy() - ref[f])) <= 2e-13 * 8 * np.sqrt(np.mean(u[f] ** 2)) * 40
+    with pytest.raises(cg.CGError):
+        cg.diffuse(mesh, torch.from_numpy(u).cuda(), cg.Params(max_rounds=4, **par))
+    mesh.close()
