@@ -4094,14 +4094,28 @@ __global__ void k_mass_batched(const SnapDesc<TS> *__restrict__ sd, int nf, doub
 }
 
 // sum_k V_c,k u_k per field (1-D grid-stride; any mesh)
+// sum_k V_k u_k per field.  Few blocks of many cells each: a block's FP64 reduction and the
+// last block's sum of the partials cost more than its cells on a small mesh (GB300 issues a
+// warp's FP64 instruction in 16 cycles).
 __global__ void k_mass(int n, const double *__restrict__ u_all, const double *__restrict__ vc,
                        double vcu, double *__restrict__ partials_all, unsigned int *tickets,
                        double *__restrict__ out) {
     const int f = blockIdx.y;
     const double *u = u_all + (size_t)f * n;
     double s = 0.0;
-    for (int k = blockIdx.x * kThreads + threadIdx.x; k < n; k += gridDim.x * kThreads)
-        s += (vc ? vc[k] : vcu) * u[k];
+    const int step = gridDim.x * kThreads;
+    int k = blockIdx.x * kThreads + threadIdx.x;
+    for (; k + 7 * (long long)step < n; k += 8 * step) {   // eight cells in flight
+        double x[8], v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            x[j] = u[k + j * step];
+            v[j] = vc ? vc[k + j * step] : vcu;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s += v[j] * x[j];
+    }
+    for (; k < n; k += step) s += (vc ? vc[k] : vcu) * u[k];
     double v = block_sum(s);
     double *partials = partials_all + (size_t)f * gridDim.x;
     if (arrive(partials, 1, &v, blockIdx.x, gridDim.x, &tickets[f])) {
@@ -5039,7 +5053,8 @@ cg_status solid_velocity_run(int64_t n, int ncomp, const double *eps, const doub
 static cg_status field_mass_launch(cg_mesh *m, int nf, const double *cells, cudaStream_t st,
                                    double *keep = nullptr) {
     int n = (int)m->ncells;
-    int G = stencil_grid(n);
+    // a block per 2048 cells, at most four to an SM over all fields
+    const int G = std::max(1, std::min((n + 2047) / 2048, std::max(1, 4 * num_sms() / nf)));
     size_t need = align_up((size_t)nf * G * 8) + 64 * 8 + 64 * 4;
     CGK_TRY(m->ws_small.ensure(4096 + need));
     char *base = m->ws_small.as<char>() + 4096;
