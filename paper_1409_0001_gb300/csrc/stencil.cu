@@ -1455,8 +1455,10 @@ __device__ __forceinline__ DF df_add_f(DF a, float b) {
     s.lo += a.lo;
     return df_fast2sum(s.hi, s.lo);
 }
+// (Products are rounded explicitly: fused into the sum that follows, as the compiler may in
+// one instantiation and not in another, they would change its bits.)
 __device__ __forceinline__ DF df_mul(DF a, DF b) {
-    float p = a.hi * b.hi;
+    float p = __fmul_rn(a.hi, b.hi);
     float e = fmaf(a.hi, b.hi, -p);
     e = fmaf(a.hi, b.lo, e);
     e = fmaf(a.lo, b.hi, e);
@@ -1468,7 +1470,7 @@ __device__ __forceinline__ float df_f(DF a) { return a.hi + a.lo; }
 // the cross terms, as an unevaluated pair (for a value that is rounded to FP32 or added
 // into another pair next).
 __device__ __forceinline__ DF df_mul_un(DF c, DF a) {
-    const float p = c.hi * a.hi;
+    const float p = __fmul_rn(c.hi, a.hi);
     float e = fmaf(c.hi, a.hi, -p);
     e = fmaf(c.hi, a.lo, e);
     e = fmaf(c.lo, a.hi, e);
@@ -1478,7 +1480,7 @@ __device__ __forceinline__ DF df_mul_un(DF c, DF a) {
 // L = s - nn v: the Laplacian numerator of a cell from its neighbour sum s (as the
 // engines accumulate it) and its own value v; one TwoSum where the two meet.
 __device__ __forceinline__ DF df_lap(DF s, DF v, float nn) {
-    const float p = nn * v.hi;
+    const float p = __fmul_rn(nn, v.hi);
     const float ep = fmaf(nn, v.hi, -p);
     const DF t = df_two_sum(s.hi, -p);
     return DF{t.hi, ((s.lo - fmaf(nn, v.lo, ep)) + t.lo)};
@@ -3831,6 +3833,64 @@ __device__ __forceinline__ void batched_refine(const SnapDesc<TS> &d, int nf, co
     if (is_thread0() && part) *part = tot;
 }
 
+// The merged pass of k_refine_mid for a flat-plane snapshot: the iterate alternates between U
+// (even steps' u_s) and X2, so that no block writes what another still reads.
+template <class TS, bool COH>
+__device__ __forceinline__ void batched_mid(const SnapDesc<TS> &d, int nf, const BItem &it, int step, bool end,
+                                            double *part, double *part_next) {
+    const Geo g = d.g;
+    const int scheme = d.scheme, pts = d.pts;
+    const DF cf_ce = d.cfdf.ce;
+    const int f = it.zf / d.nzc;
+    const int zc = it.zf - f * d.nzc;
+    const int z0 = zc * d.zlen, z1 = min(g.nz, z0 + d.zlen);
+    const size_t off = (size_t)f * g.n, off_ts = (size_t)f * g.nz * pts, ds = (size_t)nf * g.nz * pts;
+    const DF *u = ((step & 1) ? d.X2 : d.U) + off;
+    DF *xout = ((step & 1) ? d.U : d.X2) + off;
+    const DF *b = scheme == 1 ? d.B + off : u;
+    DF *bo = d.B + off;
+    const float *e = d.D + step * ds + off_ts, *en = e + ds;
+    const TS *dd = d.Yb + off_ts;
+    TS *r = d.R + off_ts, *y1 = d.Ya + off_ts;
+    const float gamma = d.gamma;
+    float acc = 0.0f, acc_b = 0.0f;
+    sweep_flat_at<DFe, kFlatCptDF>(
+        g, pts, it.bx, z0, z1,
+        [&](int k, int kt) {
+            return DFeRaw{bld_df<COH>(u, k), e[kt], bld<COH>(dd, kt), end ? 0.0f : en[kt]};
+        },
+        [](DFeRaw v) { return DFe{df_add_f(df_add_f(v.u, v.e), v.d), DF{v.en, 0.0f}}; },
+        [&](int k) { return bld_df<COH>(b, k); },
+        [&](int k, int kt, DFe v, DFe sm, int nn, DF bk) {
+            xout[k] = v.x;
+            const DF lx = df_lap(sm.x, v.x, (float)nn);
+            const float rf = df_f(df_res(bk, v.x, cf_ce, lx));
+            acc = fmaf(rf, rf, acc);
+            if (!end) {
+                const DF le = df_lap(sm.e, v.e, (float)nn);
+                DF bn = v.x, m = lx;
+                if (scheme == 1) {
+                    bn = v.x + df_mul(cf_ce, lx);
+                    bo[k] = bn;
+                    m = DF{2.0f * lx.hi, 2.0f * lx.lo};
+                }
+                const float bf = df_f(bn);
+                acc_b = fmaf(bf, bf, acc_b);
+                const DF t = df_two_sum(m.hi, le.hi);
+                const DF q = df_mul_un(cf_ce, DF{t.hi, (m.lo + le.lo) + t.lo});
+                const DF w = df_two_sum(-v.e.hi, q.hi);
+                const float rn = w.hi + (q.lo + w.lo);
+                st(r, kt, rn);
+                st(y1, kt, gamma * rn);
+            }
+        });
+    const double tb = block_sum_f(acc_b), tot = block_sum_f(acc);
+    if (is_thread0()) {
+        *part = tot;
+        if (!end) *part_next = tb;
+    }
+}
+
 template <class TS, bool COH>
 __device__ __forceinline__ void batched_cheb(const SnapDesc<TS> &d, const BItem &it, int k) {
     const Geo g = d.g;   // register copies of the descriptor's fields (see batched_refine)
@@ -3872,7 +3932,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
                                                       int nf, const BItem *__restrict__ ritems,
                                                       int nr, const BItem *__restrict__ citems,
                                                       int nc, int nsteps, int R, int mmax, int pred,
-                                                      int cn, double *__restrict__ part_rr,
+                                                      int cn, int mid, double *__restrict__ part_rr,
                                                       double *__restrict__ part_bb, GridBar *gb,
                                                       long long budget) {
     // phase 0: u^0 -> double-float (with the expansion it has run: k_bconvert)
@@ -3899,6 +3959,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
         }
         for (int round = 1; round <= R; ++round) {
             const bool shared = pred && round == 1;
+            if (shared && mid && step > 0) continue;   // the merged pass has started the step
             for (int k = 1; k < (shared ? 1 : mmax); ++k) {
                 for (int i = blockIdx.x; i < nc; i += gridDim.x) {
                     const BItem it = citems[i];
@@ -3908,6 +3969,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
             }
             for (int i = blockIdx.x; i < nr; i += gridDim.x) {
                 const BItem it = ritems[i];
+                if constexpr (sizeof(TS) == 4)
+                    if (mid && round == R) {
+                        batched_mid<TS, true>(sd[it.snap], nf, it, step, step + 1 == nsteps,
+                                              part_rr + (size_t)step * nr + i,
+                                              part_bb + (size_t)(step + 1 < nsteps ? step + 1 : step) * nr + i);
+                        continue;
+                    }
                 batched_refine<TS, true>(sd[it.snap], nf, it, false, round, R,
                                    round == R ? part_rr + (size_t)step * nr + i : nullptr,
                                    round == R && step + 1 < nsteps && (!pred || cn)
@@ -3962,6 +4030,20 @@ __global__ void __launch_bounds__(kThreads, 3) k_brefine(const SnapDesc<TS> *__r
     const BItem it = ritems[i];
     batched_refine<TS, false>(sd[it.snap], nf, it, first != 0, round, R, part ? part + i : nullptr,
                               part_next ? part_next + i : nullptr, pstep, part_b ? part_b + i : nullptr);
+}
+
+// A merged pass of every snapshot (see batched_mid).  64 snapshots x 5 fields: 1.49 ms at 128
+// registers (2.6 TB/s, latency) in the place of two k_brefine passes of 1.00 ms each; the call 85
+// -> 80 ms.
+template <class TS>
+__global__ void __launch_bounds__(kThreads, 2) k_bmid(const SnapDesc<TS> *__restrict__ sd, int nf,
+                                                    const BItem *__restrict__ ritems, int step, int end,
+                                                    double *part, double *part_next) {
+    chain_wait();
+    chain_release();
+    const int i = blockIdx.x;
+    const BItem it = ritems[i];
+    batched_mid<TS, false>(sd[it.snap], nf, it, step, end != 0, part + i, part_next + i);
 }
 
 // The shared expansion of a batch, one field of every snapshot at a time (so that the
@@ -4066,14 +4148,14 @@ __global__ void k_batched_hist(const int *__restrict__ first_item, int nsnap, in
 // the tolerance (otherwise the inputs stay intact for a run with more rounds).
 template <class TS>
 __global__ void k_batched_final(const SnapDesc<TS> *__restrict__ sd, int nf, double *const *cells,
-                                const unsigned int *__restrict__ bad) {
+                                const unsigned int *__restrict__ bad, int in_x2) {
     if (*bad != 0u) return;
     const SnapDesc<TS> &d = sd[blockIdx.y];
     const size_t cnt = (size_t)d.g.n * nf;
     double *out = cells[blockIdx.y];
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (size_t)gridDim.x * blockDim.x) {
-        DF v = d.U[i];
+        DF v = in_x2 ? d.X2[i] : d.U[i];
         out[i] = (double)v.hi + (double)v.lo;
     }
 }
@@ -6472,6 +6554,11 @@ static cg_status batch_upload(BatchPlan<TS> &P, BatchArena &A, char *ab, int nsn
     return CG_OK;
 }
 
+// One inner solve per step: the steps of a batch with the expansion end in merged passes,
+// whose last iterate is in X2 after an odd number of steps.
+static bool batch_mid(bool pred, int R) { return pred && R == 2; }
+static int batch_in_x2(bool pred, int R, int nsteps) { return batch_mid(pred, R) && nsteps % 2 ? 1 : 0; }
+
 // The launches of the shared expansion (before either schedule): u^0 -> double-float, then
 // per field the recurrence and the combination.
 template <class TS>
@@ -6521,7 +6608,7 @@ static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A,
     for (const auto &d : P.descs)
         for (int k = 1; k < d.m; ++k) cheb_bytes[(size_t)k] += (double)d.g.n * nf * 4.0 * sizeof(TS);
     const double ref_bytes = cells_f * (24.0 + 3.0 * sizeof(TS));
-    const bool cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON;
+    const bool cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON, mid = batch_mid(pred, R);
     if (!pred)
         CGK_LAUNCH("bconvert", cells_f * 16.0, st,
                    launch_chain(k_bconvert<TS>, dim3(num_sms() * 2, nsnap), dim3(TX, TY), st, dsd, nf));
@@ -6532,9 +6619,18 @@ static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A,
                                     (double *)nullptr, -1, (double *)nullptr));
         for (int round = 1; round <= R; ++round) {
             const bool shared = pred && round == 1;
+            if (shared && mid && step > 0) continue;
             for (int k = 1; k < (shared ? 1 : P.mmax); ++k)
                 CGK_LAUNCH(cname, cheb_bytes[(size_t)k], st,
                            launch_chain(k_bcheb<TS>, dim3(nc), dim3(TX, TY), st, dsd, dci, k));
+            if constexpr (sizeof(TS) == 4)
+                if (mid && round == R) {
+                    const int end = step + 1 == nsteps ? 1 : 0;
+                    CGK_LAUNCH("bmid_fp32", cells_f * (end ? 24.0 : 36.0), st,
+                               launch_chain(k_bmid<TS>, dim3(nr), dim3(TX, TY), st, dsd, nf, dri, step, end,
+                                            prr + (size_t)step * nr, pbb + (size_t)(end ? step : step + 1) * nr));
+                    continue;
+                }
             double *part = round == R ? prr + (size_t)step * nr : nullptr;
             double *next = round == R && step + 1 < nsteps && (!pred || cn) ? pbb + (size_t)(step + 1) * nr : nullptr;
             double *partb = shared && !cn ? pbb + (size_t)step * nr : nullptr;
@@ -6567,9 +6663,10 @@ static cg_status batch_issue(const BatchPlan<TS> &P, const BatchArena &A, int ns
     CGK_CUDA(cudaMemsetAsync(bad, 0, sizeof(unsigned int), st));
     int a_ns = nsnap, a_nf = nf, a_nr = nr, a_nc = nc, a_steps = nsteps, a_R = R, a_mm = P.mmax;
     int a_pred = pred ? 1 : 0, a_cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON ? 1 : 0;
+    int a_mid = batch_mid(pred, R) ? 1 : 0;
     long long a_budget = budget;
     if (pred) CGK_TRY(batch_issue_pred(P, A, nf, nsteps, st));
-    void *args[] = {&dsd, &a_ns, &a_nf, &dri, &a_nr, &dci, &a_nc, &a_steps, &a_R, &a_mm, &a_pred, &a_cn,
+    void *args[] = {&dsd, &a_ns, &a_nf, &dri, &a_nr, &dci, &a_nc, &a_steps, &a_R, &a_mm, &a_pred, &a_cn, &a_mid,
                     &prr, &pbb, &gb, &a_budget};
     double bytes = 0.0;
     for (const auto &d : P.descs)
@@ -6590,7 +6687,7 @@ static cg_status batch_issue(const BatchPlan<TS> &P, const BatchArena &A, int ns
     if (final) {
         CGK_LAUNCH("batched_final", 16.0 * P.cells_total * nf, st,
                    k_batched_final<TS><<<dim3(num_sms() * 2, nsnap), kThreads, 0, st>>>(
-                       dsd, nf, (double *const *)(ab + A.o_out), bad));
+                       dsd, nf, (double *const *)(ab + A.o_out), bad, batch_in_x2(pred, R, nsteps)));
         CGK_CUDA(cudaGetLastError());
     }
     return CG_OK;
@@ -6856,7 +6953,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
             CGK_LAUNCH("batched_final", 16.0 * P.cells_total * nf, st,
                        k_batched_final<TS><<<dim3(num_sms() * 2, nsnap), kThreads, 0, st>>>(
                            (const SnapDesc<TS> *)(A.ab + A.o_desc), nf,
-                           (double *const *)(A.ab + A.o_out), bad));
+                           (double *const *)(A.ab + A.o_out), bad, batch_in_x2(P.pred, R, p->nsteps)));
             CGK_CUDA(cudaGetLastError());
             if (rep) {
                 CGK_LAUNCH("mass", 8.0 * P.cells_total * nf, st,
