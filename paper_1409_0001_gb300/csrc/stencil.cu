@@ -694,16 +694,15 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
 // iteration against 19 in the two-launch form that forms A p twice) plus the barriers;
 // the two-launch form spends 12-13 us per launch on meshes this small, most of it launch
 // latency, the last block's sum of the partials and too few resident warps.  Measured per
-// iteration (b = 3 dx, one field): 32^3 27.0 -> 10.2 us, 48^3 27.1 -> 12.2, 64^3 33.0 ->
-// 15.6, 96^3 65.1 -> 30.2.  Each block adds all blocks' partials itself, in block order,
+// iteration (b = 3 dx, one field): 32^3 27.0 -> 9.6 us, 48^3 27.1 -> 11.5, 64^3 33.0 ->
+// 15.3, 96^3 65.1 -> 30.1.  Each block adds all blocks' partials itself, in block order,
 // so the sums are the same bits in every block and every run.  (Partials tagged with the
-// sum's number and polled by every block, which needs no arrival counter, took 12.2 us at
-// 32^3: 152 blocks polling 152 slots.)
+// sum's number and polled by every block, which needs no arrival counter, took 2 us more
+// at 32^3: 152 blocks polling 152 slots.)
 struct CoopBar {
     unsigned int count;
     int err;
 };
-constexpr int kCoopThreads = 512;
 constexpr int kCoopMaxC = 12;    // cells per thread: 6 C registers of state within 128
 
 // Arrival number `target / gridDim.x` of every block; bounded like grid_sync.
@@ -743,18 +742,18 @@ struct CoopScal {
 // fin(a, b) runs on thread 0 with the totals, and its writes to shared memory are visible
 // to the block on return.  The block sum goes through shared memory in full-warp
 // additions (36 FP64 warp instructions for 512 threads; a shuffle tree in every warp
-// would take 85).
-template <bool TWO, class Fin>
+// would take 85).  NT: the block's threads (a multiple of 128).
+template <int NT, bool TWO, class Fin>
 __device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, CoopBar *gb, unsigned target,
                                          long long budget, Fin fin) {
-    __shared__ double2 sv[kCoopThreads];
+    __shared__ double2 sv[NT];
     const int t = threadIdx.x;
     sv[t] = make_double2(a, b);
     __syncthreads();
     if (t < 128) {
         double2 v = sv[t];
 #pragma unroll
-        for (int q = 1; q < kCoopThreads / 128; ++q) {
+        for (int q = 1; q < NT / 128; ++q) {
             const double2 o = sv[t + 128 * q];
             v.x += o.x;
             if (TWO) v.y += o.y;
@@ -800,13 +799,13 @@ __device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, Coop
 // neighbours; part: 2 x gridDim.x partials (alternating); hist[s * nf + f].  A field's
 // iteration stops as in the two-launch form: converged, breakdown, or max_it.  After a
 // step in which a field did not converge nothing more runs.
-template <int C>
-__global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
+template <int NT, int C>
+__global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
     Geo g, int per_block, double c, Coef64 cf, int scheme, int nf, int nsteps, int max_it, double tol2,
     const double *__restrict__ cells, double *X, double *V, double2 *part, Scal *__restrict__ hist,
     CoopBar *gb, long long budget) {
     __shared__ double sdg[8];
-    __shared__ unsigned short face[C][kCoopThreads];
+    __shared__ unsigned short face[C][NT];
     __shared__ CoopScal S;
     stage_table(sdg, cf.dg);
     __syncthreads();
@@ -817,7 +816,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
     // bits per face (0: the adjacent cell, 1: none, 2: the other end of the axis)
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int k = k0 + j * kCoopThreads;
+        const int k = k0 + j * NT;
         if (k < kend) {
             const int z = k / nxy, q = k - z * nxy, y = q / nx, x = q - y * nx;
             const unsigned wx = (g.per & 1) ? 2u : 1u, wy = (g.per & 2) ? 2u : 1u, wz = (g.per & 4) ? 2u : 1u;
@@ -848,7 +847,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
             double rr = 0.0, bb = 0.0;
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                const int k = k0 + j * kCoopThreads;
+                const int k = k0 + j * NT;
                 x[j] = r[j] = p[j] = 0.0;
                 if (k < kend) {
                     int nn;
@@ -862,7 +861,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
                 }
             }
             target += gridDim.x;
-            if (!coop_sum<true>(rr, bb, part + par * gridDim.x, gb, target, budget, [&](double RR, double BB) {
+            if (!coop_sum<NT, true>(rr, bb, part + par * gridDim.x, gb, target, budget, [&](double RR, double BB) {
                     S.rr = RR;
                     S.bb = BB;
                     S.stop = tol2 * BB;
@@ -877,7 +876,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
                 const double beta = S.beta;
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
-                    const int k = k0 + j * kCoopThreads;
+                    const int k = k0 + j * NT;
                     if (k < kend) {
                         p[j] = fma(beta, p[j], r[j]);
                         __stcg(V + k, p[j]);
@@ -889,7 +888,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
                 double pap = 0.0;
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
-                    const int k = k0 + j * kCoopThreads;
+                    const int k = k0 + j * NT;
                     ap[j] = 0.0;
                     if (k < kend) {
                         int nn;
@@ -899,7 +898,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
                     }
                 }
                 target += gridDim.x;
-                if (!coop_sum<false>(pap, 0.0, part + par * gridDim.x, gb, target, budget, [&](double PAP, double) {
+                if (!coop_sum<NT, false>(pap, 0.0, part + par * gridDim.x, gb, target, budget, [&](double PAP, double) {
                         S.breakdown = !(PAP > 0.0);
                         S.alpha = S.rr / PAP;
                     }))
@@ -915,7 +914,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
                     rn = fma(r[j], r[j], rn);
                 }
                 target += gridDim.x;
-                if (!coop_sum<false>(rn, 0.0, part + par * gridDim.x, gb, target, budget, [&](double RR, double) {
+                if (!coop_sum<NT, false>(rn, 0.0, part + par * gridDim.x, gb, target, budget, [&](double RR, double) {
                         S.beta = RR / S.rr;
                         S.rr = RR;
                         S.done = RR <= S.stop;
@@ -926,7 +925,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_cg_coop(
             }
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                const int k = k0 + j * kCoopThreads;
+                const int k = k0 + j * NT;
                 if (k < kend) __stcg(Xf + k, x[j]);
             }
             if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -5189,25 +5188,29 @@ cg_status field_mass_many(int nmesh, cg_mesh *const *ms, int nf, const double *c
 // FP64 CG as one cooperative launch (k_cg_coop) where a field's cells fit in the SMs'
 // registers; *solved stays false where it does not apply or a wait gave up, and the
 // caller's field is then untouched.
-template <int C>
+template <int NT, int C>
 static cudaError_t launch_cg_coop(int grid, Geo g, int per_block, double c, Coef64 cf, int scheme, int nf,
                                   int nsteps, int max_it, double tol2, const double *cells, double *X,
                                   double *V, double2 *part, Scal *hist, CoopBar *gb, cudaStream_t st) {
     long long budget = 2000000000LL;   // clock cycles a wait may take (about one second)
     void *args[] = {&g, &per_block, &c, &cf, &scheme, &nf, &nsteps, &max_it, &tol2, &cells, &X, &V, &part,
                     &hist, &gb, &budget};
-    return cudaLaunchCooperativeKernel((const void *)k_cg_coop<C>, dim3(grid), dim3(kCoopThreads), args, 0, st);
+    return cudaLaunchCooperativeKernel((const void *)k_cg_coop<NT, C>, dim3(grid), dim3(NT), args, 0, st);
 }
 
 static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, const cg_params *p, double c,
                            const Coef64 &cf, cg_report *rep, cudaStream_t st, bool *solved) {
     const int n = g.n;
-    // a block per SM, but at least 64 cells to a block (8^3 on 8 blocks: 8.7 us per
-    // iteration).  Up to 933,888 cells (12 per thread on 152 SMs); there the cooperative form
-    // is still 2.2 times as fast as the two-launch form (30.2 against 65.1 us at 96^3)
+    // A block per SM, but at least 64 cells to a block (8^3 on 8 blocks: 7.5 us per iteration);
+    // up to 933,888 cells (512 threads of 12 on 152 SMs), where the cooperative form is still 2.2
+    // times as fast as the two-launch form (30.1 against 65.1 us at 96^3).  Small meshes take
+    // blocks of fewer threads, so that the solves of several streams share the SMs: blocks of
+    // 512 threads at any size ran six concurrent 32^3 calls one after another, 15.2 ms
+    // against 8.6 with the two-launch form (now 6.0; 64^3 20.3 -> 16.2 ms).
     const int grid = std::max(1, std::min(num_sms(), (n + 63) / 64));
     const int per_block = (n + grid - 1) / grid;
-    const int need = (per_block + kCoopThreads - 1) / kCoopThreads;
+    const int nt = per_block <= 128 * 4 ? 128 : per_block <= 256 * 8 ? 256 : 512;
+    const int need = (per_block + nt - 1) / nt;
     if (need > kCoopMaxC) return CG_OK;
     const size_t vec = align_up((size_t)n * nf * 8), one = align_up((size_t)n * 8);
     const size_t hist_n = (size_t)p->nsteps * nf;
@@ -5225,15 +5228,21 @@ static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, cons
     const int max_it = p->max_iter > 0x7ffffff0 ? 0x7ffffff0 : (p->max_iter + 7) / 8 * 8;
     const double tol2 = p->tol * p->tol;
     cudaError_t e = cudaSuccess;
-#define CGK_COOP(C)                                                                                        \
+#define CGK_COOP(NT, C)                                                                                    \
     CGK_LAUNCH("cg64_coop", (double)n * nf * 16, st,                                                       \
-               e = launch_cg_coop<C>(grid, g, per_block, c, cf, p->scheme, nf, p->nsteps, max_it, tol2,    \
+               e = launch_cg_coop<NT, C>(grid, g, per_block, c, cf, p->scheme, nf, p->nsteps, max_it, tol2,    \
                                      cells, X, V, part, hist, gb, st))
-    if (need <= 1) CGK_COOP(1);
-    else if (need <= 2) CGK_COOP(2);
-    else if (need <= 4) CGK_COOP(4);
-    else if (need <= 8) CGK_COOP(8);
-    else CGK_COOP(12);
+    if (nt == 128) {
+        if (need <= 1) CGK_COOP(128, 1);
+        else if (need <= 2) CGK_COOP(128, 2);
+        else CGK_COOP(128, 4);
+    } else if (nt == 256) {
+        if (need <= 4) CGK_COOP(256, 4);
+        else CGK_COOP(256, 8);
+    } else {
+        if (need <= 8) CGK_COOP(512, 8);
+        else CGK_COOP(512, 12);
+    }
 #undef CGK_COOP
     if (e != cudaSuccess) {   // not launched: the two-launch form takes the call
         cudaGetLastError();
