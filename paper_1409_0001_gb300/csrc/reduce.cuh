@@ -12,6 +12,31 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Programmatic dependent launch: a kernel of the solver chain is launched while its
+// predecessor drains; it waits here until the predecessor grid has completed and its
+// writes are visible, and lets its own successor start launching right away.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch a kernel of the solver chain with programmatic dependent launch enabled.
+template <class... KArgs, class... Args>
+inline void launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
+                  Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double ws[kThreads / 32];
     const int t = threadIdx.y * blockDim.x + threadIdx.x;

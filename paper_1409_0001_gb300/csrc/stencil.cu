@@ -46,14 +46,6 @@ struct Geo {
     int per = 0;   // periodic axes: bit 0 x, bit 1 y, bit 2 z (scalar engines only)
 };
 
-// Programmatic dependent launch: a kernel of the solver chain is launched while its
-// predecessor drains; it waits here until the predecessor grid has completed and its
-// writes are visible, and lets its own successor start launching right away.
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_release() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Launch geometry of a 2.5D sweep: blocks of TX x TY columns, each marching over zlen
 // planes; blockIdx.z = f * nzc + z-chunk.
 struct Sweep {
@@ -4479,23 +4471,6 @@ int cheb_iters(double lmax, double eps) {
     double rho = (std::sqrt(kappa) - 1.0) / (std::sqrt(kappa) + 1.0);
     int m = (int)std::ceil(std::log(2.0 * std::sqrt(kappa) / eps) / std::log(1.0 / rho));
     return m < 1 ? 1 : (m > 400 ? 400 : m);
-}
-
-// Launch a kernel of the solver chain with programmatic dependent launch enabled.
-template <class... KArgs, class... Args>
-void launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
-                  Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 // One launch of the TMA-staged sweep (FP32 storage): zlen planes per block.  The tensor
