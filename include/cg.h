@@ -205,7 +205,7 @@ typedef struct {
     double mass_out[CG_REPORT_MAX_FIELDS];  /* ... after smoothing (Eq. (conserve)) */
     long long n_out_of_domain;
     int fixed_point_bits[CG_REPORT_MAX_FIELDS];
-    int inner_iters_per_round;/* mixed: Chebyshev iterations per refinement round */
+    int inner_iters_per_round;/* mixed: Chebyshev iterations per refinement round (the most of any step) */
     int sweep_shape_used;     /* mixed hex: the sweep shape (or batched z planes) that ran */
 } cg_report;
 

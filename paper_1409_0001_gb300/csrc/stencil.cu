@@ -1588,32 +1588,61 @@ __device__ __forceinline__ DF2 df2_of(float4 v) {
 }
 __device__ __forceinline__ float4 f4_of(DF2 a) { return make_float4(a.hi.x, a.hi.y, a.lo.x, a.lo.y); }
 
+// A double as hi = fl32(v), lo = fl32(v - hi).  (By integer arithmetic on the significand, as
+// df_join: the integer to float conversion is no faster than the four FP64 instructions
+// it saves, 163 against 129 us for 16.8 M values.)
+__device__ __forceinline__ DF df_split(double v) {
+    const float hi = __double2float_rn(v);
+    return DF{hi, __double2float_rn(v - (double)hi)};
+}
+// fl64(hi + lo) without the FP64 pipe, which takes 16 cycles per warp instruction and bound
+// the conversion (three instructions a value): where hi's exponent lies in [-70, 126], hi's
+// significand with 29 more bits plus lo in units of its last one, rounded half to even; the
+// FP64 definition elsewhere and where the sum falls below hi's power of two.  The same
+// bits; 16.8 M values 101 -> 56 us, 512 x 256 x 256 193 -> 100 us (5.3 TB/s).
+__device__ __forceinline__ double df_join(float hi, float lo) {
+    const unsigned hb = __float_as_uint(hi);
+    const int e = (int)((hb >> 23) & 0xffu) - 127;
+    if (e >= -70 && e <= 126) {
+        const float l = __fmul_rn((hb >> 31) ? -lo : lo, __uint_as_float((unsigned)(52 - e + 127) << 23));
+        const float k = floorf(l), fr = __fsub_rn(l, k);
+        const long long h = (long long)((hb & 0x7fffffu) | 0x800000u) << 29;
+        if (fabsf(l) < 1073741824.0f) {
+            const long long s0 = h + (long long)__float2int_rn(k);
+            const long long s = s0 + ((fr > 0.5f || (fr == 0.5f && (s0 & 1))) ? 1 : 0);
+            if (s0 >= (1ll << 52) && s <= (1ll << 53))
+                return __longlong_as_double((long long)((((unsigned long long)(e + 1023)) << 52) +
+                                                        (unsigned long long)(s - (1ll << 52)) +
+                                                        ((unsigned long long)(hb & 0x80000000u) << 32)));
+        }
+    } else if (((hb | __float_as_uint(lo)) & 0x7fffffffu) == 0) {
+        return __longlong_as_double((long long)((unsigned long long)(hb & __float_as_uint(lo)) << 32));
+    }
+    return (double)hi + (double)lo;
+}
+
 __global__ void k_to_df(size_t n, const double *__restrict__ u, DF *__restrict__ x) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        double v = u[i];
-        float hi = __double2float_rn(v);
-        x[i] = DF{hi, __double2float_rn(v - (double)hi)};
-    }
+         i += (size_t)gridDim.x * blockDim.x)
+        x[i] = df_split(u[i]);
 }
 
 __global__ void k_from_df(size_t n, const DF *__restrict__ x, double *__restrict__ u) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x) {
-        DF v = x[i];
-        u[i] = (double)v.hi + (double)v.lo;
+        const DF v = x[i];
+        u[i] = df_join(v.hi, v.lo);
     }
 }
 
 // The same conversions in the pair layout of the two-cells-per-thread kernels: cells
 // 2i and 2i + 1 as one float4 (hi0, hi1, lo0, lo1).  Same values as k_to_df / k_from_df.
+// (the caller's field may start at any multiple of eight bytes)
 __global__ void k_to_df_pairs(size_t npairs, const double *__restrict__ u, float4 *__restrict__ x) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < npairs;
          i += (size_t)gridDim.x * blockDim.x) {
-        const double v0 = u[2 * i], v1 = u[2 * i + 1];
-        const float h0 = __double2float_rn(v0), h1 = __double2float_rn(v1);
-        x[i] = make_float4(h0, h1, __double2float_rn(v0 - (double)h0),
-                           __double2float_rn(v1 - (double)h1));
+        const DF a = df_split(u[2 * i]), b = df_split(u[2 * i + 1]);
+        x[i] = make_float4(a.hi, b.hi, a.lo, b.lo);
     }
 }
 
@@ -1621,8 +1650,8 @@ __global__ void k_from_df_pairs(size_t npairs, const float4 *__restrict__ x, dou
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < npairs;
          i += (size_t)gridDim.x * blockDim.x) {
         const float4 v = x[i];
-        u[2 * i] = (double)v.x + (double)v.z;
-        u[2 * i + 1] = (double)v.y + (double)v.w;
+        u[2 * i] = df_join(v.x, v.z);
+        u[2 * i + 1] = df_join(v.y, v.w);
     }
 }
 
@@ -3934,9 +3963,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batched(const SnapDesc<TS> *__r
         const double *u = sd[s].cells;
         DF *U = sd[s].U;
         for (size_t i = tid; i < cnt; i += nthr) {
-            double v = u[i];
-            float hi = __double2float_rn(v);
-            U[i] = DF{hi, __double2float_rn(v - (double)hi)};
+            U[i] = df_split(u[i]);
         }
     }
     if (!grid_sync(gb, gridDim.x, budget)) return;
@@ -3993,9 +4020,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_bconvert(const SnapDesc<TS> *__
     const size_t cnt = (size_t)d.g.n * nf;
     const size_t tid = (size_t)blockIdx.x * kThreads + threadIdx.y * TX + threadIdx.x;
     for (size_t i = tid; i < cnt; i += (size_t)gridDim.x * kThreads) {
-        double v = d.cells[i];
-        float hi = __double2float_rn(v);
-        d.U[i] = DF{hi, __double2float_rn(v - (double)hi)};
+        d.U[i] = df_split(d.cells[i]);
     }
 }
 
@@ -4146,8 +4171,8 @@ __global__ void k_batched_final(const SnapDesc<TS> *__restrict__ sd, int nf, dou
     double *out = cells[blockIdx.y];
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (size_t)gridDim.x * blockDim.x) {
-        DF v = in_x2 ? d.X2[i] : d.U[i];
-        out[i] = (double)v.hi + (double)v.lo;
+        const DF v = in_x2 ? d.X2[i] : d.U[i];
+        out[i] = df_join(v.hi, v.lo);
     }
 }
 
@@ -5547,8 +5572,10 @@ static cg_status diffuse_explicit(cg_mesh *m, int nf, double *cells, const cg_pa
 //
 // Whether it pays: in units of one sweep (16 B per cell) a call's own inner solves take
 // 2 (m - 1) per step and the predicted ones about half of that plus, per run, K recurrence
-// sweeps of 12 B and the combination (K + 1 vectors read, `len` written).  Measured at
-// 128^3, b = 2 dx: see launch site.
+// sweeps of 12 B and the combination (K + 1 vectors read, `len` written).  By that count two
+// steps cost as much either way and three are worth it; measured (whole diffusions, own
+// rounds -> expansion): 128^3, 3 steps, c = 0.025 0.436 -> 0.392 ms, c = 0.4 0.813 -> 0.749 ms;
+// 10 steps 1.10 -> 0.83 and 2.36 -> 1.78 ms; 32^3, 3 steps, c = 0.1 0.234 -> 0.196 ms.
 static void pred_build(PredPlan &pl) {
     const double ce = pl.scheme == CG_SCHEME_CRANK_NICOLSON ? 0.5 * pl.c : pl.c;
     const double mu_max = (pl.lmax - 1.0) / ce;
@@ -5886,7 +5913,8 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     // the adaptive host-driven loop below.)
     if constexpr (kDF) {
         // rounds per step: remembered for this signature, else an a-priori start (two
-        // FP32 inner solves of ~1e-6 each reach 1e-13 from a residual below |b|)
+        // FP32 inner solves of ~1e-6 each, the first of them the shared expansion's where
+        // it runs, reach 1e-13 from a residual below |b|)
         const int max_r = p->max_rounds > 0 ? p->max_rounds : 12;
         // (BF16 rounds gain about 2.5 digits each: five from r = c L u, three and the shared
         // expansion's from there)
