@@ -939,6 +939,9 @@ def extras():
 # (5), A p = dg p - ce s (3) and p.Ap (2); its second pass the sum and A p again (8),
 # x += alpha p, r -= alpha Ap and r.r (6): 26.  A step's initial residual c L x with
 # r.r and b.b: 12.  Bytes per cell and iteration: 24 (pass 1) + 40 (pass 2).
+# These are the operations of the method with A p formed twice; where the workspace holds
+# A p the second pass reads it (18 operations, 32 + 48 bytes), so the units' own rate is
+# 18/26 of the figure reported.
 FP64_FLOPS_PER_ITER, FP64_FLOPS_PER_INIT, FP64_BYTES_PER_ITER = 26, 12, 64
 FP64_NOMINAL_TFLOPS = 1.25
 
