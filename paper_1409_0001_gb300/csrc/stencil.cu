@@ -1022,9 +1022,12 @@ __global__ void k_from_f32(size_t n, const float *__restrict__ v, double *__rest
 // a block of 32 lanes x 32 rows holds a tile of 128 columns x 32 rows.  x neighbours
 // inside a thread's four cells are in registers, across lanes they come by shuffle; y
 // neighbours come from the per-level shared plane as 128-bit loads; each thread stages
-// its own four input cells of a plane with one 16-byte cp.async.  The tile keeps a fixed
-// halo of four columns on each side (so every tile starts 16-byte aligned, whatever K)
-// and K rows above and below; it writes the inner 120 x (32 - 2K) columns.  Every cell
+// its own four input cells of a plane with one 16-byte cp.async.  Between tiles there is a
+// fixed halo of four columns (so every tile starts 16-byte aligned, whatever K) and of K
+// rows; a tile at a wall starts or ends there without one, so that a tile writes 120, 124
+// or 128 columns and 32 - 2K, 32 - K or 32 rows: 128 columns take one tile, not two.
+// Beyond a tile's edge the x and y neighbours read zero (a zero row precedes every shared
+// plane), which is the wall's value, and in a halo never reaches a written cell.  Every cell
 // update is k_explicit_tb's expression in the same order, so the two kernels agree bit
 // for bit.
 // Issue-bound, so the instructions per cell and step decide: sums and updates run on cell
@@ -1032,13 +1035,17 @@ __global__ void k_from_f32(size_t n, const float *__restrict__ v, double *__rest
 // unrolled by the ring's four slots (slots, parities and shared addresses are constants,
 // and the two queue planes of a level change roles by name), the plane to stage is
 // carried along instead of wrapped anew, and the z walls' face counts are off the common
-// path.  Three steps per launch on 256 x 128 x 128 with two fields: 51.7 -> 39.5 us; 40
-// steps on 512 x 256 x 256 take 1.92 ms (2.33 before), on 128^3 0.36 ms (0.44).
+// path: 41 -> 26 instructions per cell and step, 143 -> 110 us per launch of three steps on
+// 512 x 256 x 256; what bounds it now is the shared planes' traffic (70 % of the LSU data
+// pipe) beside issue (62 %).  40 steps, three per launch: 256 x 128 x 128 with two fields
+// 0.88 -> 0.71 ms, 512 x 256 x 256 2.33 -> 1.87, 128^3 0.44 -> 0.36 and, with one tile over
+// the 128 columns, 0.31.
 constexpr int kE4W = 128, kE4H = 32, kE4OX = kE4W - 8;
+constexpr int kE4P = kE4H + 1;   // rows of a level's shared plane: a zero row, then the tile's
 constexpr dim3 kE4Block(32, kE4H);
 
 __host__ __device__ constexpr size_t explicit_tb4_smem(int K) {
-    return (size_t)(kEStages + 2 * K) * kE4H * kE4W * sizeof(float);
+    return ((size_t)kEStages * kE4H + (size_t)2 * K * kE4P + 1) * kE4W * sizeof(float);
 }
 
 template <int K>
@@ -1046,9 +1053,10 @@ __global__ void __launch_bounds__(1024, 1) k_explicit_tb4(Geo g, int zlen, int n
                                                           const float *__restrict__ uin_all,
                                                           float *__restrict__ uout_all) {
     extern __shared__ float4 tb4_smem[];
-    // stage[slot][row][128]; buf[level][parity][row][128], levels 0..K-1
+    // stage[slot][row][128]; buf[level][parity][1 + row][128], levels 0..K-1, row 0 zero (and
+    // a last zero row after the last plane)
     float(*stage)[kE4H][kE4W] = reinterpret_cast<float(*)[kE4H][kE4W]>(tb4_smem);
-    float(*buf)[2][kE4H][kE4W] = reinterpret_cast<float(*)[2][kE4H][kE4W]>(&stage[kEStages][0][0]);
+    float(*buf)[2][kE4P][kE4W] = reinterpret_cast<float(*)[2][kE4P][kE4W]>(&stage[kEStages][0][0]);
     constexpr int OY = kE4H - 2 * K;
     const int lane = threadIdx.x, w = threadIdx.y;
     const int f = blockIdx.z / nzc, zc = blockIdx.z - f * nzc;
@@ -1058,8 +1066,8 @@ __global__ void __launch_bounds__(1024, 1) k_explicit_tb4(Geo g, int zlen, int n
     float *uout = uout_all + (size_t)f * g.n;
 
     // this thread's four cells: columns 4 lane .. 4 lane + 3 of row w
-    const int xa = blockIdx.x * kE4OX - 4 + 4 * lane;   // first column (a multiple of 4)
-    const int y = blockIdx.y * OY - K + w;
+    const int xa = (int)blockIdx.x * kE4OX - (px ? 4 : 0) + 4 * lane;   // first column (a multiple of 4)
+    const int y = (int)blockIdx.y * OY - (py ? K : 0) + w;
     const bool ey = py || (y >= 0 && y < g.ny);
     const bool ex = px || (xa >= 0 && xa < g.nx);        // the four cells share it (nx % 4 == 0)
     const int gx = px ? wrap_coord(xa, g.nx) : min(max(xa, 0), g.nx - 4);
@@ -1073,10 +1081,15 @@ __global__ void __launch_bounds__(1024, 1) k_explicit_tb4(Geo g, int zlen, int n
     const float2 cm = (ex && ey) ? make_float2(c, c) : make_float2(0.f, 0.f);
     const float2 nm01 = make_float2(-(nxy[0] + 2.f), -(nxy[1] + 2.f));   // - faces, away from the z walls
     const float2 nm23 = make_float2(-(nxy[2] + 2.f), -(nxy[3] + 2.f));
-    const bool wr = lane >= 1 && lane <= 30 && xa >= 0 && xa < g.nx && w >= K && w < kE4H - K && y >= 0 &&
-                    y < g.ny;   // columns 4 .. 123 of the tile, rows K .. 31 - K
+    // written: the mesh's cells that no other tile writes.  At a wall the first tile writes
+    // from its first column and row, the last one to the mesh's end.
+    const bool wx = xa >= 0 && xa < g.nx && (lane >= 1 || (!px && blockIdx.x == 0)) &&
+                    (lane <= 30 || (!px && blockIdx.x == gridDim.x - 1));
+    const bool wy = y >= 0 && y < g.ny && (w >= K || (!py && blockIdx.y == 0)) &&
+                    (w < kE4H - K || (!py && blockIdx.y == gridDim.y - 1));
+    const bool wr = wx && wy;
     // the level buffers start at zero, so every value a cell ever reads is finite
-    for (int k = threadIdx.y * 32 + threadIdx.x; k < K * 2 * kE4H * kE4W; k += 1024)
+    for (int k = threadIdx.y * 32 + threadIdx.x; k < (K * 2 * kE4P + 1) * kE4W; k += 1024)
         (&buf[0][0][0][0])[k] = 0.f;
     __syncthreads();
     float4 Q[K][2];   // planes q-1 and q of the level below K; the planes of the march alternate
@@ -1102,11 +1115,7 @@ __global__ void __launch_bounds__(1024, 1) k_explicit_tb4(Geo g, int zlen, int n
         if (++si >= g.nz) si = pz ? 0 : g.nz - 1;
     };
     float *out = uout + (ptrdiff_t)(p_begin - K) * g.nxy + rowoff;   // level K's plane at p
-    float(*const own)[2][kE4H][kE4W] = reinterpret_cast<float(*)[2][kE4H][kE4W]>(&buf[0][0][w][4 * lane]);
-    float(*const above)[2][kE4H][kE4W] =
-        reinterpret_cast<float(*)[2][kE4H][kE4W]>(&buf[0][0][max(w - 1, 0)][4 * lane]);
-    float(*const below)[2][kE4H][kE4W] =
-        reinterpret_cast<float(*)[2][kE4H][kE4W]>(&buf[0][0][min(w + 1, kE4H - 1)][4 * lane]);
+    float(*const own)[2][kE4P][kE4W] = reinterpret_cast<float(*)[2][kE4P][kE4W]>(&buf[0][0][1 + w][4 * lane]);
 #pragma unroll
     for (int d = 0; d < kEStages - 1; ++d) stage_plane(d);
     for (int p0 = p_begin; p0 < p_end; p0 += kEStages) {
@@ -1131,10 +1140,12 @@ __global__ void __launch_bounds__(1024, 1) k_explicit_tb4(Geo g, int zlen, int n
                         n23 = __fadd2_rn(n23, make_float2(a, a));
                     }
                     const float4 b = Q[t - 1][par ^ 1], za = Q[t - 1][par];
-                    const float4 up = *reinterpret_cast<const float4 *>(&above[t - 1][par ^ 1][0][0]);
-                    const float4 dn = *reinterpret_cast<const float4 *>(&below[t - 1][par ^ 1][0][0]);
-                    const float xl = __shfl_up_sync(0xffffffffu, b.w, 1);
-                    const float xr = __shfl_down_sync(0xffffffffu, b.x, 1);
+                    const float4 up = *reinterpret_cast<const float4 *>(&own[t - 1][par ^ 1][0][0] - kE4W);
+                    const float4 dn = *reinterpret_cast<const float4 *>(&own[t - 1][par ^ 1][0][0] + kE4W);
+                    float xl = __shfl_up_sync(0xffffffffu, b.w, 1);
+                    float xr = __shfl_down_sync(0xffffffffu, b.x, 1);
+                    if (lane == 0) xl = 0.f;
+                    if (lane == 31) xr = 0.f;
                     const float2 b01 = make_float2(b.x, b.y), b23 = make_float2(b.z, b.w);
                     float2 s01 = make_float2(__fadd_rn(xl, b.y), __fadd_rn(b.x, b.z));
                     float2 s23 = make_float2(__fadd_rn(b.y, b.w), __fadd_rn(b.z, xr));
@@ -5445,7 +5456,10 @@ static int explicit_zlen(const Geo &g, long long cols, long long slots, int kt) 
 static cg_status launch_explicit_tb4(const Geo &g, int nf, int kt, float c, const float *a, float *b,
                                      cudaStream_t st) {
     const int OY = kE4H - 2 * kt;
-    const int gx = (g.nx + kE4OX - 1) / kE4OX, gy = (g.ny + OY - 1) / OY;
+    // tiles per axis: at walls the first and the last tile need no halo outside
+    const bool px = g.per & 1, py = (g.per >> 1) & 1;
+    const int gx = px ? (g.nx + kE4OX - 1) / kE4OX : std::max(1, (g.nx - 8 + kE4OX - 1) / kE4OX);
+    const int gy = py ? (g.ny + OY - 1) / OY : std::max(1, (g.ny - 2 * kt + OY - 1) / OY);
     const size_t smem = explicit_tb4_smem(kt);
     const int per_sm = kt == 1 ? explicit_tb4_blocks_per_sm<1>(smem)
                      : kt == 2 ? explicit_tb4_blocks_per_sm<2>(smem)
