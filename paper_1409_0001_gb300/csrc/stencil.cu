@@ -30,6 +30,7 @@
 #include <mutex>
 #include <vector>
 
+#include "grid_stride.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
 
@@ -636,31 +637,31 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
     const double *p = pall + off, *q = qall + off;
     double *x = xall + off, *r = rall + off;
     double rr = 0.0;
-    const int step = gridDim.x * kThreads;
-    int k = blockIdx.x * kThreads + threadIdx.x;
-    for (; k + 3 * step < n; k += 4 * step) {   // four cells in flight
-        double pv[4], qv[4], xv[4], rv[4];
+    grid_stride<4>(
+        n, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads,
+        [&](int64_t k, int64_t step) {   // four cells in flight
+            double pv[4], qv[4], xv[4], rv[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            pv[j] = p[k + j * step];
-            qv[j] = q[k + j * step];
-            xv[j] = x[k + j * step];
-            rv[j] = r[k + j * step];
-        }
+            for (int j = 0; j < 4; ++j) {
+                pv[j] = p[k + j * step];
+                qv[j] = q[k + j * step];
+                xv[j] = x[k + j * step];
+                rv[j] = r[k + j * step];
+            }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            x[k + j * step] = fma(alpha, pv[j], xv[j]);
-            const double rk = fma(-alpha, qv[j], rv[j]);
-            r[k + j * step] = rk;
+            for (int j = 0; j < 4; ++j) {
+                x[k + j * step] = fma(alpha, pv[j], xv[j]);
+                const double rk = fma(-alpha, qv[j], rv[j]);
+                r[k + j * step] = rk;
+                rr = fma(rk, rk, rr);
+            }
+        },
+        [&](int64_t k) {
+            x[k] = fma(alpha, p[k], x[k]);
+            const double rk = fma(-alpha, q[k], r[k]);
+            r[k] = rk;
             rr = fma(rk, rk, rr);
-        }
-    }
-    for (; k < n; k += step) {
-        x[k] = fma(alpha, p[k], x[k]);
-        const double rk = fma(-alpha, q[k], r[k]);
-        r[k] = rk;
-        rr = fma(rk, rk, rr);
-    }
+        });
     double val = block_sum(rr);
     double *partials = partials_all + (size_t)f * 2 * nb;
     if (arrive(partials, 1, &val, blockIdx.x, gridDim.x, &sc[f].ticket)) {
@@ -4234,8 +4235,7 @@ __global__ void k_mass_batched(const SnapDesc<TS> *__restrict__ sd, int nf, doub
     if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
 
-// sum_k V_c,k u_k per field (1-D grid-stride; any mesh)
-// sum_k V_k u_k per field.  Few blocks of many cells each: a block's FP64 reduction and the
+// sum_k V_k u_k per field (any mesh).  Few blocks of many cells each: a block's FP64 reduction and the
 // last block's sum of the partials cost more than its cells on a small mesh (GB300 issues a
 // warp's FP64 instruction in 16 cycles).
 __global__ void k_mass(int n, const double *__restrict__ u_all, const double *__restrict__ vc,
@@ -4244,19 +4244,19 @@ __global__ void k_mass(int n, const double *__restrict__ u_all, const double *__
     const int f = blockIdx.y;
     const double *u = u_all + (size_t)f * n;
     double s = 0.0;
-    const int step = gridDim.x * kThreads;
-    int k = blockIdx.x * kThreads + threadIdx.x;
-    for (; k + 7 * (long long)step < n; k += 8 * step) {   // eight cells in flight
-        double x[8], v[8];
+    grid_stride<8>(
+        n, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads,
+        [&](int64_t k, int64_t step) {   // eight cells in flight
+            double x[8], v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            x[j] = u[k + j * step];
-            v[j] = vc ? vc[k + j * step] : vcu;
-        }
+            for (int j = 0; j < 8; ++j) {
+                x[j] = u[k + j * step];
+                v[j] = vc ? vc[k + j * step] : vcu;
+            }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s += v[j] * x[j];
-    }
-    for (; k < n; k += step) s += (vc ? vc[k] : vcu) * u[k];
+            for (int j = 0; j < 8; ++j) s += v[j] * x[j];
+        },
+        [&](int64_t k) { s += (vc ? vc[k] : vcu) * u[k]; });
     double v = block_sum(s);
     double *partials = partials_all + (size_t)f * gridDim.x;
     if (arrive(partials, 1, &v, blockIdx.x, gridDim.x, &tickets[f])) {
