@@ -71,11 +71,14 @@ struct BatchKey {
         tsize = 0, scheme = 0, phased = 0, pred = 0, np = 0;
     long long budget = 0;
     double tol2 = 0.0;
+    // the arena's layout: the launches hold addresses inside it
+    std::vector<size_t> layout;
     bool operator==(const BatchKey &o) const {
         return arena == o.arena && gen == o.gen && nsnap == o.nsnap && nf == o.nf &&
                nsteps == o.nsteps && R == o.R && mmax == o.mmax && nr == o.nr && nc == o.nc &&
                grid == o.grid && zlen == o.zlen && tsize == o.tsize && scheme == o.scheme &&
-               phased == o.phased && pred == o.pred && np == o.np && budget == o.budget && tol2 == o.tol2;
+               phased == o.phased && pred == o.pred && np == o.np && budget == o.budget && tol2 == o.tol2 &&
+               layout == o.layout;
     }
 };
 

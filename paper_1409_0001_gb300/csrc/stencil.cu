@@ -6548,13 +6548,20 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
     return CG_OK;
 }
 
-// The batch arena on the first mesh: descriptors | weights | items | partials | hist |
-// barrier | failure count | output pointers.
+// The batch arena on the first mesh: descriptors | items | partials | hist | barrier | failure
+// count | output pointers | masses | expansion items | Chebyshev weights | expansion
+// coefficients.  The last two differ in length between calls of one shape (they follow the
+// bandwidths) and are reached through the descriptors alone, so they come behind everything
+// whose address a captured launch holds.
 struct BatchArena {
     char *ab = nullptr;
     size_t o_desc = 0, o_om = 0, o_ri = 0, o_ci = 0, o_fi = 0, o_prr = 0, o_pbb = 0, o_hist = 0,
            o_gb = 0, o_bad = 0, o_out = 0, o_mass = 0, o_pi = 0, o_pc = 0, total = 0;
     size_t nh = 0;
+    // every offset that a captured launch holds
+    std::vector<size_t> offsets() const {
+        return {o_desc, o_ri, o_ci, o_fi, o_prr, o_pbb, o_hist, o_gb, o_bad, o_out, o_mass, o_pi};
+    }
 };
 
 template <class TS>
@@ -6562,8 +6569,7 @@ static BatchArena batch_layout(const BatchPlan<TS> &P, int nsnap, int nf, int ns
     BatchArena A;
     const size_t nr = P.ritems.size();
     A.o_desc = 0;
-    A.o_om = align_up(A.o_desc + P.descs.size() * sizeof(SnapDesc<TS>));
-    A.o_ri = align_up(A.o_om + P.omegas.size() * sizeof(float));
+    A.o_ri = align_up(A.o_desc + P.descs.size() * sizeof(SnapDesc<TS>));
     A.o_ci = align_up(A.o_ri + P.ritems.size() * sizeof(BItem));
     A.o_fi = align_up(A.o_ci + P.citems.size() * sizeof(BItem));
     A.o_prr = align_up(A.o_fi + P.first_item.size() * sizeof(int));
@@ -6575,7 +6581,8 @@ static BatchArena batch_layout(const BatchPlan<TS> &P, int nsnap, int nf, int ns
     A.o_out = align_up(A.o_bad + sizeof(unsigned int));
     A.o_mass = align_up(A.o_out + (size_t)nsnap * sizeof(double *));
     A.o_pi = align_up(A.o_mass + 2 * (size_t)nsnap * nf * 8);
-    A.o_pc = align_up(A.o_pi + P.pitems.size() * sizeof(BItem));
+    A.o_om = align_up(A.o_pi + P.pitems.size() * sizeof(BItem));
+    A.o_pc = align_up(A.o_om + P.omegas.size() * sizeof(float));
     A.total = align_up(A.o_pc + P.pcoef.size() * sizeof(float));
     return A;
 }
@@ -6917,6 +6924,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
         key.phased = Gx == 0 ? 1 : 0;
         key.pred = P.pred ? P.Kmax : 0;
         key.np = (int)P.pitems.size();
+        key.layout = A.offsets();
         key.tsize = (int)sizeof(TS);
         key.scheme = p->scheme;
         key.budget = budget;
