@@ -67,6 +67,11 @@ Sweep make_sweep_z(const Geo &g, int nf, int zlen) {
     return s;
 }
 
+// Whether a launch of zlen planes a block has a valid grid (blockIdx.z: chunks x fields).
+inline bool grid_z_fits(const Geo &g, int nf, int zlen) {
+    return (long long)((g.nz + zlen - 1) / zlen) * nf <= 65535;
+}
+
 Sweep make_sweep(const Geo &g, int nf) {
     Sweep s;
     int gx = (g.nx + TX - 1) / TX, gy = (g.ny + TY - 1) / TY;
@@ -4777,7 +4782,7 @@ inline Sweep mid_sweep(const Geo &g, int nf) {
     long long cost = -1;
     for (int nzc = 1; nzc <= g.nz; ++nzc) {
         const int z = (g.nz + nzc - 1) / nzc;
-        if (z > 16) continue;
+        if (z > 16 || !grid_z_fits(g, nf, z)) continue;
         const long long c = (cols * ((g.nz + z - 1) / z) + slots - 1) / slots * (z + 2);
         if (cost < 0 || c < cost) {
             cost = c;
@@ -5769,17 +5774,19 @@ static void launch_pred_combine(size_t n, size_t stride, const PredPlan &pl, int
 // renaming) in 64 registers, four blocks to an SM: 128^3 4.7 us (1 plane 6.0; 4 planes at three
 // blocks 5.5, 8 at two 7.0), 512 x 256 x 256 70.5 us = 5.7 TB/s (1 plane 96.9; 4 planes 73.4, 8 72.2).
 constexpr int kPredPlanes = 2;
+static int pred_sweep_planes(const Geo &g, int nf) {
+    return g.nx % 4 == 0 ? kPredPlanes : g.per ? make_sweep(g, nf).zlen : 4;
+}
 static void launch_pred_sweep(const Geo &g, int nf, float w, const float *t, const float *tp, float *tn,
                               cudaStream_t st) {
     const dim3 blk(TX, TY);
     const int gy = (g.ny + TY - 1) / TY;
+    const int zl = pred_sweep_planes(g, nf), nzc = (g.nz + zl - 1) / zl;
     if (g.nx % 4 == 0) {
-        const int nzc = (g.nz + kPredPlanes - 1) / kPredPlanes;
         const dim3 grid((g.nx + 4 * TX - 1) / (4 * TX), gy, nzc * nf);
         if (g.per) launch_chain(k_pred_v4<kPredPlanes, true>, grid, blk, st, g, kPredPlanes, nzc, w, t, tp, tn);
         else launch_chain(k_pred_v4<kPredPlanes, false>, grid, blk, st, g, kPredPlanes, nzc, w, t, tp, tn);
     } else {
-        const int zl = g.per ? make_sweep(g, nf).zlen : 4, nzc = (g.nz + zl - 1) / zl;
         const dim3 grid((g.nx + TX - 1) / TX, gy, nzc * nf);
         if (g.per) launch_chain(k_pred_any<true>, grid, blk, st, g, zl, nzc, w, t, tp, tn);
         else launch_chain(k_pred_any<false>, grid, blk, st, g, zl, nzc, w, t, tp, tn);
@@ -5877,8 +5884,10 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     const size_t vpd = align_up((size_t)n * nf * 4);   // one FP32 vector of the expansion
     if (kDF && !persistent) {
         const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, cheb_iters(lmax, 1e-6), c, lmax);
-        // (a round cap that the own rounds' start would exceed is refused as ever)
-        if (q.use && p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
+        // (a round cap that the own rounds' start would exceed is refused as ever; a mesh whose
+        // sweeps of two or four planes a block would exceed a grid's z extent keeps the own rounds)
+        if (q.use && grid_z_fits(g, nf, pred_sweep_planes(g, nf)) &&
+            p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
             (p->max_rounds <= 0 || p->max_rounds >= (sizeof(TS) == 2 ? 5 : 2)) &&
             m->ws_diffuse.ensure(base_b + (size_t)(q.maxK + 1 + pred_vectors(q.maxlen)) * vpd) == CG_OK)
             pred = &q;
