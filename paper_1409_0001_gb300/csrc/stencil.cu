@@ -4780,10 +4780,10 @@ inline Sweep mid_sweep(const Geo &g, int nf) {
     const long long cols = (long long)((g.nx + w - 1) / w) * ((g.ny + TY - 1) / TY) * nf;
     int best = 1;
     long long cost = -1;
-    for (int nzc = 1; nzc <= g.nz; ++nzc) {
-        const int z = (g.nz + nzc - 1) / nzc;
-        if (z > 16 || !grid_z_fits(g, nf, z)) continue;
-        const long long c = (cols * ((g.nz + z - 1) / z) + slots - 1) / slots * (z + 2);
+    for (int z = std::min(16, g.nz); z >= 1; --z) {
+        const int nzc = (g.nz + z - 1) / z;
+        if ((g.nz + nzc - 1) / nzc != z || !grid_z_fits(g, nf, z)) continue;   // (no even chunks of z)
+        const long long c = (cols * nzc + slots - 1) / slots * (z + 2);
         if (cost < 0 || c < cost) {
             cost = c;
             best = z;
