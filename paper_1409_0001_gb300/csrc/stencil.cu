@@ -697,14 +697,30 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
 // so the sums are the same bits in every block and every run.  (Partials tagged with the
 // sum's number and polled by every block, which needs no arrival counter, took 2 us more
 // at 32^3: 152 blocks polling 152 slots.)
-struct CoopBar {
+// Fields are independent, so several run at a time: the launch's blocks form groups of
+// `blocks`, as many as the SMs hold (a block of 128 threads takes a quarter of an SM's
+// registers), each with its own barrier and partial sums; group q solves fields q, q + groups,
+// .. and the groups meet once per step.  A field's block layout, and with it its bits, do not
+// depend on how many there are.  (One field after the other, 8^3 x 8 fields took 12.7 ms a
+// call and 32^3 x 5 fields 10.9, against 5.7 and 7.4 in the two-launch form, which runs all
+// fields in one launch; in groups 1.8 and 5.2.)
+struct __align__(128) CoopBar {   // a group's; the last one is the whole launch's
     unsigned int count;
     int err;
+    int failed[2];   // a field of an even / odd step did not converge (the last one's)
 };
 constexpr int kCoopMaxC = 12;    // cells per thread: 6 C registers of state within 128
 
-// Arrival number `target / gridDim.x` of every block; bounded like grid_sync.
-__device__ __forceinline__ bool coop_sync(CoopBar *gb, unsigned target, long long budget) {
+// One group's place in the launch.
+struct CoopGroup {
+    int id, count, block, blocks;   // the group, of how many; this block's number in it, of how many
+    CoopBar *bars;                  // every group's, then the whole launch's
+};
+
+// Arrival of every block that counts on bar b, `target` in all; bounded like grid_sync.  A wait
+// that gives up raises every bar's err, so that no other block waits on.
+__device__ __forceinline__ bool coop_sync(const CoopGroup &cg, int b, unsigned target, long long budget) {
+    CoopBar *gb = cg.bars + b;
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -717,7 +733,7 @@ __device__ __forceinline__ bool coop_sync(CoopBar *gb, unsigned target, long lon
             if ((int)(v - target) >= 0) break;
             if (*(volatile int *)&gb->err) { ok = 0; break; }
             if (clock64() - t0 > budget) {
-                atomicExch(&gb->err, 1);
+                for (int q = 0; q <= cg.count; ++q) atomicExch(&cg.bars[q].err, 1);
                 ok = 0;
                 break;
             }
@@ -736,13 +752,13 @@ struct CoopScal {
     int done, breakdown;
 };
 
-// Grid-wide sums of a value (TWO: two values) per thread, the same bits in every block;
+// Group-wide sums of a value (TWO: two values) per thread, the same bits in every block;
 // fin(a, b) runs on thread 0 with the totals, and its writes to shared memory are visible
 // to the block on return.  The block sum goes through shared memory in full-warp
 // additions (36 FP64 warp instructions for 512 threads; a shuffle tree in every warp
 // would take 85).  NT: the block's threads (a multiple of 128).
 template <int NT, bool TWO, class Fin>
-__device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, CoopBar *gb, unsigned target,
+__device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, const CoopGroup &cg, unsigned target,
                                          long long budget, Fin fin) {
     __shared__ double2 sv[NT];
     const int t = threadIdx.x;
@@ -772,12 +788,12 @@ __device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, Coop
             v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
             if (TWO) v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
         }
-        if (t == 0) __stcg(&part[blockIdx.x], v);
+        if (t == 0) __stcg(&part[cg.block], v);
     }
-    if (!coop_sync(gb, target, budget)) return false;
+    if (!coop_sync(cg, cg.id, target, budget)) return false;
     if (t < 32) {
         double2 v = make_double2(0.0, 0.0);
-        for (int i = t; i < (int)gridDim.x; i += 32) {
+        for (int i = t; i < cg.blocks; i += 32) {
             const double2 o = __ldcg(&part[i]);
             v.x += o.x;
             if (TWO) v.y += o.y;
@@ -793,23 +809,27 @@ __device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, Coop
     return true;
 }
 
-// cells (read only) -> X (the solution); V: the vector published for the
-// neighbours; part: 2 x gridDim.x partials (alternating); hist[s * nf + f].  A field's
-// iteration stops as in the two-launch form: converged, breakdown, or max_it.  After a
-// step in which a field did not converge nothing more runs.
+// cells (read only) -> X (the solution); V: per group (vstride apart) the vector published
+// for the neighbours; part: 2 x gridDim.x partials (alternating); hist[s * nf + f].  A
+// field's iteration stops as in the two-launch form: converged, breakdown, or max_it.  After
+// a step in which a field did not converge nothing more runs.
 template <int NT, int C>
 __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
-    Geo g, int per_block, double c, Coef64 cf, int scheme, int nf, int nsteps, int max_it, double tol2,
-    const double *__restrict__ cells, double *X, double *V, double2 *part, Scal *__restrict__ hist,
-    CoopBar *gb, long long budget) {
+    Geo g, int blocks, int per_block, double c, Coef64 cf, int scheme, int nf, int nsteps, int max_it, double tol2,
+    const double *__restrict__ cells, double *X, double *V, size_t vstride, double2 *part,
+    Scal *__restrict__ hist, CoopBar *bars, long long budget) {
     __shared__ double sdg[8];
     __shared__ unsigned short face[C][NT];
     __shared__ CoopScal S;
     stage_table(sdg, cf.dg);
     __syncthreads();
     const int n = g.n, nx = g.nx, nxy = g.nxy;
-    const int k0 = blockIdx.x * per_block + threadIdx.x;
-    const int kend = min(n, (int)(blockIdx.x + 1) * per_block);
+    const int gid = (int)blockIdx.x / blocks;
+    const CoopGroup cg{gid, (int)gridDim.x / blocks, (int)blockIdx.x - gid * blocks, blocks, bars};
+    V += gid * vstride;
+    part += 2 * gid * blocks;
+    const int k0 = cg.block * per_block + threadIdx.x;
+    const int kend = min(n, (cg.block + 1) * per_block);
     // per cell: which neighbours lie across a wall (no neighbour) or a periodic face, two
     // bits per face (0: the adjacent cell, 1: none, 2: the other end of the axis)
 #pragma unroll
@@ -823,7 +843,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                 (y + 1 == g.ny ? wy : 0u) << 6 | (z == 0 ? wz : 0u) << 8 | (z + 1 == g.nz ? wz : 0u) << 10);
         }
     }
-    unsigned target = 0;
+    unsigned target = 0, target_all = 0;
     int par = 0;
     auto nb = [&](const double *v, int k, unsigned w, int step, int wrap) -> double {
         return w == 1u ? 0.0 : __ldcg(v + k + (w == 0u ? step : wrap));
@@ -838,7 +858,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
     };
     bool failed = false;
     for (int s = 0; s < nsteps && !failed; ++s) {
-        for (int f = 0; f < nf; ++f) {
+        for (int f = cg.id; f < nf; f += cg.count) {
             double *Xf = X + (size_t)f * n;
             const double *xin = s == 0 ? cells + (size_t)f * n : Xf;
             double x[C], r[C], p[C];
@@ -858,8 +878,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                     bb += bk * bk;
                 }
             }
-            target += gridDim.x;
-            if (!coop_sum<NT, true>(rr, bb, part + par * gridDim.x, gb, target, budget, [&](double RR, double BB) {
+            target += blocks;
+            if (!coop_sum<NT, true>(rr, bb, part + par * blocks, cg, target, budget, [&](double RR, double BB) {
                     S.rr = RR;
                     S.bb = BB;
                     S.stop = tol2 * BB;
@@ -880,8 +900,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                         __stcg(V + k, p[j]);
                     }
                 }
-                target += gridDim.x;
-                if (!coop_sync(gb, target, budget)) return;
+                target += blocks;
+                if (!coop_sync(cg, cg.id, target, budget)) return;
                 double ap[C];
                 double pap = 0.0;
 #pragma unroll
@@ -895,8 +915,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                         pap = fma(p[j], ap[j], pap);
                     }
                 }
-                target += gridDim.x;
-                if (!coop_sum<NT, false>(pap, 0.0, part + par * gridDim.x, gb, target, budget, [&](double PAP, double) {
+                target += blocks;
+                if (!coop_sum<NT, false>(pap, 0.0, part + par * blocks, cg, target, budget, [&](double PAP, double) {
                         S.breakdown = !(PAP > 0.0);
                         S.alpha = S.rr / PAP;
                     }))
@@ -911,8 +931,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                     r[j] = fma(-alpha, ap[j], r[j]);
                     rn = fma(r[j], r[j], rn);
                 }
-                target += gridDim.x;
-                if (!coop_sum<NT, false>(rn, 0.0, part + par * gridDim.x, gb, target, budget, [&](double RR, double) {
+                target += blocks;
+                if (!coop_sum<NT, false>(rn, 0.0, part + par * blocks, cg, target, budget, [&](double RR, double) {
                         S.beta = RR / S.rr;
                         S.rr = RR;
                         S.done = RR <= S.stop;
@@ -926,7 +946,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
                 const int k = k0 + j * NT;
                 if (k < kend) __stcg(Xf + k, x[j]);
             }
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (cg.block == 0 && threadIdx.x == 0) {
                 Scal &H = hist[(size_t)s * nf + f];
                 H.rr = S.rr;
                 H.bb = S.bb;
@@ -936,8 +956,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
             }
             if (S.breakdown ? S.rr > S.stop : !S.done) failed = true;
             // X is read by other blocks in the next step's first pass (and V rewritten)
-            target += gridDim.x;
-            if (!coop_sync(gb, target, budget)) return;
+            target += blocks;
+            if (!coop_sync(cg, cg.id, target, budget)) return;
+        }
+        if (cg.count > 1) {   // every group has finished the step; one that failed stops all
+            int *flag = &bars[cg.count].failed[s & 1];   // (alternating: read before it is set again)
+            if (failed && cg.block == 0 && threadIdx.x == 0) atomicExch(flag, 1);
+            target_all += gridDim.x;
+            if (!coop_sync(cg, cg.count, target_all, budget)) return;
+            failed = *(volatile int *)flag != 0;
         }
     }
 }
@@ -945,8 +972,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
 // The solution of k_cg_coop into the caller's array, unless a wait gave up (the caller's
 // field is then as it was, and the two-launch form solves it).
 __global__ void k_cg_coop_out(size_t n, const double *__restrict__ X, double *__restrict__ cells,
-                              const CoopBar *gb) {
-    if (gb->err) return;
+                              const CoopBar *bars) {
+    if (bars->err) return;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         cells[i] = X[i];
 }
@@ -5237,21 +5264,22 @@ cg_status field_mass_many(int nmesh, cg_mesh *const *ms, int nf, const double *c
 // registers; *solved stays false where it does not apply or a wait gave up, and the
 // caller's field is then untouched.
 template <int NT, int C>
-static cudaError_t launch_cg_coop(int grid, Geo g, int per_block, double c, Coef64 cf, int scheme, int nf,
-                                  int nsteps, int max_it, double tol2, const double *cells, double *X,
-                                  double *V, double2 *part, Scal *hist, CoopBar *gb, cudaStream_t st) {
+static cudaError_t launch_cg_coop(int groups, int blocks, Geo g, int per_block, double c, Coef64 cf, int scheme,
+                                  int nf, int nsteps, int max_it, double tol2, const double *cells, double *X,
+                                  double *V, size_t vstride, double2 *part, Scal *hist, CoopBar *bars,
+                                  cudaStream_t st) {
     long long budget = 2000000000LL;   // clock cycles a wait may take (about one second)
-    void *args[] = {&g, &per_block, &c, &cf, &scheme, &nf, &nsteps, &max_it, &tol2, &cells, &X, &V, &part,
-                    &hist, &gb, &budget};
-    return cudaLaunchCooperativeKernel((const void *)k_cg_coop<NT, C>, dim3(grid), dim3(NT), args, 0, st);
+    void *args[] = {&g, &blocks, &per_block, &c, &cf, &scheme, &nf, &nsteps, &max_it, &tol2, &cells, &X, &V,
+                    &vstride, &part, &hist, &bars, &budget};
+    return cudaLaunchCooperativeKernel((const void *)k_cg_coop<NT, C>, dim3(groups * blocks), dim3(NT), args, 0, st);
 }
 
 static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, const cg_params *p, double c,
                            const Coef64 &cf, cg_report *rep, cudaStream_t st, bool *solved) {
     const int n = g.n;
     // A block per SM, but at least 64 cells to a block (8^3 on 8 blocks: 7.5 us per iteration);
-    // up to 933,888 cells (512 threads of 12 on 152 SMs), where the cooperative form is still 2.2
-    // times as fast as the two-launch form (30.1 against 65.1 us at 96^3).  Small meshes take
+    // up to 12 cells for each of 512 threads on every SM (933,888 cells on 152 SMs), where the
+    // cooperative form is still twice as fast as the two-launch form (30.7 against 58.7 us at 96^3).  Small meshes take
     // blocks of fewer threads, so that the solves of several streams share the SMs: blocks of
     // 512 threads at any size ran six concurrent 32^3 calls one after another, 15.2 ms
     // against 8.6 with the two-launch form (now 6.0; 64^3 20.3 -> 16.2 ms).
@@ -5260,26 +5288,35 @@ static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, cons
     const int nt = per_block <= 128 * 4 ? 128 : per_block <= 256 * 8 ? 256 : 512;
     const int need = (per_block + nt - 1) / nt;
     if (need > kCoopMaxC) return CG_OK;
+    // Groups of fields: 512 / nt blocks to an SM (the kernel's launch bounds).  Many fields of a
+    // small mesh take so many turns of about 8.5 us an iteration that the two-launch form, one
+    // pair of launches for all of them, is the faster one: it costs about 24 us and, per million
+    // cells, 19 us more than the turns' arithmetic.  Measured per iteration, this form against
+    // that one: 16^3 x 16 fields 17.5 and 23.9 us, x 32 34.0 and 27.5; 32^3 x 8 23.4 and 29.6, x 16
+    // 46.4 and 42.8; 48^3 x 8 58.0 and 66.3, x 16 115 and 115; 64^3 x 16 170 and 209.
+    const int groups = std::min(nf, 512 / nt * num_sms() / grid), turns = (nf + groups - 1) / groups;
+    if (8.5 * turns > 24.0 + 1.9e-5 * nf * n) return CG_OK;
     const size_t vec = align_up((size_t)n * nf * 8), one = align_up((size_t)n * 8);
     const size_t hist_n = (size_t)p->nsteps * nf;
-    const size_t part_b = align_up((size_t)2 * grid * sizeof(double2));
-    if (hist_n > (1u << 20) || m->ws_diffuse.ensure(vec + one) != CG_OK ||
-        m->ws_small.ensure(4096 + part_b + 256 + hist_n * sizeof(Scal)) != CG_OK ||
-        m->h_small.ensure(4096 + 256 + hist_n * sizeof(Scal)) != CG_OK)
+    const size_t part_b = align_up((size_t)2 * groups * grid * sizeof(double2));
+    const size_t bars_b = align_up((size_t)(groups + 1) * sizeof(CoopBar));
+    if (hist_n > (1u << 20) || m->ws_diffuse.ensure(vec + groups * one) != CG_OK ||
+        m->ws_small.ensure(4096 + part_b + bars_b + hist_n * sizeof(Scal)) != CG_OK ||
+        m->h_small.ensure(4096 + bars_b + hist_n * sizeof(Scal)) != CG_OK)
         return CG_OK;
     double *X = m->ws_diffuse.as<double>(), *V = (double *)(m->ws_diffuse.as<char>() + vec);
     double2 *part = (double2 *)(m->ws_small.as<char>() + 4096);
-    CoopBar *gb = (CoopBar *)(m->ws_small.as<char>() + 4096 + part_b);
-    Scal *hist = (Scal *)((char *)gb + 256);
-    CGK_CUDA(cudaMemsetAsync(gb, 0, 256 + hist_n * sizeof(Scal), st));
+    CoopBar *bars = (CoopBar *)(m->ws_small.as<char>() + 4096 + part_b);
+    Scal *hist = (Scal *)((char *)bars + bars_b);
+    CGK_CUDA(cudaMemsetAsync(bars, 0, bars_b + hist_n * sizeof(Scal), st));
     // the two-launch form checks its iteration cap every eight iterations
     const int max_it = p->max_iter > 0x7ffffff0 ? 0x7ffffff0 : (p->max_iter + 7) / 8 * 8;
     const double tol2 = p->tol * p->tol;
     cudaError_t e = cudaSuccess;
 #define CGK_COOP(NT, C)                                                                                    \
     CGK_LAUNCH("cg64_coop", (double)n * nf * 16, st,                                                       \
-               e = launch_cg_coop<NT, C>(grid, g, per_block, c, cf, p->scheme, nf, p->nsteps, max_it, tol2,    \
-                                     cells, X, V, part, hist, gb, st))
+               e = launch_cg_coop<NT, C>(groups, grid, g, per_block, c, cf, p->scheme, nf, p->nsteps, max_it,  \
+                                     tol2, cells, X, V, one / 8, part, hist, bars, st))
     if (nt == 128) {
         if (need <= 1) CGK_COOP(128, 1);
         else if (need <= 2) CGK_COOP(128, 2);
@@ -5298,13 +5335,13 @@ static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, cons
     }
     CGK_LAUNCH("cg64_coop_out", (double)n * nf * 16, st,
                k_cg_coop_out<<<stencil_grid((int)std::min<size_t>((size_t)n * nf, 1u << 30)), kThreads, 0, st>>>(
-                   (size_t)n * nf, X, cells, gb));
+                   (size_t)n * nf, X, cells, bars));
     CGK_CUDA(cudaGetLastError());
     char *hb = m->h_small.as<char>() + 4096;
-    CGK_CUDA(cudaMemcpyAsync(hb, gb, 256 + hist_n * sizeof(Scal), cudaMemcpyDeviceToHost, st));
+    CGK_CUDA(cudaMemcpyAsync(hb, bars, bars_b + hist_n * sizeof(Scal), cudaMemcpyDeviceToHost, st));
     CGK_CUDA(cudaStreamSynchronize(st));
     if (((CoopBar *)hb)->err) return CG_OK;
-    const Scal *h = (const Scal *)(hb + 256);
+    const Scal *h = (const Scal *)(hb + bars_b);
     long long total_iters = 0;
     double worst = 0.0;
     int bad = -1;
