@@ -402,6 +402,10 @@ cg_status cg_profile_get(int i, char *name, int name_len, long long *launches, d
  * cg_set_workspace_limit: a process-wide cap on that total (0, the default: none); a
  * call that would grow a workspace beyond it returns CG_ENOMEM before allocating and
  * before writing any output, as a failed cudaMalloc does, and the library stays usable.
+ * Memory that a call can do without (the vectors of the expansion that serves the first
+ * rounds of precision modes 3 and 4, one vector of the FP64 solver) never makes a call
+ * fail: it is not taken where it would not fit, and what other meshes hold of it is freed
+ * when a call needs the room.
  * Lets a caller budget device memory, and tests the allocation-failure path without
  * exhausting a GPU.  CG_EINVAL for a negative limit. */
 cg_status cg_set_workspace_limit(long long bytes);

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <algorithm>
 #include <atomic>
+#include <condition_variable>
 #include <mutex>
 #include <new>
 #include <string>
@@ -39,32 +40,111 @@ cg_status cuda_fail(cudaError_t e, const char *what, const char *file, int line)
 static std::atomic<long long> g_ws_bytes{0};
 static std::atomic<long long> g_ws_limit{0};
 
-cg_status DevBuf::ensure(size_t n) {
-    if (n <= bytes) return CG_OK;
+// One attempt at a buffer of n bytes (and an eighth more); refused by the limit, the buffer
+// stays as it is.
+static cg_status try_grow(DevBuf &d, size_t n) {
     size_t want = n + n / 8;
     const long long lim = g_ws_limit.load();
-    if (lim > 0 && g_ws_bytes.load() - (long long)bytes + (long long)want > lim)
+    if (lim > 0 && g_ws_bytes.load() - (long long)d.bytes + (long long)want > lim)
         return fail(CG_ENOMEM,
                     "device workspace of %zu bytes refused: the library would hold %lld bytes, "
                     "above the limit of %lld (cg_set_workspace_limit)",
-                    want, g_ws_bytes.load() - (long long)bytes + (long long)want, lim);
-    if (p) {
-        cudaError_t e = cudaFree(p);
-        p = nullptr;
-        g_ws_bytes -= (long long)bytes;
-        bytes = 0;
+                    want, g_ws_bytes.load() - (long long)d.bytes + (long long)want, lim);
+    if (d.p) {
+        cudaError_t e = cudaFree(d.p);
+        d.p = nullptr;
+        g_ws_bytes -= (long long)d.bytes;
+        d.bytes = 0;
         if (e != cudaSuccess) return cuda_fail(e, "cudaFree", __FILE__, __LINE__);
     }
-    ++gen;
-    cudaError_t e = cudaMalloc(&p, want);
+    ++d.gen;
+    cudaError_t e = cudaMalloc(&d.p, want);
     if (e != cudaSuccess) {
-        p = nullptr;
+        d.p = nullptr;
         cudaGetLastError();
         return fail(CG_ENOMEM, "cudaMalloc of %zu bytes failed: %s", want, cudaGetErrorString(e));
     }
-    bytes = want;
+    d.bytes = want;
     g_ws_bytes += (long long)want;
     return CG_OK;
+}
+
+// The optional buffers that hold memory.
+static std::mutex g_opt_mu;
+static std::condition_variable g_opt_cv;
+static std::vector<OptBuf *> g_opt;
+static unsigned g_opt_epoch = 1;
+static thread_local int t_opt_held = 0;   // this thread's buffers in use
+
+// Frees every optional buffer not in use; where there is none, waits for one in use (unless this
+// thread holds one itself).  False: nothing was or will be freed.
+static bool opt_reclaim() {
+    std::unique_lock<std::mutex> lock(g_opt_mu);
+    for (;;) {
+        bool freed = false, used = false;
+        for (OptBuf *o : g_opt) {
+            if (!o->b.bytes) continue;
+            if (o->busy) {
+                used = true;
+                continue;
+            }
+            o->b.release();
+            freed = true;
+        }
+        if (freed) return true;
+        if (!used || t_opt_held > 0) return false;
+        g_opt_cv.wait(lock);
+    }
+}
+
+cg_status DevBuf::ensure(size_t n) {
+    if (n <= bytes) return CG_OK;
+    for (;;) {
+        const cg_status s = try_grow(*this, n);
+        if (s != CG_ENOMEM || !opt_reclaim()) return s;
+    }
+}
+
+bool OptBuf::known_refused(size_t n) {
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    return n > b.bytes && refused && epoch == g_opt_epoch && n >= refused;
+}
+
+bool OptBuf::acquire(size_t n) {
+    if (known_refused(n)) return false;
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    if (n > b.bytes && try_grow(b, n) != CG_OK) {
+        refused = n;
+        epoch = g_opt_epoch;
+        return false;
+    }
+    if (!listed) g_opt.push_back(this);
+    listed = busy = true;
+    ++t_opt_held;
+    return true;
+}
+
+void OptBuf::done() {
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    busy = false;
+    --t_opt_held;
+    g_opt_cv.notify_all();
+}
+
+void OptBuf::release() {
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    for (size_t i = 0; listed && i < g_opt.size(); ++i)
+        if (g_opt[i] == this) {
+            g_opt.erase(g_opt.begin() + (long)i);
+            break;
+        }
+    listed = false;
+    b.release();
+}
+
+void opt_epoch_bump() {
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    ++g_opt_epoch;
 }
 
 void DevBuf::release() {
@@ -318,6 +398,7 @@ long long cg_launch_count(void) { return g_launches.load(); }
 cg_status cg_set_workspace_limit(long long bytes) {
     if (bytes < 0) return fail(CG_EINVAL, "the workspace limit must be >= 0 (0: no limit)");
     g_ws_limit.store(bytes);
+    opt_epoch_bump();
     return CG_OK;
 }
 
@@ -457,12 +538,14 @@ cg_status cg_destroy_mesh(cg_mesh *m) {
     m->ws_locate.release();
     m->ws_sort.release();
     m->ws_diffuse.release();
+    m->ws_opt.release();
     m->ws_small.release();
     m->ws_stage.release();
     m->ws_shared_in.release();
     m->ws_shared_dep.release();
     m->ws_order.release();
     m->ws_batch.release();
+    opt_epoch_bump();
     m->h_small.release();
     for (auto &e : m->graphs) graph_release(e);
     m->graphs.clear();

@@ -40,6 +40,33 @@ struct DevBuf {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
+// A device buffer that a call can do without (it then runs a slower form).  It never costs any
+// call its DevBufs: a DevBuf that is refused (the workspace limit, or the device is full) takes
+// back every OptBuf that no running call uses, of all meshes, waits for those in use, and
+// asks again.  So a call acquires its OptBuf after its last DevBuf, holds it through an OptUse,
+// and asks for no DevBuf while it does.  A refusal is remembered until a mesh is
+// destroyed or the workspace limit is set: a call that cannot have the memory does not ask,
+// and pay, for it each time.
+struct OptBuf {
+    DevBuf b;
+    bool busy = false, listed = false;   // guarded, as what follows, by one mutex for all
+    size_t refused = 0;                  // the smallest request refused at `epoch`
+    unsigned epoch = 0;
+    bool known_refused(size_t n);
+    bool acquire(size_t n);              // true: n bytes are this call's until done()
+    void done();
+    void release();
+    template <class T> T *as() const { return b.as<T>(); }
+};
+struct OptUse {
+    OptBuf *o = nullptr;
+    bool take(OptBuf &q, size_t n) { return q.acquire(n) ? (o = &q, true) : false; }
+    ~OptUse() {
+        if (o) o->done();
+    }
+};
+void opt_epoch_bump();   // memory may have become available: refusals are forgotten
+
 // A pinned host buffer that only grows (readback of scalars, flags, counters).
 struct HostBuf {
     void *p = nullptr;
@@ -90,7 +117,7 @@ struct GraphEntry {
     long long wait_budget = 0;      // resident waits' clock-cycle budget captured
     double T = 0, tol = 0;
     const void *cells = nullptr;
-    unsigned gen_diffuse = 0, gen_small = 0;
+    unsigned gen_diffuse = 0, gen_small = 0, gen_opt = 0;   // (gen_opt: with predicted only)
     bool profiled = false;
     bool predicted = false;         // first rounds from the shared expansion
     cudaGraphExec_t exec = nullptr;
@@ -170,6 +197,7 @@ struct cg_mesh {
     cgk::DevBuf ws_locate;   // cell ids / keys / values / counts
     cgk::DevBuf ws_sort;     // radix sort ping-pong and histograms
     cgk::DevBuf ws_diffuse;  // solver vectors
+    cgk::OptBuf ws_opt;      // the shared expansion's vectors, or A p of the FP64 solver
     cgk::DevBuf ws_small;    // scalars, partials, counters
     cgk::DevBuf ws_stage;    // device staging for the host-pointer entry point
     cgk::DevBuf ws_shared_in;  // host inputs copied once for several concurrent problems

@@ -5378,14 +5378,10 @@ static cg_status diffuse_fp64(cg_mesh *m, int nf, double *cells, const cg_params
     CGK_TRY(fp64_coop(m, g, nf, cells, p, c, cf, rep, st, &solved));
     if (solved) return CG_OK;
     const size_t vec = align_up((size_t)n * nf * 8);
-    // a fourth vector keeps A p between the passes; where the workspace may not grow to it
-    // the second pass forms A p again
-    const bool keep_q = m->ws_diffuse.ensure(4 * vec) == CG_OK;
-    if (!keep_q) CGK_TRY(m->ws_diffuse.ensure(3 * vec));
+    CGK_TRY(m->ws_diffuse.ensure(3 * vec));
     double *r = (double *)m->ws_diffuse.as<char>();
     double *P[2] = {(double *)(m->ws_diffuse.as<char>() + vec),
                     (double *)(m->ws_diffuse.as<char>() + 2 * vec)};
-    double *Q = keep_q ? (double *)(m->ws_diffuse.as<char>() + 3 * vec) : nullptr;
     const int ub = std::min(G, std::max(1, std::min((n + 4 * kThreads - 1) / (4 * kThreads), num_sms() * 8)));
     CGK_TRY(m->ws_small.ensure(4096 + align_up((size_t)nf * 2 * G * 8) + 64 * sizeof(Scal)));
     double *partials = (double *)(m->ws_small.as<char>() + 4096);
@@ -5393,6 +5389,10 @@ static cg_status diffuse_fp64(cg_mesh *m, int nf, double *cells, const cg_params
     CGK_CUDA(cudaMemsetAsync(sc, 0, nf * sizeof(Scal), st));
     CGK_TRY(m->h_small.ensure(4096 + 64 * sizeof(Scal)));
     Scal *hsc = (Scal *)(m->h_small.as<char>() + 4096);
+    // a fourth vector keeps A p between the passes; where it may not be held the second pass
+    // forms A p again
+    OptUse opt;
+    double *Q = opt.take(m->ws_opt, vec) ? m->ws_opt.as<double>() : nullptr;
     long long total_iters = 0;
     double worst = 0.0;
     const int chunk = 8;
@@ -5880,8 +5880,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     const double ce = cn ? 0.5 * c : c;
     const double tol2 = p->tol * p->tol;
     const Sweep sw = make_sweep(g, nf);
-    const Sweep sw_mid = mid_sweep(g, nf);
-    const int G = std::max(sw.nb, sw_mid.nb);
+    const int G = sw.nb;
     const dim3 blk(TX, TY);
     const Coef64 cf64 = coef64(ce);
     const Coef32 cf32 = coef32(ce);
@@ -5914,25 +5913,9 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
     // the resident inner solve (whole mesh in shared memory) where it fits; its flags and
     // faces follow the vectors
     const ResidentPlan rp = (persistent || m->per) ? ResidentPlan{} : plan_resident<TS>(g, nf, m_it);
-    // the shared expansion of the steps' first rounds (its vectors follow the resident
-    // solve's), where it pays, nothing caps the iterations, and its vectors may be held
-    const PredPlan *pred = nullptr;
-    const size_t base_b = 4 * v64 + 5 * vts + align_up(rp.ok ? rp.ws_bytes : 0);
-    const size_t vpd = align_up((size_t)n * nf * 4);   // one FP32 vector of the expansion
-    if (kDF && !persistent) {
-        const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, cheb_iters(lmax, 1e-6), c, lmax);
-        // (a round cap that the own rounds' start would exceed is refused as ever; a mesh whose
-        // sweeps of two or four planes a block would exceed a grid's z extent keeps the own rounds)
-        if (q.use && grid_z_fits(g, nf, pred_sweep_planes(g, nf)) &&
-            p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
-            (p->max_rounds <= 0 || p->max_rounds >= (sizeof(TS) == 2 ? 5 : 2)) &&
-            m->ws_diffuse.ensure(base_b + (size_t)(q.maxK + 1 + pred_vectors(q.maxlen)) * vpd) == CG_OK)
-            pred = &q;
-    }
-    if (!pred) CGK_TRY(m->ws_diffuse.ensure(base_b));
+    CGK_TRY(m->ws_diffuse.ensure(4 * v64 + 5 * vts + (rp.ok ? rp.ws_bytes : 0)));
     char *wb = m->ws_diffuse.as<char>();
     char *rws = wb + 4 * v64 + 5 * vts;
-    float *PT = (float *)(wb + base_b), *PD = pred ? PT + (size_t)(pred->maxK + 1) * (vpd / 4) : nullptr;
     XT *X1 = (XT *)wb, *X2 = (XT *)(wb + v64), *B = (XT *)(wb + 2 * v64), *X0 = (XT *)(wb + 3 * v64);
     TS *R = (TS *)(wb + 4 * v64), *Ya = (TS *)(wb + 4 * v64 + vts), *Yb = (TS *)(wb + 4 * v64 + 2 * vts);
     // two more iterate buffers for two-iterations-per-launch sweeps
@@ -5952,6 +5935,31 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                       hist_n * sizeof(RefScal))));
     RefScal *hsc = (RefScal *)(m->h_small.as<char>() + 4096);
     GridBar *hgb = (GridBar *)((char *)hsc + 64 * sizeof(RefScal));
+    // the shared expansion of the steps' first rounds, where it pays, nothing caps the
+    // iterations, and its vectors may be held: T_k, the increments, the merged pass's partials
+    const PredPlan *pred = nullptr;
+    const size_t vpd = align_up((size_t)n * nf * 4);   // one FP32 vector of the expansion
+    Sweep sw_mid = sw;
+    OptUse opt;
+    float *PT = nullptr, *PD = nullptr;
+    double *mid_part = nullptr;
+    if (kDF && !persistent) {
+        const PredPlan &q = pred_plan(m, p->scheme, p->nsteps, cheb_iters(lmax, 1e-6), c, lmax);
+        // (a round cap that the own rounds' start would exceed is refused as ever; a mesh whose
+        // sweeps of two or four planes a block would exceed a grid's z extent keeps the own rounds)
+        if (q.use && grid_z_fits(g, nf, pred_sweep_planes(g, nf)) &&
+            p->max_iter >= std::max(q.maxm, q.maxK) && q.maxm <= kResidentMaxIters &&
+            (p->max_rounds <= 0 || p->max_rounds >= (sizeof(TS) == 2 ? 5 : 2))) {
+            sw_mid = mid_sweep(g, nf);
+            const size_t nt = (size_t)(q.maxK + 1), nd = (size_t)pred_vectors(q.maxlen);
+            if (opt.take(m->ws_opt, (nt + nd) * vpd + (size_t)nf * 2 * sw_mid.nb * 8)) {
+                pred = &q;
+                PT = m->ws_opt.as<float>();
+                PD = PT + nt * (vpd / 4);
+                mid_part = (double *)(PD + nd * (vpd / 4));
+            }
+        }
+    }
 
     int cheb_code = p->sweep_shape;
     bool resident = false;
@@ -6031,7 +6039,8 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                     ++it;
                     continue;
                 }
-                if (it->gen_diffuse != m->ws_diffuse.gen || it->gen_small != m->ws_small.gen) {
+                if (it->gen_diffuse != m->ws_diffuse.gen || it->gen_small != m->ws_small.gen ||
+                    (it->predicted && it->gen_opt != m->ws_opt.b.gen)) {
                     graph_release(*it);
                     it = m->graphs.erase(it);
                     continue;
@@ -6060,6 +6069,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 e.cells = cells;
                 e.gen_diffuse = m->ws_diffuse.gen;
                 e.gen_small = m->ws_small.gen;
+                e.gen_opt = m->ws_opt.b.gen;
                 e.profiled = prof;
                 e.predicted = pred != nullptr;
                 e.code = shape_used;
@@ -6170,7 +6180,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                                  (const float *)yc,
                                                                  merged_in ? e0 + vpd / 4 : nullptr, (const DF *)bp_,
                                                                  (DF *)xn, (DF *)B, (float *)R_, (float *)y1,
-                                                                 (float)gamma, partials, slot, slot + nf, cs));
+                                                                 (float)gamma, mid_part, slot, slot + nf, cs));
                                     xc = xn;
                                     break;
                                 }
