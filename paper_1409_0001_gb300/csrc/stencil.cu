@@ -6479,6 +6479,7 @@ struct BatchPlan {
     std::vector<BItem> pitems;     // the shared expansion's sweeps (one field)
     std::vector<float> pcoef;
     std::vector<size_t> pc_off;
+    std::vector<size_t> opt_bytes; // the expansion's vectors, per snapshot
     bool pred = false;
     int Kmax = 0;
     std::vector<int> first_item;   // per (snapshot, field), into ritems
@@ -6496,6 +6497,7 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
     P.descs.resize((size_t)nsnap);
     P.omega_off.resize((size_t)nsnap);
     P.pc_off.resize((size_t)nsnap);
+    P.opt_bytes.resize((size_t)nsnap);
     // the shared expansion serves the batch where it pays for every snapshot: FP32 inner
     // storage, one run of steps, rows the flat-plane engine takes
     P.pred = sizeof(TS) == 4 && want_pred && p->nsteps <= kPredMaxSteps;
@@ -6559,8 +6561,7 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         const size_t vts = align_up((size_t)m->nz * d.pts * nf * sizeof(TS));
         const size_t t1 = align_up((size_t)m->nz * d.pts * 4);
         if (pl) {
-            if (m->ws_diffuse.ensure(4 * v64 + 3 * vts + (pl->maxK + 1) * t1 + p->nsteps * vts) != CG_OK)
-                return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, P);
+            P.opt_bytes[s] = p->nsteps * vts + (pl->maxK + 1) * t1;
             d.K = pl->K[0];
             d.w = (float)(2.0 * ce / (lmax - 1.0));
             P.Kmax = std::max(P.Kmax, d.K);
@@ -6571,8 +6572,6 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         }
         CGK_TRY(m->ws_diffuse.ensure(4 * v64 + 3 * vts));
         char *wb = m->ws_diffuse.as<char>();
-        d.D = (float *)(wb + 4 * v64 + 3 * vts);
-        d.T = d.D + (size_t)m->nz * d.pts * nf * p->nsteps;
         d.U = (DF *)wb;
         d.X1 = (DF *)(wb + v64);
         d.X2 = (DF *)(wb + 2 * v64);
@@ -6602,6 +6601,31 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
     }
     P.first_item.push_back((int)P.ritems.size());
     return CG_OK;
+}
+
+// The expansions' vectors of every snapshot, each in its mesh's optional buffer; false, and
+// nothing more held than before, where one is refused.
+template <class TS>
+static bool batch_take(BatchPlan<TS> &P, int nsnap, cg_mesh *const *meshes, int nf, int nsteps,
+                       std::vector<OptUse> &opt) {
+    std::vector<char> grown((size_t)nsnap, 0);
+    for (int s = 0; s < nsnap; ++s) {
+        OptBuf &o = meshes[s]->ws_opt;
+        const unsigned gen = o.b.gen;
+        if (!opt[s].take(o, P.opt_bytes[s])) {
+            for (int q = 0; q < s; ++q) {
+                opt[q].o->done();
+                if (grown[q]) opt[q].o->release();
+                opt[q].o = nullptr;
+            }
+            return false;
+        }
+        grown[s] = o.b.gen != gen;
+        SnapDesc<TS> &d = P.descs[s];
+        d.D = o.as<float>();
+        d.T = d.D + (size_t)d.g.nz * d.pts * nf * nsteps;
+    }
+    return true;
 }
 
 // The batch arena on the first mesh: descriptors | items | partials | hist | barrier | failure
@@ -6918,14 +6942,26 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
     const int zlen = code % kPhasedCode;
     const int Gx = code >= kPhasedCode ? 0 : G;
     if (zlen < 1) return fail(CG_EINVAL, "cg_diffuse_batched: bad sweep_shape %d", code);
+    // the plan's needed memory first, then the expansions' vectors; where those are refused,
+    // the plan without them
     BatchPlan<TS> P;
-    CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, p->max_rounds <= 0 || p->max_rounds >= 2, P));
-    BatchArena A = batch_layout(P, nsnap, nf, p->nsteps);
-    CGK_TRY(m0->ws_batch.ensure(A.total));
-    CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
-    const size_t nh = A.nh;
+    BatchArena A;
+    std::vector<OptUse> opt((size_t)nsnap);
+    const size_t nh = (size_t)p->nsteps * nsnap * nf;
     const size_t nm = (size_t)nsnap * nf;   // masses per snapshot-field, before and after
     CGK_TRY(m0->h_small.ensure(4096 + nh * sizeof(double2) + 64 + 2 * nm * 8));
+    for (bool want = p->max_rounds <= 0 || p->max_rounds >= 2;; want = false) {
+        CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, want, P));
+        bool refused = false;   // (before, and nothing has changed since)
+        for (int s = 0; s < nsnap; ++s)
+            refused = refused || (P.pred && meshes[s]->ws_opt.known_refused(P.opt_bytes[s]));
+        if (refused) continue;
+        A = batch_layout(P, nsnap, nf, p->nsteps);
+        const cg_status s = m0->ws_batch.ensure(A.total);
+        if (!P.pred) CGK_TRY(s);
+        if (!P.pred || (s == CG_OK && batch_take(P, nsnap, meshes, nf, p->nsteps, opt))) break;
+    }
+    CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
     double2 *hh = (double2 *)(m0->h_small.as<char>() + 4096);
     GridBar *hgb = (GridBar *)(hh + nh);
     double *hmass = (double *)(m0->h_small.as<char>() + 4096 + nh * sizeof(double2) + 64);

@@ -141,3 +141,50 @@ def test_fp64_beyond_the_cooperative_size(cg):
     assert near(x, y, u)
     mesh.close()
     a.close()
+
+
+def test_a_batch_under_its_needed_size(cg):
+    """Snapshots of which the first is the largest; one round a step, which no step ends
+    with, never takes the expansion: its workspace is what the batch needs."""
+    import torch
+    rng = np.random.default_rng(6)
+    dims = [(80, 72, 64), (40, 30, 33), (64, 64, 60), (20, 21, 22), (90, 50, 40)]
+    us = [torch.from_numpy(rng.random((2, a * b * c))).cuda() for a, b, c in dims]
+    held = cg.workspace_bytes()
+
+    def run(meshes, **kw):
+        x = [u.clone() for u in us]
+        _, rep = cg.diffuse_batched(meshes, x, cg.Params(nsteps=6, precision=3, sweep_shape=508, **kw),
+                                    bandwidths=[2.5] * len(dims), report=True)
+        return x, rep
+
+    def meshes_of():
+        return [cg.StructuredMesh(d, (0, 0, 0), 1.0) for d in dims]
+
+    meshes = meshes_of()
+    with pytest.raises(cg.CGError):
+        run(meshes, max_rounds=1)
+    plain = cg.workspace_bytes() - held
+    full, rep_full = run(meshes)
+    extra = cg.workspace_bytes() - held - plain
+    for m in meshes:
+        m.close()
+    assert extra > 0
+    for room in (0, extra // 3):              # none for the expansion; some, not enough
+        cg.set_workspace_limit(held + plain + room)
+        meshes = meshes_of()
+        sizes = []
+        for _ in range(3):
+            got, rep = run(meshes)
+            sizes.append(cg.workspace_bytes() - held)
+            assert rep["iters"] > rep_full["iters"]
+            for a, b, u in zip(got, full, us):
+                assert near(a, b, u)
+        assert sizes[0] == sizes[1] == sizes[2] <= plain + room
+        cg.set_workspace_limit(0)
+        got, rep = run(meshes)
+        assert rep["iters"] == rep_full["iters"]
+        assert all(bool((a == b).all()) for a, b in zip(got, full))
+        for m in meshes:
+            m.close()
+    assert cg.workspace_bytes() == held
