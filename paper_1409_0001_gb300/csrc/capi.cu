@@ -78,7 +78,7 @@ static thread_local int t_opt_held = 0;   // this thread's buffers in use
 
 // Frees every optional buffer not in use; where there is none, waits for one in use (unless this
 // thread holds one itself).  False: nothing was or will be freed.
-static bool opt_reclaim() {
+bool opt_reclaim() {
     std::unique_lock<std::mutex> lock(g_opt_mu);
     for (;;) {
         bool freed = false, used = false;

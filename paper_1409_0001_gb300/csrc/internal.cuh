@@ -66,6 +66,7 @@ struct OptUse {
     }
 };
 void opt_epoch_bump();   // memory may have become available: refusals are forgotten
+bool opt_reclaim();      // frees optional buffers; false: none was left to free
 
 // A pinned host buffer that only grows (readback of scalars, flags, counters).
 struct HostBuf {
