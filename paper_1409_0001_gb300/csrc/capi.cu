@@ -75,6 +75,7 @@ static std::condition_variable g_opt_cv;
 static std::vector<OptBuf *> g_opt;
 static unsigned g_opt_epoch = 1;
 static thread_local int t_opt_held = 0;   // this thread's buffers in use
+constexpr size_t kOptFreely = (size_t)64 << 20;   // no look at the device's memory up to here
 
 // Frees every optional buffer not in use; where there is none, waits for one in use (unless this
 // thread holds one itself).  False: nothing was or will be freed.
@@ -113,7 +114,15 @@ bool OptBuf::known_refused(size_t n) {
 bool OptBuf::acquire(size_t n) {
     if (known_refused(n)) return false;
     std::lock_guard<std::mutex> lock(g_opt_mu);
-    if (n > b.bytes && try_grow(b, n) != CG_OK) {
+    bool fits = true;
+    if (n > b.bytes && n > kOptFreely) {
+        size_t free_bytes = 0, total = 0, held = 0;
+        for (const OptBuf *o : g_opt) held += o->b.bytes;
+        fits = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess &&
+               opt_share(n + n / 8, b.bytes, held, free_bytes, total);
+        cudaGetLastError();
+    }
+    if (n > b.bytes && (!fits || try_grow(b, n) != CG_OK)) {
         refused = n;
         epoch = g_opt_epoch;
         return false;

@@ -43,7 +43,8 @@ struct DevBuf {
 // A device buffer that a call can do without (it then runs a slower form).  It never costs any
 // call its DevBufs: a DevBuf that is refused (the workspace limit, or the device is full) takes
 // back every OptBuf that no running call uses, of all meshes, waits for those in use, and
-// asks again.  So a call acquires its OptBuf after its last DevBuf, holds it through an OptUse,
+// asks again.  The caller's own allocations cannot do that, so what the OptBufs hold together stays
+// within a share of the device (opt_share).  So a call acquires its OptBuf after its last DevBuf, holds it through an OptUse,
 // and asks for no DevBuf while it does.  A refusal is remembered until a mesh is
 // destroyed or the workspace limit is set: a call that cannot have the memory does not ask,
 // and pay, for it each time.
@@ -65,6 +66,13 @@ struct OptUse {
         if (o) o->done();
     }
 };
+// Whether an optional buffer of `own` bytes may grow to `want` where all of them hold `held`: a
+// quarter of the device's memory for all, and a quarter of what is free for one request.
+// (The expansion of one field of 512 x 256 x 256, b = 4 dx, 40 steps, takes 6.3 GB, of four
+// fields of 512^3 101 GB beside 28 of needed vectors: that one keeps its own rounds.)
+inline bool opt_share(size_t want, size_t own, size_t held, size_t free_bytes, size_t total) {
+    return held - own + want <= total / 4 && want <= (free_bytes + own) / 4;
+}
 void opt_epoch_bump();   // memory may have become available: refusals are forgotten
 bool opt_reclaim();      // frees optional buffers; false: none was left to free
 
