@@ -222,6 +222,7 @@ struct cg_mesh {
     std::vector<cgk::PredPlan> preds;         // shared expansions per (scheme, steps, c)
     std::vector<std::pair<double, double>> spectrum;   // unstructured: lower end of the
                                                        // Chebyshev interval per dte
+    bool crowded = false;   // the last ordered deposition had a cell beyond the counting path
     cudaEvent_t dep_ev[3] = {nullptr, nullptr, nullptr};   // a deposition's phase times
     cudaEvent_t dif_ev[2] = {nullptr, nullptr};            // a diffusion's
     cudaStream_t capture_stream = nullptr;    // private stream used only for capture
@@ -333,9 +334,9 @@ cg_status hex_build(cg_mesh *m, int nx, int ny, int nz, const double *xf, const 
 void tet_release(cg_mesh *m);
 
 // Exclusive scan of n uint32 values (in and out may alias).  tmp needs
-// scan_tmp_words(n) words.
+// scan_tmp_words(n) words.  check (may be nullptr): see not_counting in deposit.cu.
 size_t scan_tmp_words(int64_t n);
 cg_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp,
-                             cudaStream_t st);
+                             cudaStream_t st, const unsigned long long *check = nullptr);
 
 }  // namespace cgk
