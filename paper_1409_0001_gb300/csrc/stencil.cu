@@ -5780,6 +5780,14 @@ static void pred_build(PredPlan &pl) {
     pl.use = cost <= 0.9 * own;
 }
 
+// A round's iterations where a step has R - 1 rounds of them.  The estimate is for one; a field that
+// decays faster than white noise (the highest frequencies alone) needs a second, and each
+// then has 0.65 of it: together (2 sg^(0.65 m))^2 instead of 2 sg^m, 4e-11 instead of 2e-8 at
+// c = 0.225.  (With 0.6 a checkerboard of 128^3 at
+// c = 0.8 took a third round.)  Checkerboards, 128^3, ten steps, two rounds of all m iterations
+// against this: c = 0.225 2.53 -> 2.00 ms, c = 0.4 3.20 -> 2.47 ms.
+static int pred_round_m(int m, int R) { return R > 2 ? std::max(2, (13 * m + 19) / 20) : m; }
+
 static const PredPlan &pred_plan(cg_mesh *m, int scheme, int nsteps, int m_it, double c, double lmax) {
     for (const PredPlan &q : m->preds)
         if (q.scheme == scheme && q.nsteps == nsteps && q.m_it == m_it && q.c == c && q.lmax == lmax) return q;
@@ -6122,7 +6130,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                                                                    (float)gamma, partials, slot, slot, cs));
                             if (!merged_in) xc = f1;
                         }
-                        const int mi = pred && sizeof(TS) == 4 ? pred->m[s2] : m_it;   // inner iterations of a round
+                        const int mi = pred && sizeof(TS) == 4 ? pred_round_m(pred->m[s2], R) : m_it;   // inner iterations of a round
                         for (int r = pred ? 1 : 0; r < R; ++r) {
                             TS *yc = y1, *yp = nullptr, *yo = (y1 == Ya) ? Yb : Ya;
                             double om = 1.0;
@@ -6265,13 +6273,14 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                     if (pred) {   // expansions, then per step one pass and R - 1 rounds
                         apps = (cn ? 1 : 0) + p->nsteps;
                         for (int K : pred->K) apps += K;
-                        for (int mi : pred->m) apps += (long long)(R - 1) * (sizeof(TS) == 4 ? mi : m_it);
+                        for (int mi : pred->m)
+                            apps += (long long)(R - 1) * (sizeof(TS) == 4 ? pred_round_m(mi, R) : m_it);
                     }
                     rep->iters = apps * nf;
                     rep->refine_rounds = (long long)p->nsteps * R;
                     rep->cell_updates = apps * nf * (long long)n;
                     rep->final_rel_residual = worst_g;
-                    rep->inner_iters_per_round = pred && sizeof(TS) == 4 ? pred->maxm : m_it;
+                    rep->inner_iters_per_round = pred && sizeof(TS) == 4 ? pred_round_m(pred->maxm, R) : m_it;
                     rep->sweep_shape_used = shape_used;
                 }
                 return CG_OK;
@@ -6490,7 +6499,7 @@ struct BatchPlan {
 template <class TS>
 static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *const *cells,
                             const cg_params *p, const double *bandwidths, int zlen,
-                            bool want_pred, BatchPlan<TS> &P) {
+                            bool want_pred, int R, BatchPlan<TS> &P) {
     const bool cn = p->scheme == CG_SCHEME_CRANK_NICOLSON;
     const double eps_inner = sizeof(TS) == 2 ? 2e-3 : 1e-6;
     P = BatchPlan<TS>();
@@ -6523,10 +6532,10 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         if (pl && (!pl->use || m->nx > kFlatMaxNx)) P.pred = false;
         if (!P.pred) pl = nullptr;
         if (want_pred && sizeof(TS) == 4 && !P.pred && s > 0 && P.Kmax > 0)   // start over without it
-            return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, P);
+            return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, R, P);
         // (counts are even here, so the estimate's last two iterations, below what the fields'
         // rounding leaves, are given up: 14 instead of 16 at b = 3 dx, errors as before)
-        if (pl) mi = std::max(mi, pl->maxm - 2);
+        if (pl) mi = R > 2 ? pred_round_m(pl->maxm, R) : std::max(mi, pl->maxm - 2);
         if (mi & 1) ++mi;
         d.m = mi;
         P.mmax = std::max(P.mmax, mi);
@@ -6879,7 +6888,7 @@ static cg_status batch_tune(int nsnap, cg_mesh *const *meshes, int nf, double *c
         const int z = code % kPhasedCode;
         const int g = code >= kPhasedCode ? 0 : G;
         BatchPlan<TS> P;
-        rc = batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, z, true, P);
+        rc = batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, z, true, 2, P);
         if (rc != CG_OK) break;
         BatchArena A = batch_layout(P, nsnap, nf, 1);
         rc = m0->ws_batch.ensure(A.total);
@@ -6942,6 +6951,21 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
     const int zlen = code % kPhasedCode;
     const int Gx = code >= kPhasedCode ? 0 : G;
     if (zlen < 1) return fail(CG_EINVAL, "cg_diffuse_batched: bad sweep_shape %d", code);
+    // rounds learned by an earlier call with the same signature
+    std::vector<double> sig = {(double)nf, (double)p->precision, (double)p->scheme,
+                               (double)p->nsteps, p->tol, p->T};
+    for (int s = 0; s < nsnap; ++s) {
+        sig.push_back(meshes[s]->nx);
+        sig.push_back(meshes[s]->ny);
+        sig.push_back(meshes[s]->nz);
+        sig.push_back(meshes[s]->dx);
+        sig.push_back(bandwidths ? bandwidths[s] : p->bandwidth);
+    }
+    int R = sizeof(TS) == 2 ? 5 : 2;
+    int *learned = nullptr;
+    for (auto &e : m0->brounds)
+        if (e.first == sig) learned = &e.second;
+    if (learned) R = std::max(R, *learned);
     // the plan's needed memory first, then the expansions' vectors; where those are refused,
     // the plan without them
     BatchPlan<TS> P;
@@ -6951,7 +6975,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
     const size_t nm = (size_t)nsnap * nf;   // masses per snapshot-field, before and after
     CGK_TRY(m0->h_small.ensure(4096 + nh * sizeof(double2) + 64 + 2 * nm * 8));
     for (bool want = p->max_rounds <= 0 || p->max_rounds >= 2;; want = false) {
-        CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, want, P));
+        CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, want, R, P));
         bool refused = false;   // (before, and nothing has changed since)
         for (int s = 0; s < nsnap; ++s)
             refused = refused || (P.pred && meshes[s]->ws_opt.known_refused(P.opt_bytes[s]));
@@ -6984,22 +7008,19 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
             rep->mass_out[f] = b;
         }
     };
-    // rounds learned by an earlier call with the same signature
-    std::vector<double> sig = {(double)nf, (double)p->precision, (double)p->scheme,
-                               (double)p->nsteps, p->tol, p->T};
-    for (int s = 0; s < nsnap; ++s) {
-        sig.push_back(meshes[s]->nx);
-        sig.push_back(meshes[s]->ny);
-        sig.push_back(meshes[s]->nz);
-        sig.push_back(meshes[s]->dx);
-        sig.push_back(bandwidths ? bandwidths[s] : p->bandwidth);
-    }
-    int R = sizeof(TS) == 2 ? 5 : 2;
-    int *learned = nullptr;
-    for (auto &e : m0->brounds)
-        if (e.first == sig) learned = &e.second;
-    if (learned) R = std::max(R, *learned);
+    const int R0 = R;
     for (; R <= max_r; ++R) {
+        if (P.pred && R == 3 && R0 < 3) {   // a second inner solve per step: other counts, the same arena
+            BatchPlan<TS> Q;
+            CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, true, R, Q));
+            for (int s = 0; s < nsnap; ++s) {
+                Q.descs[s].D = P.descs[s].D;
+                Q.descs[s].T = P.descs[s].T;
+            }
+            P = std::move(Q);
+            A = batch_layout(P, nsnap, nf, p->nsteps);   // (no longer: fewer weights)
+            CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
+        }
         // the schedule is replayed from a CUDA graph captured once per shape
         BatchKey key;
         key.arena = A.ab;
