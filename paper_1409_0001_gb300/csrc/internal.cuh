@@ -129,6 +129,7 @@ struct GraphEntry {
     unsigned gen_diffuse = 0, gen_small = 0, gen_opt = 0;   // (gen_opt: with predicted only)
     bool profiled = false;
     bool predicted = false;         // first rounds from the shared expansion
+    int m_it = 0;                   // iterations of an own inner solve (max_iter caps them)
     cudaGraphExec_t exec = nullptr;
     const void *result = nullptr;   // workspace buffer holding the final iterate
     long long kernels = 0;
@@ -142,6 +143,7 @@ struct RoundsEntry {
     double T, tol;
     int rounds;
     bool predicted;   // with the shared expansion
+    int m_it;
 };
 
 // The increments of a run of implicit steps as Chebyshev expansions of the run's first

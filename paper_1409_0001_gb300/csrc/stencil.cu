@@ -6030,12 +6030,14 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
         RoundsEntry *remembered = nullptr;
         for (RoundsEntry &re : m->rounds)
             if (re.nf == nf && re.precision == p->precision && re.scheme == p->scheme &&
-                re.nsteps == p->nsteps && re.T == T && re.tol == p->tol && re.predicted == (pred != nullptr)) {
+                re.nsteps == p->nsteps && re.T == T && re.tol == p->tol && re.predicted == (pred != nullptr) &&
+                re.m_it == m_it) {
                 R = re.rounds;
                 remembered = &re;
             }
         if (!remembered) {
-            m->rounds.push_back(RoundsEntry{nf, p->precision, p->scheme, p->nsteps, T, p->tol, R, pred != nullptr});
+            m->rounds.push_back(
+                RoundsEntry{nf, p->precision, p->scheme, p->nsteps, T, p->tol, R, pred != nullptr, m_it});
             remembered = &m->rounds.back();
         }
         XT *last_result = nullptr;
@@ -6056,7 +6058,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 if (it->nf == nf && it->precision == p->precision && it->scheme == p->scheme &&
                     it->nsteps == p->nsteps && it->rounds == R && it->T == T && it->tol == p->tol &&
                     it->cells == cells && it->profiled == prof && it->code == shape_used &&
-                    it->predicted == (pred != nullptr) &&
+                    it->predicted == (pred != nullptr) && it->m_it == m_it &&
                     it->wait_budget == rbudget)
                     ge = &*it;
                 ++it;
@@ -6080,6 +6082,7 @@ static cg_status diffuse_mixed(cg_mesh *m, int nf, double *cells, const cg_param
                 e.gen_opt = m->ws_opt.b.gen;
                 e.profiled = prof;
                 e.predicted = pred != nullptr;
+                e.m_it = m_it;
                 e.code = shape_used;
                 e.wait_budget = rbudget;
                 prof_capture_begin(&e.records, &e.kernels);
