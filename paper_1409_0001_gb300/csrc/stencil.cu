@@ -6536,9 +6536,10 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         if (!P.pred) pl = nullptr;
         if (want_pred && sizeof(TS) == 4 && !P.pred && s > 0 && P.Kmax > 0)   // start over without it
             return batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, false, R, P);
-        // (counts are even here, so the estimate's last two iterations, below what the fields'
-        // rounding leaves, are given up: 14 instead of 16 at b = 3 dx, errors as before)
-        if (pl) mi = R > 2 ? pred_round_m(pl->maxm, R) : std::max(mi, pl->maxm - 2);
+        // (with two iterations fewer, 14 instead of 16 at b = 3 dx, 64 snapshots of five fields take
+        // 79.8 instead of 86.5 ms, but the error against 64 bits, 2.1e-14 with own rounds, is 2.5e-14
+        // instead of 1.1e-14)
+        if (pl) mi = R > 2 ? pred_round_m(pl->maxm, R) : std::max(mi, pl->maxm);
         if (mi & 1) ++mi;
         d.m = mi;
         P.mmax = std::max(P.mmax, mi);
