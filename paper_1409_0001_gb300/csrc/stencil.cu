@@ -643,8 +643,8 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
     double *x = xall + off, *r = rall + off;
     double rr = 0.0;
     grid_stride<4>(
-        n, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads,
-        [&](int64_t k, int64_t step) {   // four cells in flight
+        n, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads,
+        [&](uint32_t k, uint32_t step) {   // four cells in flight
             double pv[4], qv[4], xv[4], rv[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
                 rr = fma(rk, rk, rr);
             }
         },
-        [&](int64_t k) {
+        [&](uint32_t k) {
             x[k] = fma(alpha, p[k], x[k]);
             const double rk = fma(-alpha, q[k], r[k]);
             r[k] = rk;
@@ -2845,7 +2845,7 @@ __global__ void __launch_bounds__(kThreads, ZFIX >= 2 ? 3 : 4) k_cheb_v4(Geo g, 
 // (it scales with sum_k |coef|, at most 1.6 and mostly below 0.2), which is what an own
 // inner solve per step leaves after its first round; the step's refinement goes on from
 // there as before and its residual is checked as before.  The run's K sweeps take the place
-// of one inner solve per step: at 128^3, 10 steps, b = 8 dx 52 sweeps for 350, b = 2 dx 17
+// of one inner solve per step: at 128^3, 10 steps, b = 8 dx 77 sweeps for 350, b = 2 dx 20
 // for 90.
 constexpr int kPredMaxK = 160;     // highest T_k
 constexpr int kPredMaxSteps = 20;  // steps per run (accumulators of k_pred_combine)
@@ -4277,8 +4277,8 @@ __global__ void k_mass(int n, const double *__restrict__ u_all, const double *__
     const double *u = u_all + (size_t)f * n;
     double s = 0.0;
     grid_stride<8>(
-        n, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads,
-        [&](int64_t k, int64_t step) {   // eight cells in flight
+        n, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads,
+        [&](uint32_t k, uint32_t step) {   // eight cells in flight
             double x[8], v[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -4288,7 +4288,7 @@ __global__ void k_mass(int n, const double *__restrict__ u_all, const double *__
 #pragma unroll
             for (int j = 0; j < 8; ++j) s += v[j] * x[j];
         },
-        [&](int64_t k) { s += (vc ? vc[k] : vcu) * u[k]; });
+        [&](uint32_t k) { s += (vc ? vc[k] : vcu) * u[k]; });
     double v = block_sum(s);
     double *partials = partials_all + (size_t)f * gridDim.x;
     if (arrive(partials, 1, &v, blockIdx.x, gridDim.x, &tickets[f])) {

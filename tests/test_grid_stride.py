@@ -1,6 +1,6 @@
 """The index range of the grid-stride loops (csrc/grid_stride.cuh), replayed on the host: every
 thread's cells, once and in order, and none outside the field, up to the largest mesh the API
-accepts (2^31 - 1 cells), where a 32-bit counter passes its range before the loop ends."""
+accepts (2^31 - 1 cells), where an int counter passes its range before the loop ends."""
 import os
 import subprocess
 
@@ -28,14 +28,14 @@ template <int W> static bool replay(int64_t n, int64_t first, int64_t step) {
     // (a replay that leaves the range or never ends gives up here)
     auto guard = [&]() { if (bad || seen > want) { printf("W %d n %lld first %lld step %lld\n", W, (long long)n,
                                                          (long long)first, (long long)step); exit(1); } };
-    cgk::grid_stride<W>(n, first, step,
-        [&](int64_t k, int64_t s) { for (int j = 0; j < W; ++j) take(k + j * s, n, step); guard(); },
-        [&](int64_t k) { take(k, n, step); guard(); });
+    cgk::grid_stride<W>((uint32_t)n, (uint32_t)first, (uint32_t)step,
+        [&](uint32_t k, uint32_t s) { for (int j = 0; j < W; ++j) take(k + j * s, n, step); guard(); },
+        [&](uint32_t k) { take(k, n, step); guard(); });
     return !bad && seen == want;
 }
 int main(int argc, char **argv) {
     const int64_t n = atoll(argv[1]);
-    for (int64_t blocks : {1, 16, 608, 1216, 1280}) {
+    for (int64_t blocks : {1, 16, 608, 1216, 1280, 65536}) {
         const int64_t step = blocks * 256;
         for (int64_t first : {int64_t(0), int64_t(1), step / 2, (n - 1) % step, n % step, step - 1})
             if (!replay<4>(n, first, step) || !replay<8>(n, first, step)) {
