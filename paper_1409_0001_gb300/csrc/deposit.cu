@@ -165,17 +165,8 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
     return warp_off + inc - v;
 }
 
-// The counting path of the ordered sums takes cells of at most kSegMax particles.  It is
-// launched before the host has seen the location's counters (check: outside particles,
-// non-finite weights, the most particles in a cell) and does nothing where they forbid it.
-constexpr int kSegMax = 64;
-__device__ __forceinline__ bool not_counting(const unsigned long long *check) {
-    return check && (check[0] | check[1] || check[2] > (unsigned long long)kSegMax);
-}
-
 __global__ void k_scan_reduce(const uint32_t *__restrict__ in, int64_t n,
-                              uint32_t *__restrict__ block_sums, const unsigned long long *__restrict__ check) {
-    if (not_counting(check)) return;
+                              uint32_t *__restrict__ block_sums) {
     int64_t base = (int64_t)blockIdx.x * kScanChunk;
     uint32_t s = 0;
     for (int j = threadIdx.x; j < kScanChunk; j += kThreads) {
@@ -194,8 +185,7 @@ __global__ void k_scan_reduce(const uint32_t *__restrict__ in, int64_t n,
 }
 
 // single block: exclusive scan of nb block sums, in place
-__global__ void k_scan_top(uint32_t *__restrict__ sums, int64_t nb, const unsigned long long *__restrict__ check) {
-    if (not_counting(check)) return;
+__global__ void k_scan_top(uint32_t *__restrict__ sums, int64_t nb) {
     uint32_t carry = 0;
     for (int64_t base = 0; base < nb; base += kThreads) {
         int64_t i = base + threadIdx.x;
@@ -211,9 +201,7 @@ __global__ void k_scan_top(uint32_t *__restrict__ sums, int64_t nb, const unsign
 // the chunks before it (at most kScanInline, from L2): one launch of 5 to 7 us less
 constexpr int kScanInline = 2048;
 __global__ void k_scan_down(const uint32_t *in, uint32_t *out, int64_t n,
-                            const uint32_t *__restrict__ block_off, bool sums_raw,
-                            const unsigned long long *__restrict__ check) {
-    if (not_counting(check)) return;
+                            const uint32_t *__restrict__ block_off, bool sums_raw) {
     __shared__ uint32_t tile[kScanChunk + kScanChunk / 32];
     __shared__ uint32_t before[kThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanChunk;
@@ -375,14 +363,26 @@ __global__ void k_segment_heads(int64_t n, const uint32_t *__restrict__ keys,
 // Counting path of the ordered sums (cells holding at most kSegMax particles): each
 // particle goes to the slot of its cell's segment given by its arrival rank at the
 // cell's counter (so the order inside a segment is arbitrary), then one thread per cell
-// sorts its segment's particle ids and adds the weights in ascending particle index.
+// sorts its segment's particle ids and adds the weights in ascending particle index.  Scatter
+// and sums may be launched before the host has seen the location's counters (check: outside
+// particles, non-finite weights, the most particles in a cell); they do nothing where
+// those forbid the path.
+constexpr int kSegMax = 64;
+__device__ __forceinline__ bool not_counting(const unsigned long long *check) {
+    return check && (check[0] | check[1] || check[2] > (unsigned long long)kSegMax);
+}
+
 __global__ void k_scatter_cells(int64_t n, const int32_t *__restrict__ cell,
                                 const uint32_t *__restrict__ off, const uint32_t *__restrict__ ranks,
                                 uint32_t *__restrict__ idx, const unsigned long long *__restrict__ check) {
-    if (not_counting(check)) return;
+    const bool skip = not_counting(check);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        idx[off[cell[i]] + ranks[i]] = (uint32_t)i;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t c = cell[i];
+        const uint32_t r = ranks[i];
+        if (skip) return;   // (the loads above are in flight with the counters')
+        idx[off[c] + r] = (uint32_t)i;
+    }
 }
 
 // eps_c = (sum of the cell's weights in ascending particle index, FP64 from +0.0) / V_c;
@@ -482,15 +482,15 @@ size_t scan_tmp_words(int64_t n) {
 }
 
 cg_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp,
-                             cudaStream_t st, const unsigned long long *check) {
+                             cudaStream_t st) {
     if (n <= 0) return CG_OK;
     int64_t nb = (n + kScanChunk - 1) / kScanChunk;
     CGK_LAUNCH("scan_reduce", (double)n * 4, st,
-               k_scan_reduce<<<(unsigned)nb, kThreads, 0, st>>>(in, n, tmp, check));
+               k_scan_reduce<<<(unsigned)nb, kThreads, 0, st>>>(in, n, tmp));
     const bool raw = nb <= kScanInline;
-    if (!raw) CGK_LAUNCH("scan_top", (double)nb * 8, st, k_scan_top<<<1, kThreads, 0, st>>>(tmp, nb, check));
+    if (!raw) CGK_LAUNCH("scan_top", (double)nb * 8, st, k_scan_top<<<1, kThreads, 0, st>>>(tmp, nb));
     CGK_LAUNCH("scan_down", (double)n * 8, st,
-               k_scan_down<<<(unsigned)nb, kThreads, 0, st>>>(in, out, n, tmp, raw, check));
+               k_scan_down<<<(unsigned)nb, kThreads, 0, st>>>(in, out, n, tmp, raw));
     CGK_CUDA(cudaGetLastError());
     return CG_OK;
 }
@@ -629,7 +629,7 @@ static void deposit_sort(cg_mesh *m, int64_t n, cudaStream_t st, DepositPlan &dp
     const unsigned long long *check = checked ? dp.bad : nullptr;
     dp.off = (uint32_t *)sb;
     dp.idx = (uint32_t *)(sb + s_off);
-    dp.sorted = exclusive_scan_u32(dp.counts, dp.off, dp.ncells + 1, (uint32_t *)(sb + s_off + s_idx), st, check);
+    dp.sorted = exclusive_scan_u32(dp.counts, dp.off, dp.ncells + 1, (uint32_t *)(sb + s_off + s_idx), st);
     if (dp.sorted == CG_OK && n > 0) {
         CGK_LAUNCH("scatter_cells", (double)n * 16, st,
                    k_scatter_cells<<<grid_for(n), kThreads, 0, st>>>(n, dp.cell, dp.off, dp.ranks, dp.idx, check));

@@ -336,9 +336,9 @@ cg_status hex_build(cg_mesh *m, int nx, int ny, int nz, const double *xf, const 
 void tet_release(cg_mesh *m);
 
 // Exclusive scan of n uint32 values (in and out may alias).  tmp needs
-// scan_tmp_words(n) words.  check (may be nullptr): see not_counting in deposit.cu.
+// scan_tmp_words(n) words.
 size_t scan_tmp_words(int64_t n);
 cg_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp,
-                             cudaStream_t st, const unsigned long long *check = nullptr);
+                             cudaStream_t st);
 
 }  // namespace cgk
