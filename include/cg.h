@@ -405,7 +405,8 @@ cg_status cg_profile_get(int i, char *name, int name_len, long long *launches, d
  * Memory that a call can do without (the vectors of the expansion that serves the first
  * rounds of precision modes 3 and 4, one vector of the FP64 solver) never makes a call
  * fail: it is not taken where it would not fit, and what other meshes hold of it is freed
- * when a call needs the room.  The expansion takes about 4 (K + 1 + steps) bytes per cell and
+ * when a call needs the room (under a limit: what was taken since the limit was set; what was
+ * held before counts as held, unless the limit is below the total: then it is freed).  The expansion takes about 4 (K + 1 + steps) bytes per cell and
  * field (K, of at most 160, grows with bandwidth / dx: 20 to 77 at 2 to 8 dx in ten steps;
  * at most 20 steps count) beside 52 (FP32 inner storage) or 42 (BF16) of needed vectors; all
  * meshes together hold at most a quarter of the device's memory of it.  A caller that wants the

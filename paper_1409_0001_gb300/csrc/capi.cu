@@ -42,10 +42,11 @@ static std::atomic<long long> g_ws_limit{0};
 
 // One attempt at a buffer of n bytes (and an eighth more); refused by the limit, the buffer
 // stays as it is.
-static cg_status try_grow(DevBuf &d, size_t n) {
+static cg_status try_grow(DevBuf &d, size_t n, bool *by_limit) {
     size_t want = n + n / 8;
     const long long lim = g_ws_limit.load();
-    if (lim > 0 && g_ws_bytes.load() - (long long)d.bytes + (long long)want > lim)
+    *by_limit = lim > 0 && g_ws_bytes.load() - (long long)d.bytes + (long long)want > lim;
+    if (*by_limit && g_ws_bytes.load() - (long long)d.bytes + (long long)want > lim)
         return fail(CG_ENOMEM,
                     "device workspace of %zu bytes refused: the library would hold %lld bytes, "
                     "above the limit of %lld (cg_set_workspace_limit)",
@@ -74,17 +75,20 @@ static std::mutex g_opt_mu;
 static std::condition_variable g_opt_cv;
 static std::vector<OptBuf *> g_opt;
 static unsigned g_opt_epoch = 1;
+static unsigned g_opt_limit = 0;          // how often the workspace limit has been set
 static thread_local int t_opt_held = 0;   // this thread's buffers in use
 constexpr size_t kOptFreely = (size_t)64 << 20;   // no look at the device's memory up to here
 
 // Frees every optional buffer not in use; where there is none, waits for one in use (unless this
-// thread holds one itself).  False: nothing was or will be freed.
-bool opt_reclaim() {
+// thread holds one itself).  False: nothing was or will be freed.  limit_only: those that were
+// taken under the present limit -- what was held when the limit was set counts as held, so that
+// a limit of "what is held now and x more" leaves room for x.
+bool opt_reclaim(bool limit_only) {
     std::unique_lock<std::mutex> lock(g_opt_mu);
     for (;;) {
         bool freed = false, used = false;
         for (OptBuf *o : g_opt) {
-            if (!o->b.bytes) continue;
+            if (!o->b.bytes || (limit_only && o->limit != g_opt_limit)) continue;
             if (o->busy) {
                 used = true;
                 continue;
@@ -101,8 +105,9 @@ bool opt_reclaim() {
 cg_status DevBuf::ensure(size_t n) {
     if (n <= bytes) return CG_OK;
     for (;;) {
-        const cg_status s = try_grow(*this, n);
-        if (s != CG_ENOMEM || !opt_reclaim()) return s;
+        bool by_limit = false;
+        const cg_status s = try_grow(*this, n, &by_limit);
+        if (s != CG_ENOMEM || !opt_reclaim(by_limit)) return s;
     }
 }
 
@@ -122,10 +127,14 @@ bool OptBuf::acquire(size_t n) {
                opt_share(n + n / 8, b.bytes, held, free_bytes, total);
         cudaGetLastError();
     }
-    if (n > b.bytes && (!fits || try_grow(b, n) != CG_OK)) {
-        refused = n;
-        epoch = g_opt_epoch;
-        return false;
+    bool by_limit = false;
+    if (n > b.bytes) {
+        if (!fits || try_grow(b, n, &by_limit) != CG_OK) {
+            refused = n;
+            epoch = g_opt_epoch;
+            return false;
+        }
+        limit = g_opt_limit;
     }
     if (!listed) g_opt.push_back(this);
     listed = busy = true;
@@ -154,6 +163,16 @@ void OptBuf::release() {
 void opt_epoch_bump() {
     std::lock_guard<std::mutex> lock(g_opt_mu);
     ++g_opt_epoch;
+}
+
+// A limit below what is held takes back optional memory that no call uses.
+static void opt_limit_set(long long bytes) {
+    std::lock_guard<std::mutex> lock(g_opt_mu);
+    g_ws_limit.store(bytes);
+    ++g_opt_epoch;
+    ++g_opt_limit;
+    for (OptBuf *o : g_opt)
+        if (bytes > 0 && g_ws_bytes.load() > bytes && !o->busy) o->b.release();
 }
 
 void DevBuf::release() {
@@ -406,8 +425,7 @@ long long cg_launch_count(void) { return g_launches.load(); }
 
 cg_status cg_set_workspace_limit(long long bytes) {
     if (bytes < 0) return fail(CG_EINVAL, "the workspace limit must be >= 0 (0: no limit)");
-    g_ws_limit.store(bytes);
-    opt_epoch_bump();
+    opt_limit_set(bytes);
     return CG_OK;
 }
 

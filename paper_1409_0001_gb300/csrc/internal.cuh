@@ -41,9 +41,9 @@ struct DevBuf {
 };
 
 // A device buffer that a call can do without (it then runs a slower form).  It never costs any
-// call its DevBufs: a DevBuf that is refused (the workspace limit, or the device is full) takes
-// back every OptBuf that no running call uses, of all meshes, waits for those in use, and
-// asks again.  The caller's own allocations cannot do that, so what the OptBufs hold together stays
+// call its DevBufs: a DevBuf that is refused takes back the OptBufs that no running call uses, of
+// all meshes, waits for those in use, and asks again -- all of them where the device is full,
+// those taken under the present setting of the workspace limit where that refused.  The caller's own allocations cannot do that, so what the OptBufs hold together stays
 // within a share of the device (opt_share).  So a call acquires its OptBuf after its last DevBuf, holds it through an OptUse,
 // and asks for no DevBuf while it does.  A refusal is remembered until a mesh is
 // destroyed or the workspace limit is set: a call that cannot have the memory does not ask,
@@ -52,7 +52,7 @@ struct OptBuf {
     DevBuf b;
     bool busy = false, listed = false;   // guarded, as what follows, by one mutex for all
     size_t refused = 0;                  // the smallest request refused at `epoch`
-    unsigned epoch = 0;
+    unsigned epoch = 0, limit = 0;       // limit: which setting of the limit it was taken under
     bool known_refused(size_t n);
     bool acquire(size_t n);              // true: n bytes are this call's until done()
     void done();
@@ -74,7 +74,9 @@ inline bool opt_share(size_t want, size_t own, size_t held, size_t free_bytes, s
     return held - own + want <= total / 4 && want <= (free_bytes + own) / 4;
 }
 void opt_epoch_bump();   // memory may have become available: refusals are forgotten
-bool opt_reclaim();      // frees optional buffers; false: none was left to free
+// Frees optional buffers (limit_only: those taken under the present workspace limit); false:
+// none was left to free.
+bool opt_reclaim(bool limit_only);
 
 // A pinned host buffer that only grows (readback of scalars, flags, counters).
 struct HostBuf {

@@ -33,7 +33,7 @@ template <class T> cg_status upload(T **dst, const T *src, size_t n) {
     *dst = nullptr;
     if (n == 0) return CG_OK;
     cudaError_t e = cudaMalloc((void **)dst, n * sizeof(T));
-    while (e == cudaErrorMemoryAllocation && opt_reclaim()) {   // (other meshes' optional vectors)
+    while (e == cudaErrorMemoryAllocation && opt_reclaim(false)) {   // (other meshes' optional vectors)
         cudaGetLastError();
         e = cudaMalloc((void **)dst, n * sizeof(T));
     }

@@ -131,8 +131,12 @@ def test_fp64_beyond_the_cooperative_size(cg):
     held = cg.workspace_bytes()
     smooth(cg, a, field(5))
     taken = cg.workspace_bytes() - held
-    mesh = cg.StructuredMesh(dims, (0, 0, 0), 1.0)
-    cg.set_workspace_limit(held + taken)               # three vectors fit once the expansion's are back
+    a.close()
+    cg.set_workspace_limit(held + taken)
+    a = cg.StructuredMesh(DIMS, (0, 0, 0), 1.0)
+    smooth(cg, a, field(5))
+    assert cg.workspace_bytes() == held + taken
+    mesh = cg.StructuredMesh(dims, (0, 0, 0), 1.0)     # three vectors fit once the expansion's are back
     x = u.clone()
     cg.diffuse(mesh, x, cg.Params(T=2.0, nsteps=NSTEPS))
     cg.set_workspace_limit(0)
@@ -141,6 +145,23 @@ def test_fp64_beyond_the_cooperative_size(cg):
     assert near(x, y, u)
     mesh.close()
     a.close()
+
+
+def test_a_limit_of_what_is_held_and_some_more(cg):
+    """Optional memory held when the limit is set counts as held: room for x is room for x."""
+    import torch
+    a = cg.StructuredMesh(DIMS, (0, 0, 0), 1.0)
+    smooth(cg, a, field(7))
+    held = cg.workspace_bytes()
+    b = cg.StructuredMesh((32, 32, 32), (0, 0, 0), 1.0)
+    u = torch.zeros((1, 32 ** 3), dtype=torch.float64, device="cuda")
+    cg.set_workspace_limit(held + 64 * 1024)
+    with pytest.raises(cg.CGError) as e:
+        cg.diffuse(b, u, cg.Params(T=2.0, nsteps=NSTEPS, precision=3))
+    assert e.value.code == "CG_ENOMEM"
+    assert held <= cg.workspace_bytes() <= held + 64 * 1024
+    a.close()
+    b.close()
 
 
 def test_a_batch_under_its_needed_size(cg):
