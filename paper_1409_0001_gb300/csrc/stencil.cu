@@ -6491,7 +6491,8 @@ struct BatchPlan {
     std::vector<BItem> pitems;     // the shared expansion's sweeps (one field)
     std::vector<float> pcoef;
     std::vector<size_t> pc_off;
-    std::vector<size_t> opt_bytes; // the expansion's vectors, per snapshot
+    std::vector<size_t> opt_off;   // the expansions' vectors in one optional buffer
+    size_t opt_bytes = 0;
     bool pred = false;
     int Kmax = 0;
     std::vector<int> first_item;   // per (snapshot, field), into ritems
@@ -6509,7 +6510,7 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
     P.descs.resize((size_t)nsnap);
     P.omega_off.resize((size_t)nsnap);
     P.pc_off.resize((size_t)nsnap);
-    P.opt_bytes.resize((size_t)nsnap);
+    P.opt_off.resize((size_t)nsnap);
     // the shared expansion serves the batch where it pays for every snapshot: FP32 inner
     // storage, one run of steps, rows the flat-plane engine takes
     P.pred = sizeof(TS) == 4 && want_pred && p->nsteps <= kPredMaxSteps;
@@ -6574,7 +6575,8 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
         const size_t vts = align_up((size_t)m->nz * d.pts * nf * sizeof(TS));
         const size_t t1 = align_up((size_t)m->nz * d.pts * 4);
         if (pl) {
-            P.opt_bytes[s] = p->nsteps * vts + (pl->maxK + 1) * t1;
+            P.opt_off[s] = P.opt_bytes;
+            P.opt_bytes += p->nsteps * vts + (pl->maxK + 1) * t1;
             d.K = pl->K[0];
             d.w = (float)(2.0 * ce / (lmax - 1.0));
             P.Kmax = std::max(P.Kmax, d.K);
@@ -6614,31 +6616,6 @@ static cg_status batch_plan(int nsnap, cg_mesh *const *meshes, int nf, double *c
     }
     P.first_item.push_back((int)P.ritems.size());
     return CG_OK;
-}
-
-// The expansions' vectors of every snapshot, each in its mesh's optional buffer; false, and
-// nothing more held than before, where one is refused.
-template <class TS>
-static bool batch_take(BatchPlan<TS> &P, int nsnap, cg_mesh *const *meshes, int nf, int nsteps,
-                       std::vector<OptUse> &opt) {
-    std::vector<char> grown((size_t)nsnap, 0);
-    for (int s = 0; s < nsnap; ++s) {
-        OptBuf &o = meshes[s]->ws_opt;
-        const unsigned gen = o.b.gen;
-        if (!opt[s].take(o, P.opt_bytes[s])) {
-            for (int q = 0; q < s; ++q) {
-                opt[q].o->done();
-                if (grown[q]) opt[q].o->release();
-                opt[q].o = nullptr;
-            }
-            return false;
-        }
-        grown[s] = o.b.gen != gen;
-        SnapDesc<TS> &d = P.descs[s];
-        d.D = o.as<float>();
-        d.T = d.D + (size_t)d.g.nz * d.pts * nf * nsteps;
-    }
-    return true;
 }
 
 // The batch arena on the first mesh: descriptors | items | partials | hist | barrier | failure
@@ -6970,25 +6947,31 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
     for (auto &e : m0->brounds)
         if (e.first == sig) learned = &e.second;
     if (learned) R = std::max(R, *learned);
-    // the plan's needed memory first, then the expansions' vectors; where those are refused,
-    // the plan without them
+    // the plan's needed memory first, then the expansions' vectors, in one buffer of the first mesh
+    // (an allocation per snapshot would cost a first call of 64 snapshots 25 ms); where those are
+    // refused, the plan without them
+    auto place = [&](BatchPlan<TS> &Q) {
+        for (int s = 0; s < nsnap && Q.pred; ++s) {
+            SnapDesc<TS> &d = Q.descs[s];
+            d.D = (float *)(m0->ws_opt.as<char>() + Q.opt_off[s]);
+            d.T = d.D + (size_t)d.g.nz * d.pts * nf * p->nsteps;
+        }
+    };
     BatchPlan<TS> P;
     BatchArena A;
-    std::vector<OptUse> opt((size_t)nsnap);
+    OptUse opt;
     const size_t nh = (size_t)p->nsteps * nsnap * nf;
     const size_t nm = (size_t)nsnap * nf;   // masses per snapshot-field, before and after
     CGK_TRY(m0->h_small.ensure(4096 + nh * sizeof(double2) + 64 + 2 * nm * 8));
     for (bool want = p->max_rounds <= 0 || p->max_rounds >= 2;; want = false) {
         CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, want, R, P));
-        bool refused = false;   // (before, and nothing has changed since)
-        for (int s = 0; s < nsnap; ++s)
-            refused = refused || (P.pred && meshes[s]->ws_opt.known_refused(P.opt_bytes[s]));
-        if (refused) continue;
+        if (P.pred && m0->ws_opt.known_refused(P.opt_bytes)) continue;
         A = batch_layout(P, nsnap, nf, p->nsteps);
         const cg_status s = m0->ws_batch.ensure(A.total);
         if (!P.pred) CGK_TRY(s);
-        if (!P.pred || (s == CG_OK && batch_take(P, nsnap, meshes, nf, p->nsteps, opt))) break;
+        if (!P.pred || (s == CG_OK && opt.take(m0->ws_opt, P.opt_bytes))) break;
     }
+    place(P);
     CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
     double2 *hh = (double2 *)(m0->h_small.as<char>() + 4096);
     GridBar *hgb = (GridBar *)(hh + nh);
@@ -7017,10 +7000,7 @@ static cg_status diffuse_batched_df(int nsnap, cg_mesh *const *meshes, int nf,
         if (P.pred && R == 3 && R0 < 3) {   // a second inner solve per step: other counts, the same arena
             BatchPlan<TS> Q;
             CGK_TRY(batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, zlen, true, R, Q));
-            for (int s = 0; s < nsnap; ++s) {
-                Q.descs[s].D = P.descs[s].D;
-                Q.descs[s].T = P.descs[s].T;
-            }
+            place(Q);
             P = std::move(Q);
             A = batch_layout(P, nsnap, nf, p->nsteps);   // (no longer: fewer weights)
             CGK_TRY(batch_upload(P, A, m0->ws_batch.as<char>(), nsnap, cells, st));
