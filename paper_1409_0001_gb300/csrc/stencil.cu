@@ -6741,7 +6741,7 @@ static cg_status batch_issue_phased(const BatchPlan<TS> &P, const BatchArena &A,
     const char *rname = sizeof(TS) == 2 ? "brefine_bf16" : "brefine_fp32";
     std::vector<double> cheb_bytes((size_t)P.mmax, 0.0);
     for (const auto &d : P.descs)
-        for (int k = 1; k < d.m; ++k) cheb_bytes[(size_t)k] += (double)d.g.n * nf * 4.0 * sizeof(TS);
+        for (int k = 1; k < std::min(d.m, P.mmax); ++k) cheb_bytes[(size_t)k] += (double)d.g.n * nf * 4.0 * sizeof(TS);
     const double ref_bytes = cells_f * (24.0 + 3.0 * sizeof(TS));
     const bool cn = P.descs[0].scheme == CG_SCHEME_CRANK_NICOLSON, mid = batch_mid(pred, R);
     if (!pred)
@@ -6871,6 +6871,9 @@ static cg_status batch_tune(int nsnap, cg_mesh *const *meshes, int nf, double *c
         BatchPlan<TS> P;
         rc = batch_plan<TS>(nsnap, meshes, nf, cells, p, bandwidths, z, true, 2, P);
         if (rc != CG_OK) break;
+        // with the expansion a step has one inner solve: half the iterations in each of the two
+        // rounds, so that sweeps and passes are weighed about as the call runs them
+        if (P.pred) P.mmax = (P.mmax + 1) / 2;
         BatchArena A = batch_layout(P, nsnap, nf, 1);
         rc = m0->ws_batch.ensure(A.total);
         if (rc != CG_OK) break;
