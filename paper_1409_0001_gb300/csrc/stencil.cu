@@ -4125,8 +4125,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_brefine(const SnapDesc<TS> *__r
 }
 
 // A merged pass of every snapshot (see batched_mid).  64 snapshots x 5 fields: 1.49 ms at 128
-// registers (2.6 TB/s, latency) in the place of two k_brefine passes of 1.00 ms each; the call 85
-// -> 80 ms.
+// registers (2.6 TB/s, latency) in the place of two k_brefine passes of 1.00 ms each; the call 5
+// ms less.
 template <class TS>
 __global__ void __launch_bounds__(kThreads, 2) k_bmid(const SnapDesc<TS> *__restrict__ sd, int nf,
                                                     const BItem *__restrict__ ritems, int step, int end,
@@ -4142,8 +4142,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_bmid(const SnapDesc<TS> *__rest
 // vectors T_k take the room of one field): T_0, the recurrence's step k, the combination.
 // 64 snapshots of 32 to 96 cells a side, 5 fields, b = 3 dx, 10 steps: 29 recurrence steps of
 // 80 us per field (3.3 TB/s: the flat tile's barriers and neighbour tests) and 0.9 ms per
-// combination (4.0 TB/s) take the place of 130 k_bcheb launches of 335 us; the call 112 ->
-// 84 ms.
+// combination (4.0 TB/s) take the place of 130 k_bcheb launches of 335 us; the call, with the
+// merged pass, 112 -> 86.5 ms.
 template <class TS>
 __global__ void __launch_bounds__(kThreads) k_bpred_start(const SnapDesc<TS> *__restrict__ sd, int f) {
     chain_wait();
