@@ -369,7 +369,9 @@ __global__ void k_segment_heads(int64_t n, const uint32_t *__restrict__ keys,
 // those forbid the path.
 constexpr int kSegMax = 64;
 __device__ __forceinline__ bool not_counting(const unsigned long long *check) {
-    return check && (check[0] | check[1] || check[2] > (unsigned long long)kSegMax);
+    if (!check) return false;
+    const unsigned long long out = check[0], bad = check[1], most = check[2];   // one wait for all three
+    return ((out | bad) != 0) | (most > (unsigned long long)kSegMax);
 }
 
 __global__ void k_scatter_cells(int64_t n, const int32_t *__restrict__ cell,
