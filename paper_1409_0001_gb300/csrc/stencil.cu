@@ -697,19 +697,22 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int n, int nb, const dou
 // so the sums are the same bits in every block and every run.  (Partials tagged with the
 // sum's number and polled by every block, which needs no arrival counter, took 2 us more
 // at 32^3: 152 blocks polling 152 slots.)
-// Fields are independent, so several run at a time: the launch's blocks form groups of
-// `blocks`, as many as the SMs hold (a block of 128 threads takes a quarter of an SM's
-// registers), each with its own barrier and partial sums; group q solves fields q, q + groups,
+// Fields are independent, so several run at a time on meshes whose blocks have 128 threads: the
+// launch's blocks form groups of `blocks`, up to four blocks to an SM, each with its own barrier and partial sums; group q solves fields q, q + groups,
 // .. and the groups meet once per step.  A field's block layout, and with it its bits, do not
 // depend on how many there are.  (One field after the other, 8^3 x 8 fields took 12.7 ms a
 // call and 32^3 x 5 fields 10.9, against 5.7 and 7.4 in the two-launch form, which runs all
-// fields in one launch; in groups 1.8 and 5.2.)
+// fields in one launch; in groups 1.8 and 4.9.)
 struct __align__(128) CoopBar {   // a group's; the last one is the whole launch's
     unsigned int count;
     int err;
     int failed[2];   // a field of an even / odd step did not converge (the last one's)
 };
 constexpr int kCoopMaxC = 12;    // cells per thread: 6 C registers of state within 128
+// Blocks that an SM's registers hold: 72 and 80 registers a thread for one and two cells, else
+// 128.  Small solves of several streams share the SMs the better the more of them fit (six
+// calls of 32^3 at a time 5.4 ms, 7.6 with four blocks of 104 registers).
+constexpr int coop_blocks_per_sm(int NT, int C) { return NT == 128 && C <= 2 ? 8 - C : 512 / NT; }
 
 // One group's place in the launch.
 struct CoopGroup {
@@ -814,7 +817,7 @@ __device__ __forceinline__ bool coop_sum(double a, double b, double2 *part, cons
 // field's iteration stops as in the two-launch form: converged, breakdown, or max_it.  After
 // a step in which a field did not converge nothing more runs.
 template <int NT, int C>
-__global__ void __launch_bounds__(NT, 512 / NT) k_cg_coop(
+__global__ void __launch_bounds__(NT, coop_blocks_per_sm(NT, C)) k_cg_coop(
     Geo g, int blocks, int per_block, double c, Coef64 cf, int scheme, int nf, int nsteps, int max_it, double tol2,
     const double *__restrict__ cells, double *X, double *V, size_t vstride, double2 *part,
     Scal *__restrict__ hist, CoopBar *bars, long long budget) {
@@ -5282,19 +5285,23 @@ static cg_status fp64_coop(cg_mesh *m, const Geo &g, int nf, double *cells, cons
     // cooperative form is still twice as fast as the two-launch form (30.7 against 58.7 us at 96^3).  Small meshes take
     // blocks of fewer threads, so that the solves of several streams share the SMs: blocks of
     // 512 threads at any size ran six concurrent 32^3 calls one after another, 15.2 ms
-    // against 8.6 with the two-launch form (now 6.0; 64^3 20.3 -> 16.2 ms).
+    // against 8.6 with the two-launch form (now 5.4; 64^3 20.3 -> 16.2 ms).
     const int grid = std::max(1, std::min(num_sms(), (n + 63) / 64));
     const int per_block = (n + grid - 1) / grid;
     const int nt = per_block <= 128 * 4 ? 128 : per_block <= 256 * 8 ? 256 : 512;
     const int need = (per_block + nt - 1) / nt;
     if (need > kCoopMaxC) return CG_OK;
-    // Groups of fields: 512 / nt blocks to an SM (the kernel's launch bounds).  Many fields of a
-    // small mesh take so many turns of about 8.5 us an iteration that the two-launch form, one
-    // pair of launches for all of them, is the faster one: it costs about 24 us and, per million
-    // cells, 19 us more than the turns' arithmetic.  Measured per iteration, this form against
-    // that one: 16^3 x 16 fields 17.5 and 23.9 us, x 32 34.0 and 27.5; 32^3 x 8 23.4 and 29.6, x 16
-    // 46.4 and 42.8; 48^3 x 8 58.0 and 66.3, x 16 115 and 115; 64^3 x 16 170 and 209.
-    const int groups = std::min(nf, 512 / nt * num_sms() / grid), turns = (nf + groups - 1) / groups;
+    // Groups of fields side by side: up to four blocks of 128 threads on an SM, evened out over the
+    // turns.  Blocks of 256 threads run one field at a time: an SM holds two of them, and a second
+    // problem's fill that place as well as a second field would (four problems of 48^3 x 3 fields
+    // at a time 19.2 ms, 26.9 with two groups each).
+    const int cap = nt == 128 ? std::min(nf, 4 * num_sms() / grid) : 1, turns = (nf + cap - 1) / cap;
+    const int groups = (nf + turns - 1) / turns;
+    // Many fields of a small mesh take so many turns of about 8.5 us an iteration that the two-launch
+    // form, one pair of launches for all of them, is the faster one: it costs about 24 us and, per
+    // million cells, 19 us more than the turns' arithmetic.  Measured per iteration, this form
+    // against that one: 16^3 x 16 fields 17.5 and 23.9 us, x 32 34.0 and 27.5; 32^3 x 8 23.4 and 29.6,
+    // x 16 46.4 and 42.8; 48^3 x 3 35.8 and 35.8, x 4 47.8 and 42.5; 64^3 x 5 79.6 and 79.9, x 8 127 and 112.
     if (8.5 * turns > 24.0 + 1.9e-5 * nf * n) return CG_OK;
     const size_t vec = align_up((size_t)n * nf * 8), one = align_up((size_t)n * 8);
     const size_t hist_n = (size_t)p->nsteps * nf;

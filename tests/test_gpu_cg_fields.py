@@ -1,8 +1,8 @@
 """GPU: several fields in one FP64 conjugate gradient call.  In the cooperative form fields run in
-groups of blocks side by side, and a field's block layout does not depend on how many there are:
-each field has the bits of its own call -- fewer fields than groups, as many, one more, several
-turns -- also where a call stops short (all fields after the same step).  Where the many fields
-take the two-launch form the results agree to the stopping tolerance: 1e-13 of ||b|| per step
+groups of blocks side by side (one after another on larger meshes), and a field's block layout
+does not depend on how many there are: each field has the bits of its own call -- fewer fields
+than groups, as many, one more, several turns -- also where a call stops short (all fields after
+the same step).  Where the many fields take the two-launch form the results agree to the stopping tolerance: 1e-13 of ||b|| per step
 and form, four steps, times 100 for the largest cell against the root mean square.
 """
 import numpy as np
@@ -10,7 +10,8 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-DIMS = [(3, 2, 1), (8, 8, 8), (16, 15, 17), (33, 30, 32), (49, 48, 47), (64, 64, 63), (77, 90, 80)]
+CASES = [(d, nf) for d in [(3, 2, 1), (8, 8, 8), (16, 15, 17), (33, 30, 32), (42, 40, 41)] for nf in (2, 3, 5, 9)]
+CASES += [((49, 48, 47), 2), ((49, 48, 47), 3), ((64, 64, 63), 5), ((77, 90, 80), 2), ((77, 90, 80), 9)]
 
 
 def solve(cg, u, dims, **kw):
@@ -26,8 +27,7 @@ def solve(cg, u, dims, **kw):
     return x.cpu().numpy(), code
 
 
-@pytest.mark.parametrize("dims", DIMS)
-@pytest.mark.parametrize("nf", [2, 3, 5, 9])
+@pytest.mark.parametrize("dims,nf", CASES)
 def test_each_field_as_alone(dims, nf):
     import paper_1409_0001_gb300 as cg
     n = dims[0] * dims[1] * dims[2]
@@ -57,7 +57,7 @@ def test_no_convergence_stops_every_field_after_the_step(dims, nf):
     assert np.array_equal(got[0], u[0])
 
 
-@pytest.mark.parametrize("dims,nf", [((16, 16, 16), 64), ((32, 32, 32), 40)])
+@pytest.mark.parametrize("dims,nf", [((16, 16, 16), 64), ((32, 32, 32), 40), ((49, 48, 47), 9), ((64, 64, 63), 9)])
 def test_many_fields(dims, nf):
     import paper_1409_0001_gb300 as cg
     n = dims[0] * dims[1] * dims[2]
