@@ -102,10 +102,11 @@ bool opt_reclaim(bool limit_only) {
     }
 }
 
-cg_status DevBuf::ensure(size_t n) {
+cg_status DevBuf::ensure(size_t n, size_t room) {
     if (n <= bytes) return CG_OK;
+    bool by_limit = false;
+    if (room > n && try_grow(*this, room, &by_limit) == CG_OK) return CG_OK;
     for (;;) {
-        bool by_limit = false;
         const cg_status s = try_grow(*this, n, &by_limit);
         if (s != CG_ENOMEM || !opt_reclaim(by_limit)) return s;
     }

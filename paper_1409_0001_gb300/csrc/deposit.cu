@@ -509,7 +509,7 @@ cg_status tet_locate_launch(cg_mesh *m, int64_t n, const double *pos, int nf, co
 static cg_status locate_launch(cg_mesh *m, int64_t n, const double *pos, int nf, const double *w,
                                int32_t *cell_out, uint32_t *counts, uint32_t *ranks, cudaStream_t st,
                                unsigned long long *bad_zeroed = nullptr) {
-    CGK_TRY(m->ws_small.ensure(4096));
+    CGK_TRY(m->ws_small.ensure(4096, kSmallRoom));
     CGK_TRY(m->h_small.ensure(4096));
     unsigned long long *bad = bad_zeroed ? bad_zeroed : m->ws_small.as<unsigned long long>();
     if (!bad_zeroed) CGK_CUDA(cudaMemsetAsync(bad, 0, 3 * sizeof(unsigned long long), st));

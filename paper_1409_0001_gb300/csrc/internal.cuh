@@ -35,10 +35,13 @@ struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
     unsigned gen = 0;        // bumped on every reallocation (invalidates captured graphs)
-    cg_status ensure(size_t n);
+    // room > n: that much where it may be had, for a buffer that a call asks for in several sizes
+    // (growing it costs a free and an allocation, 65 us)
+    cg_status ensure(size_t n, size_t room = 0);
     void release();
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
+constexpr size_t kSmallRoom = 256 << 10;   // ws_small: the counters, masses and partials of most calls
 
 // A device buffer that a call can do without (it then runs a slower form).  It never costs any
 // call its DevBufs: a DevBuf that is refused takes back the OptBufs that no running call uses, of

@@ -5215,7 +5215,7 @@ static cg_status field_mass_launch(cg_mesh *m, int nf, const double *cells, cuda
     // a block per 2048 cells, at most four to an SM over all fields
     const int G = std::max(1, std::min((n + 2047) / 2048, std::max(1, 4 * num_sms() / nf)));
     size_t need = align_up((size_t)nf * G * 8) + 64 * 8 + 64 * 4;
-    CGK_TRY(m->ws_small.ensure(4096 + need));
+    CGK_TRY(m->ws_small.ensure(4096 + need, kSmallRoom));
     char *base = m->ws_small.as<char>() + 4096;
     double *partials = (double *)base;
     double *out = (double *)(base + align_up((size_t)nf * G * 8));
